@@ -16,6 +16,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "internal.h"
 
 namespace {
@@ -58,178 +60,331 @@ __global__ void k_rowconst(const af_rowstats_t* __restrict__ st, int ndm, int64_
 }
 
 constexpr int kBT = 256;             // threads per block
-constexpr int kPer = 16;             // outputs per thread
-constexpr int kBOut = kBT * kPer;    // outputs per block
+constexpr int kBW = kBT / 32;        // warps
+constexpr int kFloatBits = 22;       // the float path needs |prefix| and |q - w mu0| below 2^22
 
-// Block = one tile of kBOut outputs of one row.
-//  1. Y[t0 .. t0 + L), L = kBOut + wmax - 1 (clipped at nout), is loaded into
-//     shared memory with coalesced (16-byte when aligned) loads, all issued
-//     before any is used.
-//  2. Prefix sums P[j] = sum_{k<j} Y[t0+k] (mod 2^32) in one pass: thread i
-//     scans its own segment of C consecutive values (C odd, so a warp's
-//     segment accesses fall in distinct banks), the segment totals are scanned
-//     across the block, and each thread adds its offset.
-//  3. Output t0 + lt (lt = tid + kBT*i) evaluates every width from P[lt] and
-//     P[lt + w]: B = P[lt+w] - P[lt], snr = (B - q) * k - c.
-// With SMALL (every window sum < 2^31) the difference B - q is formed and
-// converted in 32 bits.
-template <bool SMALL>
-__global__ void __launch_bounds__(kBT, 4)
-k_boxcar(const int32_t* __restrict__ Y, int64_t nout, unsigned tiles, af_widths_t w,
-         const af_rowconst_t* __restrict__ rc, float* __restrict__ snr, uint8_t* __restrict__ bw)
+// Two fp32 operations in one instruction (each rounded like the scalar one).
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
 {
-    extern __shared__ uint32_t sP[];  // 3 words of padding, then P[0 .. kBT*C]
-    __shared__ int64_t sq[AF_MAX_WIDTHS];
-    __shared__ float sk[AF_MAX_WIDTHS], sc[AF_MAX_WIDTHS];
-    __shared__ int sw[AF_MAX_WIDTHS];
-    __shared__ uint32_t swarp[kBT / 32];
-    uint32_t* P = sP + 3;             // P[1 + j] holds Y[t0 + j]: 16-byte aligned for j % 4 == 0
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 
-    const int d = (int)(blockIdx.x / tiles);
-    const int64_t t0 = (int64_t)(blockIdx.x % tiles) * kBOut;
-    const int nw = w.n;
-    const int wmax = w.w[nw - 1];
-    const int L = (int)(min(nout, t0 + kBOut + wmax - 1) - t0);
-    const int64_t base = (int64_t)d * nout + t0;
-    const int32_t* y = Y + base;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// One width of a tile's outputs, e = q - w mu0 (an integer, or -e as a float
+// where the float path runs) and the constants twice, as the paired
+// instructions take them.
+struct __align__(16) BoxWidth {
+    int32_t e, e2;
+    float k, k2;
+    float nc, nc2;   // -c
+    int w, pad;
+};
 
-    if (tid < nw) {
-        const af_rowconst_t c = rc[(int64_t)d * AF_MAX_WIDTHS + tid];
-        sq[tid] = c.q;
-        sk[tid] = c.k;
-        sc[tid] = c.c;
-        sw[tid] = w.w[tid];
-    }
-    // 1. load Y into P[1 .. L]
-    int done = 0;
-    if ((reinterpret_cast<uintptr_t>(y) & 15) == 0) {
-        // every load of the tile is issued before the first shared store
-        constexpr int NB = (kBOut + 1024) / 4 / kBT;  // 16-byte loads per thread (L <= kBOut + 1023)
-        const int L4 = L >> 2;
-        const int4* y4 = reinterpret_cast<const int4*>(y);
-        int4 v[NB];
-#pragma unroll
-        for (int u = 0; u < NB; u++)
-            if (tid + u * kBT < L4) v[u] = __ldg(y4 + tid + u * kBT);
-#pragma unroll
-        for (int u = 0; u < NB; u++)
-            if (tid + u * kBT < L4) reinterpret_cast<int4*>(P + 1)[tid + u * kBT] = v[u];
-        for (int j = tid + NB * kBT; j < L4; j += kBT) reinterpret_cast<int4*>(P + 1)[j] = __ldg(y4 + j);
-        done = 4 * L4;
-    }
-    for (int j = done + tid; j < L; j += kBT) P[j + 1] = (uint32_t)__ldg(y + j);
-    const int C = ((L + kBT - 1) / kBT) | 1;
-    for (int j = L + 1 + tid; j <= kBT * C; j += kBT) P[j] = 0u;  // pad the last segments
-    if (tid == 0) P[0] = 0u;
-    __syncthreads();
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
 
-    // 2. prefix sums: the segment of thread tid is P[1 + tid*C .. 1 + (tid+1)*C)
-    uint32_t* seg = P + 1 + tid * C;
-    uint32_t run = 0;
-    for (int k = 0; k < C; k++) {
-        run += seg[k];
-        seg[k] = run;
-    }
-    uint32_t incl = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) swarp[warp] = incl;
-    __syncthreads();
-    uint32_t off = incl - run;
-    for (int k = 0; k < warp; k++) off += swarp[k];
-    for (int k = 0; k < C; k++) seg[k] += off;
-    __syncthreads();
+enum { kPathFloat, kPathInt, kPathWide };
 
-    // 3. S/N of every width, best width.  Tiles whose every window ends
-    //    inside the row take the unchecked path: widths outer, the thread's
-    //    kPer outputs inner (independent chains).
-    if (t0 + kBOut + wmax - 1 <= nout) {
-        uint32_t p0[kPer];
-        float best[kPer];
-        int bi[kPer];
+// Pairs of prefix words P[i + w] .. P[i + w + 3] for i % 4 == 0, given the
+// four words at i (x) and at i + 4 (y), r = w % 4.
+__device__ __forceinline__ void shift_words(const ulonglong2& x, const ulonglong2& y, int r, uint64_t (&p)[2])
+{
+    if (r == 1) {
+        p[0] = x.x >> 32 | x.y << 32;
+        p[1] = x.y >> 32 | y.x << 32;
+    } else if (r == 2) {
+        p[0] = x.y;
+        p[1] = y.x;
+    } else {
+        p[0] = x.y >> 32 | y.x << 32;
+        p[1] = y.x >> 32 | y.y << 32;
+    }
+}
+
+// Every width's S/N of the four outputs lt .. lt + 3 (lt % 4 == 0): the best
+// and its index.  PATH kPathFloat: the words are floats holding exact integers
+// below 2^22, so both differences are exact in fp32 and equal the converted
+// integer difference bit for bit; kPathInt: 32-bit integers; kPathWide: 32-bit
+// prefix, 64-bit difference.  TAIL: windows that pass the row's end do not
+// count.  Widths are taken three at a time (the list padded with copies of its
+// last, which never win a tie against it): one three-input maximum, one
+// comparison with the best so far, and the first two values of the winning
+// group kept; which of its three widths it was is found once, at the end.
+template <int PATH, bool TAIL>
+__device__ __forceinline__ void box_outputs(const uint32_t* P, const BoxWidth* sw, const int64_t* sq, int nw, int left,
+                                            int lt, float (&best)[4], int (&bi)[4])
+{
+    const ulonglong2 p0 = *reinterpret_cast<const ulonglong2*>(P + lt);
+    float s0[4], s1[4];
+    const uint64_t minus1 = pack2(-1.0f, -1.0f);
+    auto group = [&](int k0, auto first) {
+        float v[3][4];
 #pragma unroll
-        for (int i = 0; i < kPer; i++) {
-            p0[i] = P[i * kBT + tid];
-            best[i] = -INFINITY;
-            bi[i] = AF_NO_WIDTH;
-        }
-        for (int k = 0; k < nw; k++) {
-            const int ww = sw[k];
-            const float kk = sk[k], cc = -sc[k];
-            const int64_t qq = sq[k];
+        for (int i = 0; i < 3; i++) {
+            const BoxWidth c = sw[k0 + i];
+            const uint32_t* Pw = P + lt + (c.w & ~3);
+            const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(Pw);
+            uint64_t p[2] = {x.x, x.y};
+            if (c.w & 3) shift_words(x, *reinterpret_cast<const ulonglong2*>(Pw + 4), c.w & 3, p);  // uniform
+            if (PATH == kPathFloat) {
+                const uint64_t ne = pack2(__int_as_float(c.e), __int_as_float(c.e2));
+                const uint64_t k2 = pack2(c.k, c.k2), nc = pack2(c.nc, c.nc2);
+                unpack2(fma2(add2(fma2(p0.x, minus1, p[0]), ne), k2, nc), v[i][0], v[i][1]);
+                unpack2(fma2(add2(fma2(p0.y, minus1, p[1]), ne), k2, nc), v[i][2], v[i][3]);
+            } else {
+                const int64_t qq = PATH == kPathWide ? sq[k0 + i] : 0;
 #pragma unroll
-            for (int i = 0; i < kPer; i++) {
-                const uint32_t B = P[i * kBT + tid + ww] - p0[i];
-                float x;
-                if (SMALL)
-                    x = (float)((int32_t)B - (int32_t)qq);
-                else
-                    x = (float)((int64_t)B - qq);
-                const float v = fmaf(x, kk, cc);
-                if (v > best[i]) {
-                    best[i] = v;
-                    bi[i] = k;
+                for (int j = 0; j < 4; j++) {
+                    const uint64_t own = j < 2 ? p0.x : p0.y;
+                    const uint32_t B = (uint32_t)(p[j >> 1] >> (32 * (j & 1))) - (uint32_t)(own >> (32 * (j & 1)));
+                    const float x1 = PATH == kPathInt ? (float)(int32_t)(B - (uint32_t)c.e) : (float)((int64_t)B - qq);
+                    v[i][j] = fmaf(x1, c.k, c.nc);
                 }
             }
-        }
+            if (TAIL) {
 #pragma unroll
-        for (int i = 0; i < kPer; i++) {
-            const int64_t o = base + i * kBT + tid;
-            snr[o] = best[i];
-            if (bw) bw[o] = (uint8_t)bi[i];
-        }
-        return;
-    }
-#pragma unroll 1
-    for (int i = 0; i < kPer; i++) {
-        const int lt = i * kBT + tid;
-        const int64_t t = t0 + lt;
-        if (t >= nout) break;
-        const uint32_t p0 = P[lt];
-        float best = -INFINITY;
-        int bi = AF_NO_WIDTH;
-        for (int k = 0; k < nw; k++) {
-            const int ww = sw[k];
-            if (t + ww > nout) break;
-            const uint32_t B = P[lt + ww] - p0;
-            float x;
-            if (SMALL)
-                x = (float)((int32_t)B - (int32_t)sq[k]);
-            else
-                x = (float)((int64_t)B - sq[k]);
-            const float v = fmaf(x, sk[k], -sc[k]);
-            if (v > best) {
-                best = v;
-                bi = k;
+                for (int j = 0; j < 4; j++)
+                    if (lt + j + c.w > left) v[i][j] = -INFINITY;
             }
         }
-        const int64_t o = base + lt;
-        snr[o] = best;
-        if (bw) bw[o] = (uint8_t)bi;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const float m = max3(v[0][j], v[1][j], v[2][j]);
+            if (decltype(first)::value) {
+                best[j] = m;
+                s0[j] = v[0][j];
+                s1[j] = v[1][j];
+                bi[j] = 0;
+            } else if (m > best[j]) {
+                best[j] = m;
+                s0[j] = v[0][j];
+                s1[j] = v[1][j];
+                bi[j] = k0;
+            }
+        }
+    };
+    group(0, std::true_type{});
+    for (int k0 = 3; k0 < nw; k0 += 3) group(k0, std::false_type{});
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        bi[j] += s0[j] == best[j] ? 0 : (s1[j] == best[j] ? 1 : 2);
+        if (TAIL && best[j] == -INFINITY) bi[j] = AF_NO_WIDTH;
     }
+}
+
+// Block = one tile of one row: `outs` outputs from t0 on, and the prefix words
+// of the tile and its halo, kBW * NCH chunks of 128; t0 is a multiple of outs
+// less the row's misalignment (0 to 3 words), so that every load and store is
+// a whole 16-byte one wherever the row starts (rows of odd length: three of
+// four start off a 16-byte boundary).
+//  1. NCH consecutive chunks per warp are read, one 16-byte load per lane, all
+//     issued first; values outside the row count as mu0, an integer near the
+//     row's mean.
+//  2. P[j] = sum_{k<j} (Y[t0+k] - mu0) mod 2^32: 4 values per lane, a warp
+//     scan per chunk, chunk and warp offsets; one 16-byte store per lane.  The
+//     window sum is P[t+w] - P[t] + w mu0, and B - q = P[t+w] - P[t] - e with
+//     e = q - w mu0.
+//  3. If no |P| of the tile reaches 2^22 (noise: a random walk of a few tens of
+//     thousands), P is stored as floats: B - q then takes two exact fp32
+//     operations, issued two outputs at a time, and no integer-to-float
+//     conversion per (output, width).  Otherwise the integers are stored.
+//  4. A thread takes 4 consecutive outputs at a time, so one 16-byte shared load
+//     brings P[t+w] for four outputs.
+// Bound by instruction issue (99 warp instructions per 32 outputs at 9 widths:
+// 38 of them loads, scan and stores, then 20 per three widths).  1001 x 215261
+// plane, 9 widths up to 256: 0.86 ms with an integer difference, a conversion
+// and a 4-byte shared load per (output, width) and 4-byte global loads on rows
+// off a 16-byte boundary; 0.68 ms so.  Measured slower: two 4-output groups per
+// thread together (80 registers, spills: 0.80 ms), one comparison and two
+// selects per width (0.75 ms), 3 or 5 blocks per SM (0.73 ms).
+template <bool SMALL, int NCH>
+__global__ void __launch_bounds__(kBT, NCH <= 6 ? 4 : 3)
+k_boxcar(const int32_t* __restrict__ Y, int ndm, int64_t nout, int outs, af_widths_t w,
+         const af_rowconst_t* __restrict__ rc, float* __restrict__ snr, uint8_t* __restrict__ bw)
+{
+    constexpr int kWords = kBW * NCH * 128;
+    __shared__ __align__(16) uint32_t P[kWords + 8];
+    __shared__ BoxWidth sw[AF_MAX_WIDTHS + 2];
+    __shared__ int64_t sq[AF_MAX_WIDTHS + 2];
+    __shared__ __align__(16) uint32_t swarp[kBW];
+
+    const int64_t d = blockIdx.y + (int64_t)gridDim.y * blockIdx.z;
+    if (d >= ndm) return;
+    const int nw = w.n;
+    const int nw3 = (nw + 2) / 3 * 3;  // the list in whole groups of three
+    const int32_t* row = Y + d * nout;
+    const int mis = (int)((reinterpret_cast<uintptr_t>(row) >> 2) & 3);
+    const int64_t t0 = (int64_t)blockIdx.x * outs - mis;
+    if (t0 >= nout) return;
+    const int first = blockIdx.x == 0 ? mis : 0;                                 // words before the row's start
+    const int left = (int)(nout - t0 < 2 * kWords ? nout - t0 : 2 * kWords);     // row samples from t0 on (clipped)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const af_rowconst_t* rcd = rc + d * AF_MAX_WIDTHS;
+
+    // 1. loads
+    const int32_t* yt = row + t0;
+    const int i0 = warp * NCH * 128 + 4 * lane;
+    int4 v[NCH];
+#pragma unroll
+    for (int u = 0; u < NCH; u++) {
+        const int i = i0 + 128 * u;
+        v[u] = make_int4(0, 0, 0, 0);
+        if (i >= first && i + 3 < left) v[u] = __ldg(reinterpret_cast<const int4*>(yt + i));
+    }
+    const int32_t mu0 = SMALL ? __float2int_rn(__fdividef(__ll2float_rn(rcd[nw - 1].q), (float)w.w[nw - 1])) : 0;
+    bool wide_e = false;  // an offset e too large for the float path
+    if (tid < nw3) {
+        const int k = min(tid, nw - 1);
+        const af_rowconst_t c = rcd[k];
+        BoxWidth o;
+        o.w = w.w[k];
+        const int32_t e = (int32_t)((uint32_t)c.q - (uint32_t)o.w * (uint32_t)mu0);
+        wide_e = e <= -(1 << kFloatBits) || e >= (1 << kFloatBits);
+        o.e = o.e2 = e;
+        o.k = o.k2 = c.k;
+        o.nc = o.nc2 = -c.c;
+        o.pad = 0;
+        sw[tid] = o;
+        sq[tid] = c.q;
+    }
+#pragma unroll
+    for (int u = 0; u < NCH; u++) {
+        const int i = i0 + 128 * u;
+        if (i >= first && i + 3 < left) {
+            v[u].x -= mu0;
+            v[u].y -= mu0;
+            v[u].z -= mu0;
+            v[u].w -= mu0;
+        } else if (i + 3 >= first && i < left) {  // the row's ends
+            if (i >= first) v[u].x = __ldg(yt + i) - mu0;
+            if (i + 1 >= first && i + 1 < left) v[u].y = __ldg(yt + i + 1) - mu0;
+            if (i + 2 >= first && i + 2 < left) v[u].z = __ldg(yt + i + 2) - mu0;
+            if (i + 3 < left) v[u].w = __ldg(yt + i + 3) - mu0;
+        }
+    }
+
+    // 2. exclusive prefix sums: ex[u] = sum of everything of the warp before the lane's chunk-u values
+    uint32_t ex[NCH], run = 0;
+#pragma unroll
+    for (int u = 0; u < NCH; u++) {
+        const uint32_t own = (uint32_t)v[u].x + (uint32_t)v[u].y + (uint32_t)v[u].z + (uint32_t)v[u].w;
+        uint32_t incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        ex[u] = run + incl - own;
+        run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) swarp[warp] = run;
+    __syncthreads();
+    uint32_t off = 0;
+#pragma unroll
+    for (int k = 0; k < kBW; k++) off += k < warp ? swarp[k] : 0u;
+    int32_t hi = 0, lo = 0;  // range of the tile's prefix sums
+#pragma unroll
+    for (int u = 0; u < NCH; u++) {  // v[u] becomes the lane's four prefix words
+        const uint32_t a = off + ex[u], b = a + (uint32_t)v[u].x, c = b + (uint32_t)v[u].y, e = c + (uint32_t)v[u].z;
+        v[u] = make_int4((int)a, (int)b, (int)c, (int)e);
+        hi = __vimax3_s32(__vimax3_s32(hi, v[u].x, v[u].y), v[u].z, v[u].w);
+        lo = __vimin3_s32(__vimin3_s32(lo, v[u].x, v[u].y), v[u].z, v[u].w);
+    }
+    const bool bad = wide_e || hi >= (1 << kFloatBits) || lo <= -(1 << kFloatBits);
+    // 3. the prefix words in the form the tile's path reads
+    const bool flt = SMALL && __syncthreads_or(bad) == 0;
+#pragma unroll
+    for (int u = 0; u < NCH; u++) {
+        if (flt)
+            *reinterpret_cast<float4*>(P + i0 + 128 * u) =
+                make_float4((float)v[u].x, (float)v[u].y, (float)v[u].z, (float)v[u].w);
+        else
+            *reinterpret_cast<int4*>(P + i0 + 128 * u) = v[u];
+    }
+    if (flt && tid < nw3) sw[tid].e = sw[tid].e2 = __float_as_int(-(float)sw[tid].e);
+    __syncthreads();
+
+    // 4. every width's S/N and the best
+    const int nown = min(outs, left);                     // the tile's outputs
+    const bool tail = left < outs + w.w[nw - 1];          // some windows pass the row's end (uniform)
+    float* so = snr + d * nout + t0;
+    uint8_t* bo = bw ? bw + d * nout + t0 : nullptr;
+    const bool vec = (reinterpret_cast<uintptr_t>(so) & 15) == 0 && (reinterpret_cast<uintptr_t>(bo) & 3) == 0;
+#pragma unroll 1
+    for (int lt = 4 * tid; lt < nown; lt += 4 * kBT) {
+        float best[4];
+        int bi[4];
+        if (!SMALL) {
+            if (tail) box_outputs<kPathWide, true>(P, sw, sq, nw, left, lt, best, bi);
+            else box_outputs<kPathWide, false>(P, sw, sq, nw, left, lt, best, bi);
+        } else if (flt) {
+            if (tail) box_outputs<kPathFloat, true>(P, sw, sq, nw, left, lt, best, bi);
+            else box_outputs<kPathFloat, false>(P, sw, sq, nw, left, lt, best, bi);
+        } else {
+            if (tail) box_outputs<kPathInt, true>(P, sw, sq, nw, left, lt, best, bi);
+            else box_outputs<kPathInt, false>(P, sw, sq, nw, left, lt, best, bi);
+        }
+        if (vec && lt >= first && lt + 3 < nown) {
+            *reinterpret_cast<float4*>(so + lt) = make_float4(best[0], best[1], best[2], best[3]);
+            if (bo)
+                *reinterpret_cast<uint32_t*>(bo + lt) =
+                    (uint32_t)bi[0] | (uint32_t)bi[1] << 8 | (uint32_t)bi[2] << 16 | (uint32_t)bi[3] << 24;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (lt + j >= first && lt + j < nown) {
+                    so[lt + j] = best[j];
+                    if (bo) bo[lt + j] = (uint8_t)bi[j];
+                }
+        }
+    }
+}
+
+template <bool SMALL, int NCH>
+int launch_boxcar_nch(const int32_t* d_plane, int ndm, int64_t nout, const af_widths_t& w,
+                      const af_rowconst_t* d_rowconst, float* d_best_snr, uint8_t* d_best_w, cudaStream_t s)
+{
+    // a tile's prefix words less its halo, in whole 16-byte groups
+    const int outs = (kBW * NCH * 128 - w.w[w.n - 1]) & ~3;
+    const int64_t tiles = (nout + 3 + outs - 1) / outs;  // a row may start up to 3 words into its first tile
+    if ((long double)tiles * ndm > 0x7fffffffLL) return af_set_error(AF_EINVAL, "boxcar: problem too large for one grid");
+    const int gy = ndm < 32768 ? ndm : 32768;
+    const dim3 grid((unsigned)tiles, (unsigned)gy, (unsigned)((ndm + gy - 1) / gy));
+    k_boxcar<SMALL, NCH><<<grid, kBT, 0, s>>>(d_plane, ndm, nout, outs, w, d_rowconst, d_best_snr, d_best_w);
+    return af_cuda_check(cudaGetLastError(), "boxcar launch");
 }
 
 int launch_boxcar_tiles(const int32_t* d_plane, int ndm, int64_t nout, const af_widths_t& w,
                         const af_rowconst_t* d_rowconst, float* d_best_snr, uint8_t* d_best_w, cudaStream_t s)
 {
-    const unsigned tiles = (unsigned)((nout + kBOut - 1) / kBOut);
-    const unsigned long long nblk = (unsigned long long)tiles * (unsigned long long)ndm;
-    if (nblk > 0x7fffffffULL) return af_set_error(AF_EINVAL, "boxcar: problem too large for one grid");
-    const int L = kBOut + w.w[w.n - 1] - 1;
-    const int C = ((L + kBT - 1) / kBT) | 1;
-    const size_t smem = (size_t)(kBT * C + 4) * sizeof(uint32_t);
-    const void* fn = w.small ? (const void*)k_boxcar<true> : (const void*)k_boxcar<false>;
-    if (smem > 48 * 1024)
-        if (int rc = af_ensure_smem(fn, smem)) return rc;
+    // 6144 prefix words per tile for widths up to 1024 samples, 12288 up to 8192
+    const bool near = w.w[w.n - 1] <= 1024;
     if (w.small)
-        k_boxcar<true><<<(unsigned)nblk, kBT, smem, s>>>(d_plane, nout, tiles, w, d_rowconst, d_best_snr, d_best_w);
-    else
-        k_boxcar<false><<<(unsigned)nblk, kBT, smem, s>>>(d_plane, nout, tiles, w, d_rowconst, d_best_snr, d_best_w);
-    return af_cuda_check(cudaGetLastError(), "boxcar launch");
+        return near ? launch_boxcar_nch<true, 6>(d_plane, ndm, nout, w, d_rowconst, d_best_snr, d_best_w, s)
+                    : launch_boxcar_nch<true, 12>(d_plane, ndm, nout, w, d_rowconst, d_best_snr, d_best_w, s);
+    return near ? launch_boxcar_nch<false, 6>(d_plane, ndm, nout, w, d_rowconst, d_best_snr, d_best_w, s)
+                : launch_boxcar_nch<false, 12>(d_plane, ndm, nout, w, d_rowconst, d_best_snr, d_best_w, s);
 }
 
 // ---------------------------------------------------------------- robust S/N
