@@ -11,6 +11,7 @@
 // result is within a few ulp of the exact S/N.  Window sums come from 32-bit
 // prefix sums taken modulo 2^32, which are exact as long as every window sum
 // is below 2^32 (checked on the host: w * 255 * nchan < 2^32).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
@@ -19,6 +20,8 @@
 #include <type_traits>
 
 #include "internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -528,16 +531,23 @@ __device__ bool robust_select(const int32_t* __restrict__ y, int64_t n, int32_t 
     return true;
 }
 
-__global__ void __launch_bounds__(kRT, 2) k_row_robust(const int32_t* __restrict__ Y, int64_t nout,
-                                                    af_robust_t* __restrict__ out)
+// Scratch of the selection over a whole row by one block.
+struct RobustScratch {
+    uint32_t hist[kRB];
+    long long sel[3];
+    long long sred[kRT / 32];
+    int32_t smin[kRT / 32], smax[kRT / 32];
+    float ssq[kRT / 32];
+};
+
+// Median and MAD of a row in up to three passes (the windows above).
+__device__ __noinline__ void row_robust_general(const int32_t* __restrict__ y, int64_t nout, RobustScratch& sc,
+                                   af_robust_t* __restrict__ out)
 {
-    __shared__ uint32_t hist[kRB];
-    __shared__ long long sel[3];
-    __shared__ long long sred[kRT / 32];
-    __shared__ int32_t smin[kRT / 32], smax[kRT / 32];
-    __shared__ float ssq[kRT / 32];
-    const int d = blockIdx.x;
-    const int32_t* y = Y + (int64_t)d * nout;
+    uint32_t* hist = sc.hist;
+    long long *sel = sc.sel, *sred = sc.sred;
+    int32_t *smin = sc.smin, *smax = sc.smax;
+    float* ssq = sc.ssq;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // pass 1: range, and sums of u = v - y[0] (exact) and of u^2 (fp32 per thread; only the window depends on it)
     const int32_t y0 = __ldg(y);
@@ -598,9 +608,317 @@ __global__ void __launch_bounds__(kRT, 2) k_row_robust(const int32_t* __restrict
     if (!robust_select<1>(y, nout, med, (uint64_t)wm + 1, k, hist, sel, sred, &mad))
         robust_select<1>(y, nout, med, (uint64_t)r2 + 1, k, hist, sel, sred, &mad);
     if (tid == 0) {
-        out[d].median = med;
-        out[d].mad = mad;
+        out->median = med;
+        out->mad = mad;
     }
+}
+
+__global__ void __launch_bounds__(kRT, 2) k_row_robust(const int32_t* __restrict__ Y, int64_t nout,
+                                                    af_robust_t* __restrict__ out)
+{
+    __shared__ RobustScratch sc;
+    row_robust_general(Y + (int64_t)blockIdx.x * nout, nout, sc, out + blockIdx.x);
+}
+
+// ---- long rows: one pass.  A sample of 4096 values (1024 16-byte pieces at
+// even steps) gives estimates m of the median and M of the MAD, good to a few
+// hundredths of sigma on any smooth distribution.  One pass over the row then
+// counts, at unit resolution, the values in three windows -- around m, m - M
+// and m + M, each a few estimate errors wide -- and the values below each
+// window.  Cumulative counts C(z) = #(v < z) are therefore exact for z inside a
+// window, and the exact median (the value holding rank k = (n - 1) / 2) and MAD
+// (the smallest x with C(med + x + 1) - C(med - x) > k) follow without another
+// pass: both are checked against the windows' edges, and a row whose answer
+// lies outside them (none seen on noise) takes the general selection.  Where
+// the windows meet (M of a few units) one dense window covers them all.
+// A cluster of blocks shares a row, each counting one part; the first block
+// adds up the others' counts through distributed shared memory.  Bound by issue
+// (about 25 instructions per 32 values, the three window tests and counts) and
+// HBM: 1001 x 215261 plane 0.53 ms in three passes, 0.24 ms in one.
+// Rows below 16384 values keep the general selection: the sample would be a
+// quarter of the row and more.
+constexpr int kRS = 4096;                 // sample values
+constexpr int64_t kRobustOnePass = 16384; // shortest row for the one-pass kernel
+constexpr int kRH = 6144;                 // histogram bins of all windows
+
+struct RobustOnePass {
+    union {
+        RobustScratch gen;
+        struct {
+            uint32_t hist[kRH];           // counts per bin, then exclusive prefix sums
+            uint32_t wsum[kRT / 32];
+            uint32_t below[3];            // values below each window (of this block's part)
+            int32_t lo, hi;               // sample range
+            uint32_t bin, cum;            // a search's answer
+            int32_t med, mad;
+            int ok;
+        } one;
+    };
+};
+
+// Block-wide: the bin of hist[0 .. 4 kRT) where the running count passes rank
+// and the count before it, in sc.bin and sc.cum.
+__device__ __forceinline__ void find_rank(RobustOnePass& sc, uint32_t rank)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint4 h = *reinterpret_cast<const uint4*>(sc.one.hist + 4 * tid);
+    const uint32_t own = h.x + h.y + h.z + h.w;
+    uint32_t incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) sc.one.wsum[warp] = incl;
+    __syncthreads();
+    uint32_t cum = incl - own;
+    for (int k = 0; k < warp; k++) cum += sc.one.wsum[k];
+    if (cum <= rank && rank < cum + own) {
+        const uint32_t hv[4] = {h.x, h.y, h.z, h.w};
+        int j = 0;
+        while (rank >= cum + hv[j]) cum += hv[j++];
+        sc.one.bin = 4 * tid + j;
+        sc.one.cum = cum;
+    }
+    __syncthreads();
+}
+
+// Estimate (lower median of the sample's keys, to within *res) by at most two
+// histogram passes of 2048 bins over [0, range].
+__device__ __forceinline__ uint32_t sample_median(const uint32_t (&key)[kRS / kRT], uint32_t range, RobustOnePass& sc,
+                                                  uint32_t* res)
+{
+    const int tid = threadIdx.x;
+    uint32_t start = 0, rank = (kRS - 1) / 2;
+    int s = max(0, 21 - __clz(range));  // bins of 2^s: range >> s < 2048
+    for (int pass = 0; pass < 2; pass++) {
+        *reinterpret_cast<uint4*>(sc.one.hist + 4 * tid) = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kRS / kRT; j++) {
+            const uint32_t b = (key[j] - start) >> s;
+            if (key[j] >= start && b < (uint32_t)kRB) atomicAdd(&sc.one.hist[b], 1u);
+        }
+        __syncthreads();
+        find_rank(sc, rank);
+        start += sc.one.bin << s;
+        rank -= sc.one.cum;
+        __syncthreads();
+        if (s == 0) break;
+        if (pass == 0) s = max(0, s - 11);
+    }
+    *res = s == 0 ? 0u : (1u << s);
+    return start;
+}
+
+__global__ void __launch_bounds__(kRT, 2)
+k_row_robust1(const int32_t* __restrict__ Y, int64_t nout, af_robust_t* __restrict__ out)
+{
+    __shared__ __align__(16) RobustOnePass sc;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
+    const int64_t d = blockIdx.x / parts;
+    const int32_t* y = Y + d * nout;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t head = (int64_t)(((16u - ((uint32_t)reinterpret_cast<uintptr_t>(y) & 15u)) & 15u) >> 2);
+    const int4* y4 = reinterpret_cast<const int4*>(y + head);
+    const int64_t n4 = (nout - head) >> 2;
+
+    // the sample, its range
+    int32_t sv[kRS / kRT];
+    {
+        const int64_t step = n4 / (kRS / 4);
+#pragma unroll
+        for (int j = 0; j < kRS / kRT / 4; j++) {
+            const int4 v = __ldg(y4 + (tid + j * kRT) * step);
+            sv[4 * j] = v.x;
+            sv[4 * j + 1] = v.y;
+            sv[4 * j + 2] = v.z;
+            sv[4 * j + 3] = v.w;
+        }
+    }
+    if (tid == 0) {
+        sc.one.lo = INT32_MAX;
+        sc.one.hi = INT32_MIN;
+        sc.one.below[0] = sc.one.below[1] = sc.one.below[2] = 0u;
+    }
+    __syncthreads();
+    int32_t lo = sv[0], hi = sv[0];
+#pragma unroll
+    for (int j = 1; j < kRS / kRT; j++) {
+        lo = min(lo, sv[j]);
+        hi = max(hi, sv[j]);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+        atomicMin(&sc.one.lo, lo);
+        atomicMax(&sc.one.hi, hi);
+    }
+    __syncthreads();
+    lo = sc.one.lo;
+    hi = sc.one.hi;
+    uint32_t key[kRS / kRT], res, rmad;
+#pragma unroll
+    for (int j = 0; j < kRS / kRT; j++) key[j] = (uint32_t)sv[j] - (uint32_t)lo;
+    const uint32_t mk = sample_median(key, (uint32_t)hi - (uint32_t)lo, sc, &res);
+    const int32_t m = (int32_t)((uint32_t)lo + mk);
+#pragma unroll
+    for (int j = 0; j < kRS / kRT; j++) key[j] = sv[j] >= m ? (uint32_t)sv[j] - (uint32_t)m : (uint32_t)m - (uint32_t)sv[j];
+    const uint32_t M = sample_median(key, max((uint32_t)hi - (uint32_t)m, (uint32_t)m - (uint32_t)lo), sc, &rmad);
+
+    // windows: 5 standard errors of a normal sample's estimates (0.029 M and 0.034 M) and the estimates' resolution
+    const bool sane = M < (1u << 20) && res < (1u << 20) && rmad < (1u << 20);
+    const int32_t dc = (int32_t)(M / 7) + 2 + (int32_t)min(res, 1u << 20);
+    const int32_t dw = (int32_t)(M / 5) + 2 + (int32_t)min(res + rmad, 1u << 20);
+    const int32_t in = (int32_t)min(M, 1u << 20) - dw, outer = (int32_t)min(M, 1u << 20) + dw;  // |v - m| of the outer windows
+    const bool dense = in <= dc;
+    const int64_t bins = dense ? 2 * (int64_t)outer + 1 : 2 * (int64_t)dc + 1 + 2 * (2 * (int64_t)dw + 1);
+    // windows inside the int32 range, so that (v - start) mod 2^32 < width exactly for the values in them
+    const bool fits = sane && bins <= kRH && (int64_t)m - outer >= INT32_MIN && (int64_t)m + outer < INT32_MAX;
+    // window starts (as v - m), widths and first bins: below m - M, around m, above m + M; dense: the first alone
+    const int32_t w0 = -outer, w1 = -dc, w2 = in;
+    const int nb0 = dense ? 2 * outer + 1 : 2 * dw + 1, nb1 = dense ? 0 : 2 * dc + 1, nb2 = dense ? 0 : 2 * dw + 1;
+    if (fits) {
+        for (int i = tid; i < nb0 + nb1 + nb2; i += kRT) sc.one.hist[i] = 0u;
+        __syncthreads();
+        uint32_t b0 = 0, b1 = 0, b2 = 0;
+        // shared address of value v's bin: 4 v + k0, k1 or k2 (mod 2^32) by its window
+        const uint32_t s0 = (uint32_t)(m + w0), s1 = (uint32_t)(m + w1), s2 = (uint32_t)(m + w2);
+        const uint32_t hb = (uint32_t)__cvta_generic_to_shared(sc.one.hist);
+        const uint32_t k0 = hb - 4u * s0, k1 = hb + 4u * ((uint32_t)nb0 - s1), k2 = hb + 4u * ((uint32_t)(nb0 + nb1) - s2);
+        auto count = [&](int32_t v) {  // dense: windows 1 and 2 are empty, their counts are not used
+            asm volatile(
+                "{\n\t.reg .pred p, q, r;\n\t.reg .u32 a, k;\n\t"
+                "setp.lt.s32 p, %3, %4;\n\t@p add.u32 %0, %0, 1;\n\t"
+                "setp.lt.s32 p, %3, %5;\n\t@p add.u32 %1, %1, 1;\n\t"
+                "setp.lt.s32 p, %3, %6;\n\t@p add.u32 %2, %2, 1;\n\t"
+                "sub.u32 a, %3, %4;\n\tsetp.lt.u32 p, a, %7;\n\t"
+                "sub.u32 a, %3, %5;\n\tsetp.lt.or.u32 q, a, %8, p;\n\t"
+                "sub.u32 a, %3, %6;\n\tsetp.lt.or.u32 r, a, %9, q;\n\t"
+                "selp.u32 k, %11, %12, q;\n\tselp.u32 k, %10, k, p;\n\t"
+                "mad.lo.u32 a, %3, 4, k;\n\t@r red.shared.add.u32 [a], 1;\n\t}"
+                : "+r"(b0), "+r"(b1), "+r"(b2)
+                : "r"(v), "r"(s0), "r"(s1), "r"(s2), "r"(nb0), "r"(nb1), "r"(nb2), "r"(k0), "r"(k1), "r"(k2)
+                : "memory");
+        };
+        // this block's part of the row, in 16-byte pieces; the first block also takes the row's unaligned ends
+        const int64_t q0 = n4 * part / parts, q1 = n4 * (part + 1) / parts;
+        const int4* p = y4 + q0 + tid;
+        const int steps = (int)((q1 - q0) / (kRT * kRU4));  // whole steps of the block
+        for (int f = 0; f < steps; f++, p += kRT * kRU4) {
+            int4 v[kRU4];
+#pragma unroll
+            for (int u = 0; u < kRU4; u++) v[u] = __ldg(p + u * kRT);
+#pragma unroll
+            for (int u = 0; u < kRU4; u++) {
+                count(v[u].x);
+                count(v[u].y);
+                count(v[u].z);
+                count(v[u].w);
+            }
+        }
+        for (const int4* e = y4 + q1; p < e; p += kRT) {  // at most kRU4 - 1 pieces a thread
+            const int4 t = __ldg(p);
+            count(t.x);
+            count(t.y);
+            count(t.z);
+            count(t.w);
+        }
+        if (part == 0) {
+            if (tid < head) count(__ldg(y + tid));
+            const int64_t t0 = head + 4 * n4;
+            if (t0 + tid < nout) count(__ldg(y + t0 + tid));  // at most 3 values
+        }
+        b0 = __reduce_add_sync(0xffffffffu, b0);
+        b1 = __reduce_add_sync(0xffffffffu, b1);
+        b2 = __reduce_add_sync(0xffffffffu, b2);
+        if (lane == 0) {
+            atomicAdd(&sc.one.below[0], b0);
+            atomicAdd(&sc.one.below[1], b1);
+            atomicAdd(&sc.one.below[2], b2);
+        }
+    }
+    cluster.sync();  // every block's counts are final (all blocks of a cluster share the windows: same sample)
+    bool done = false;
+    if (part == 0 && fits) {
+        const int nb = nb0 + nb1 + nb2;
+        for (int q = 1; q < parts; q++) {
+            const RobustOnePass* r = cluster.map_shared_rank(&sc, q);
+            for (int i = tid; i < nb; i += kRT) sc.one.hist[i] += r->one.hist[i];
+            if (tid < 3) sc.one.below[tid] += r->one.below[tid];
+        }
+        if (tid == 0) sc.one.ok = 0;
+        __syncthreads();
+        // exclusive prefix sums of the bins, in place, 4 kRT at a time
+        const int warp = tid >> 5;
+        uint32_t base = 0;
+        for (int c0 = 0; c0 < nb; c0 += 4 * kRT) {
+            const int i = c0 + 4 * tid;
+            uint32_t h[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) h[j] = i + j < nb ? sc.one.hist[i + j] : 0u;
+            const uint32_t own = h[0] + h[1] + h[2] + h[3];
+            uint32_t incl = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (lane == 31) sc.one.wsum[warp] = incl;
+            __syncthreads();
+            uint32_t e = base + incl - own;
+            for (int k = 0; k < warp; k++) e += sc.one.wsum[k];
+            for (int k = 0; k < kRT / 32; k++) base += sc.one.wsum[k];
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (i + j < nb) {
+                    sc.one.hist[i + j] = e;
+                    e += h[j];
+                }
+            __syncthreads();  // wsum is read before the next chunk writes it
+        }
+        // C(z) - (values below window s) for z = window start + i, 0 <= i <= its bins
+        const uint32_t total = base;
+        auto cnt = [&](int s, int i) -> int64_t {
+            const int first = s == 0 ? 0 : s == 1 ? nb0 : nb0 + nb1;
+            const uint32_t e = first + i < nb ? sc.one.hist[first + i] : total;
+            return (int64_t)sc.one.below[s] + (int64_t)(e - sc.one.hist[first]);
+        };
+        const int64_t k = (nout - 1) / 2;
+        const int sm = dense ? 0 : 1, nbm = dense ? nb0 : nb1, wm = dense ? w0 : w1;
+        // the median: the bin of its window that holds rank k
+        for (int i = tid; i < nbm; i += kRT)
+            if (cnt(sm, i) <= k && k < cnt(sm, i + 1)) {
+                sc.one.med = wm + i;
+                sc.one.ok = 1;
+            }
+        __syncthreads();
+        if (sc.one.ok == 1) {
+            const int med = sc.one.med;  // relative to m
+            // N(x) = C(med + x + 1) - C(med - x) = #(|v - median| <= x), for x with both ends inside their windows
+            const int sl = 0, sr = dense ? 0 : 2, wr = dense ? w0 : w2, nbr = dense ? nb0 : nb2;
+            const int xlo = dense ? -1 : max(wr - med - 1, med - (w0 + nb0));
+            const int xhi = min(wr + nbr - med - 1, med - w0);
+            auto N = [&](int x) -> int64_t { return x < 0 ? 0 : cnt(sr, med + x + 1 - wr) - cnt(sl, med - x - w0); };
+            for (int x = xlo + 1 + tid; x <= xhi; x += kRT)
+                if (N(x) > k && N(x - 1) <= k) {
+                    sc.one.mad = x;
+                    sc.one.ok = 2;
+                }
+        }
+        __syncthreads();
+        if (sc.one.ok == 2) {
+            done = true;
+            if (tid == 0) {
+                out[d].median = (int32_t)((uint32_t)m + (uint32_t)sc.one.med);
+                out[d].mad = sc.one.mad;
+            }
+        }
+        __syncthreads();
+    }
+    cluster.sync();  // the first block has read the others' shared memory
+    if (part == 0 && !done) row_robust_general(y, nout, sc.gen, out + d);
 }
 
 // Robust S/N constants: snr = (B - w*med) * k, k = 1/(1.482602218505602 * mad * sqrt(w)).
@@ -623,8 +941,25 @@ __global__ void k_rowconst_robust(const af_robust_t* __restrict__ r, int ndm, af
 
 int af_launch_row_robust(const int32_t* d_plane, int ndm, int64_t nout, af_robust_t* d_robust, cudaStream_t s)
 {
-    k_row_robust<<<ndm, kRT, 0, s>>>(d_plane, nout, d_robust);
-    return af_cuda_check(cudaGetLastError(), "robust row statistics launch");
+    if (nout < kRobustOnePass || nout > INT32_MAX) {
+        k_row_robust<<<ndm, kRT, 0, s>>>(d_plane, nout, d_robust);
+        return af_cuda_check(cudaGetLastError(), "robust row statistics launch");
+    }
+    // blocks per row: enough for two per SM, each with at least 32768 values
+    int parts = 1;
+    while (parts < 8 && (int64_t)ndm * parts < 1216 && nout / (2 * parts) >= 16384) parts *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ndm * parts));
+    cfg.blockDim = dim3(kRT);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)parts;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return af_cuda_check(cudaLaunchKernelEx(&cfg, k_row_robust1, d_plane, nout, d_robust),
+                         "robust row statistics launch");
 }
 
 int af_launch_boxcar_robust(const int32_t* d_plane, int ndm, int64_t nout, const af_robust_t* d_robust,
