@@ -15,12 +15,14 @@
 //
 // Two passes over the plane: the first finds each slice's min and max
 // (block reduction + 64-bit atomics into the caller's work array), the
-// second recomputes the values and writes Y.  One block per output row of a
-// slice; a thread per output column (strided).
+// second recomputes the values and writes Y, its blocks in reverse order so
+// that it begins with what the first left in L2.
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "internal.h"
 
@@ -39,25 +41,201 @@ __device__ __forceinline__ double dval(long long k)
     return __longlong_as_double(k >= 0 ? k : k ^ 0x7FFFFFFFFFFFFFFFLL);
 }
 
-__device__ __forceinline__ long long area_value(const int32_t* __restrict__ X, int64_t nout, int h, int64_t c0,
-                                                int w, int M, int i, int j)
+// Block-wide minimum and maximum into the slice's pair of the work array.
+__device__ __forceinline__ void slice_minmax(long long lo, long long hi, long long* work)
 {
-    const long long ri0 = (long long)i * h, ri1 = (long long)(i + 1) * h;
-    const long long cj0 = (long long)j * w, cj1 = (long long)(j + 1) * w;
-    const int r_lo = (int)(ri0 / M), r_hi = (int)((ri1 - 1) / M);
-    const int c_lo = (int)(cj0 / M), c_hi = (int)((cj1 - 1) / M);
-    long long W = 0;
-    for (int r = r_lo; r <= r_hi; r++) {
-        const long long ovr = min(ri1, (long long)(r + 1) * M) - max(ri0, (long long)r * M);
-        const int32_t* x = X + (int64_t)r * nout + c0;
-        long long row = 0;
-        for (int c = c_lo; c <= c_hi; c++) {
-            const long long ovc = min(cj1, (long long)(c + 1) * M) - max(cj0, (long long)c * M);
-            row += ovc * (long long)__ldg(x + c);
-        }
-        W += ovr * row;
+    __shared__ long long slo[kGT / 32], shi[kGT / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
-    return W;
+    if ((threadIdx.x & 31) == 0) {
+        slo[threadIdx.x >> 5] = lo;
+        shi[threadIdx.x >> 5] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < kGT / 32; k++) {
+            lo = min(lo, slo[k]);
+            hi = max(hi, shi[k]);
+        }
+        atomicMin(work, lo);
+        atomicMax(work + 1, hi);
+    }
+}
+
+// floor((510 a + r) / (2 r)), 0 <= a <= r, r > 0: from a float estimate (within
+// one) and exact 64-bit tests where 512 r fits, else by 128-bit division.
+__device__ __forceinline__ uint32_t gray(unsigned long long a, unsigned long long r)
+{
+    if (r >> 54) return (uint32_t)((510 * (unsigned __int128)a + r) / (2 * (unsigned __int128)r));
+    const unsigned long long num = 510 * a + r, den = 2 * r;
+    uint32_t y = (uint32_t)(255.0f * __fdividef((float)a, (float)r) + 0.5f);
+    if (y * den > num) y--;
+    else if ((y + 1) * den <= num) y++;
+    return y;
+}
+
+// Area path.  Block = (slice, output row i, run of kGT output columns): the
+// plane rows that row i covers are added, weighted, column by column with
+// coalesced loads into V[c] = sum_r ovr(i, r) X[r][c] (shared memory, as many
+// columns at a time as fit), and thread j sums its pixel's columns from there, the
+// first and last weighted.  V is int32 while every value of the block's columns is
+// non-negative and (their bitwise or) x h is below 2^31 (planes of 8-bit sums);
+// otherwise the block starts again with int64.  PASS 0: min / max into work;
+// PASS 1: write Y.
+// Bound by HBM (the plane twice).  22 slices of 1001 x 10173 to 512 x 512: a pass
+// took 0.42 ms with every pixel loading its own 20 columns of 2 to 3 rows (lanes
+// 80 bytes apart) and 64-bit divisions per pixel, 0.31 ms with V in int64, 0.23 ms so
+// (latency: a block's loads, sums and reduction follow one another; rows staged by
+// asynchronous copies in 128-thread blocks took the same).
+constexpr int kGU = 5;                    // columns per thread and step
+constexpr int kGCBytes = 5632 * 4;        // shared memory for V, at most
+
+struct AreaRows {
+    const int32_t* x;      // row r_lo, first column of the slice
+    int64_t nout;
+    int n, lo, hi, M;      // rows, weights of the first and last, of the others
+};
+
+// One step of kGU columns c, c + kGT, ...: adds rows at p0, p1, p2 (first column
+// c of each) with their weights, all loads first.  CHECK: columns from n on do
+// not exist.
+template <typename T, bool CHECK>
+__device__ __forceinline__ int32_t area_step(const int32_t* p0, const int32_t* p1, const int32_t* p2, int o0, int o1,
+                                             int o2, int c, int n, T (&v)[kGU])
+{
+    int32_t y[3][kGU], any = 0;
+#pragma unroll
+    for (int u = 0; u < kGU; u++) {
+        const bool in = !CHECK || c + u * kGT < n;
+        y[0][u] = in ? __ldg(p0 + u * kGT) : 0;
+        y[1][u] = in ? __ldg(p1 + u * kGT) : 0;
+        y[2][u] = in ? __ldg(p2 + u * kGT) : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < kGU; u++) {
+        any |= y[0][u] | y[1][u];
+        any |= y[2][u];
+        v[u] += (T)o0 * y[0][u] + (T)o1 * y[1][u] + (T)o2 * y[2][u];
+    }
+    return any;
+}
+
+// V[c] of columns c0 .. c0 + n - 1 into shared memory; returns the or of the
+// values read.  Rows are taken three at a time (a missing one repeats the last
+// row with weight 0); up to three rows (images of up to twice as many DMs as
+// rows) need no loop over them.
+template <typename T>
+__device__ __forceinline__ int32_t area_columns(const AreaRows& a, int c0, int n, T* V)
+{
+    const int tid = (int)threadIdx.x;
+    int32_t any = 0;
+    auto weight = [&](int k) { return k == 0 ? a.lo : k < a.n - 1 ? a.M : k == a.n - 1 ? a.hi : 0; };
+    const int32_t* x = a.x + c0 + tid;
+    if (a.n <= 3) {
+        const int32_t *p0 = x, *p1 = x + (int64_t)min(1, a.n - 1) * a.nout, *p2 = x + (int64_t)min(2, a.n - 1) * a.nout;
+        const int o0 = weight(0), o1 = weight(1), o2 = weight(2);
+        int c = tid;
+        for (; c + (kGU - 1) * kGT < n; c += kGU * kGT, p0 += kGU * kGT, p1 += kGU * kGT, p2 += kGU * kGT) {
+            T v[kGU] = {};
+            any |= area_step<T, false>(p0, p1, p2, o0, o1, o2, c, n, v);
+#pragma unroll
+            for (int u = 0; u < kGU; u++) V[c + u * kGT] = v[u];
+        }
+        if (c < n) {
+            T v[kGU] = {};
+            any |= area_step<T, true>(p0, p1, p2, o0, o1, o2, c, n, v);
+#pragma unroll
+            for (int u = 0; u < kGU; u++)
+                if (c + u * kGT < n) V[c + u * kGT] = v[u];
+        }
+        return any;
+    }
+    for (int c = tid; c < n; c += kGU * kGT, x += kGU * kGT) {
+        T v[kGU] = {};
+        for (int r = 0; r < a.n; r += 3)
+            any |= area_step<T, true>(x + (int64_t)r * a.nout, x + (int64_t)min(r + 1, a.n - 1) * a.nout,
+                                      x + (int64_t)min(r + 2, a.n - 1) * a.nout, weight(r), weight(r + 1), weight(r + 2),
+                                      c, n, v);
+#pragma unroll
+        for (int u = 0; u < kGU; u++)
+            if (c + u * kGT < n) V[c + u * kGT] = v[u];
+    }
+    return any;
+}
+
+// a / M; small: a < 2^32, where a 64-bit division would take several times as long.
+__device__ __forceinline__ int div_m(long long a, int M, bool small)
+{
+    return small ? (int)((uint32_t)a / (uint32_t)M) : (int)(a / M);
+}
+
+template <int PASS>
+__global__ void __launch_bounds__(kGT, 4)
+k_grid_area(const int32_t* __restrict__ X, int h, int64_t nout, int64_t ns, int s0, int M, unsigned runs, int cols,
+            long long* __restrict__ work, uint8_t* __restrict__ out)
+{
+    extern __shared__ long long smem[];  // cols int32
+    const unsigned blk = PASS == 0 ? blockIdx.x : gridDim.x - 1 - blockIdx.x;
+    const int i = (int)(blk / runs % (unsigned)M), s = s0 + (int)(blk / runs / (unsigned)M);
+    const int j0 = (int)(blk % runs) * kGT, j = j0 + (int)threadIdx.x;
+    const int64_t c0 = (int64_t)s * ns;
+    const int w = (int)min(ns, nout - c0);
+    const long long ri0 = (long long)i * h, ri1 = ri0 + h;
+    const bool small = (long long)M * max(h, w) + w < (1LL << 32);
+    const int r_lo = div_m(ri0, M, small), r_hi = div_m(ri1 - 1, M, small);
+    AreaRows rows;
+    rows.x = X + c0 + (int64_t)r_lo * nout;
+    rows.nout = nout;
+    rows.n = r_hi - r_lo + 1;
+    rows.lo = (int)(min(ri1, (long long)(r_lo + 1) * M) - ri0);
+    rows.hi = (int)(ri1 - (long long)r_hi * M);
+    rows.M = M;
+    // the pixel's columns [cj0, cj1) / M, the block's
+    const long long cj0 = (long long)j * w, cj1 = cj0 + w;
+    const bool in = j < M;
+    const int c_lo = in ? div_m(cj0, M, small) : 0, c_hi = in ? div_m(cj1 - 1, M, small) : 0;
+    const int b_lo = div_m((long long)j0 * w, M, small), b_hi = div_m((long long)min(j0 + kGT, M) * w - 1, M, small);
+    // weights of the parts of the pixel's first and last column outside it
+    const int out_lo = (int)(cj0 - (long long)c_lo * M), out_hi = (int)((long long)(c_hi + 1) * M - cj1);
+    long long W = 0;
+    // adds the pixel's part of columns k0 .. k0 + n - 1 (modulo 2^64: the pixel's sum fits, its parts may not)
+    auto add = [&](const auto* V, int k0, int n) {
+        const int a = max(c_lo, k0), e = min(c_hi, k0 + n - 1);
+        unsigned long long sum = 0;
+        for (int c = a; c <= e; c++) sum += (unsigned long long)((long long)V[c - k0] * M);
+        if (a == c_lo && a <= e) sum -= (unsigned long long)((long long)V[c_lo - k0] * out_lo);
+        if (e == c_hi && a <= e) sum -= (unsigned long long)((long long)V[c_hi - k0] * out_hi);
+        W = (long long)((unsigned long long)W + sum);
+    };
+    bool wide = false;
+    for (int k0 = b_lo; k0 <= b_hi && !wide; k0 += cols) {
+        const int n = min(cols, b_hi + 1 - k0);
+        int32_t* V = reinterpret_cast<int32_t*>(smem);
+        if (k0 > b_lo) __syncthreads();  // the last columns are read
+        const int32_t any = area_columns(rows, k0, n, V);
+        wide = __syncthreads_or(any < 0 || (long long)any * h > INT32_MAX);
+        if (!wide && j < M) add(V, k0, n);
+    }
+    if (wide) {
+        W = 0;
+        for (int k0 = b_lo; k0 <= b_hi; k0 += cols / 2) {
+            const int n = min(cols / 2, b_hi + 1 - k0);
+            __syncthreads();
+            area_columns(rows, k0, n, smem);
+            __syncthreads();
+            if (j < M) add(smem, k0, n);
+        }
+    }
+    if (PASS == 0) {
+        slice_minmax(j < M ? W : LLONG_MAX, j < M ? W : LLONG_MIN, work + 2 * s);
+    } else if (j < M) {
+        const long long lo = work[2 * s];
+        const unsigned long long rng = (unsigned long long)(work[2 * s + 1] - lo);
+        out[((int64_t)s * M + i) * M + j] = rng == 0 ? (uint8_t)0 : (uint8_t)gray((unsigned long long)(W - lo), rng);
+    }
 }
 
 // Lanczos-4 taps of output index i for an axis of n input samples.
@@ -84,24 +262,6 @@ __device__ __forceinline__ int lanczos_taps(int i, int n, int M, double* wt)
     return k0 - 3;
 }
 
-__device__ __forceinline__ double lanczos_value(const int32_t* __restrict__ X, int64_t nout, int h, int64_t c0,
-                                                int w, int M, const double* wr, int r0, int j)
-{
-    double wc[8];
-    const int k0 = lanczos_taps(j, w, M, wc);
-    double U = 0.0;
-#pragma unroll
-    for (int a = 0; a < 8; a++) {
-        const int r = min(max(r0 + a, 0), h - 1);
-        const int32_t* x = X + (int64_t)r * nout + c0;
-        double row = 0.0;
-#pragma unroll
-        for (int b = 0; b < 8; b++) row += wc[b] * (double)__ldg(x + min(max(k0 + b, 0), w - 1));
-        U += wr[a] * row;
-    }
-    return U;
-}
-
 __global__ void k_grid_init(long long* work, int S)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -111,75 +271,104 @@ __global__ void k_grid_init(long long* work, int S)
     }
 }
 
-// Block (slice s0 + blockIdx.x / M, row i = blockIdx.x % M).  PASS 0: min/max
-// into work; PASS 1: write Y.
-template <bool AREA, int PASS>
-__global__ void __launch_bounds__(kGT) k_grid(const int32_t* __restrict__ X, int h, int64_t nout, int64_t ns, int s0,
-                                              int M, long long* __restrict__ work, uint8_t* __restrict__ out)
+// Lanczos path.  Block = (slice, ti output rows, kLJ output columns).  Both axes'
+// taps are computed once per block into shared memory (fp64 sines and
+// divisions: on this chip the dearest part), then the horizontal sums H[r][j] of
+// the plane rows the block needs, then each pixel's vertical sum over 8 of them;
+// the products and sums in the order of the definition.  fp64-bound: 4 slices of
+// 169 x 3407 to 512 x 512 took 2.0 ms a pass with 12 taps per pixel, a twentieth so.
+constexpr int kLJ = 64, kLI = 64, kLR = 192;  // columns, most rows of output, most plane rows
+constexpr size_t kLSmem = ((size_t)kLR * kLJ + 8 * (kLI + kLJ)) * sizeof(double) + (kLI + kLJ) * sizeof(int);
+template <int PASS>
+__global__ void __launch_bounds__(kGT)
+k_grid_lanczos(const int32_t* __restrict__ X, int h, int64_t nout, int64_t ns, int s0, int M, int ti, unsigned iruns,
+               unsigned jruns, long long* __restrict__ work, uint8_t* __restrict__ out)
 {
-    __shared__ long long slo[kGT / 32], shi[kGT / 32];
-    const int s = s0 + (int)(blockIdx.x / M), i = (int)(blockIdx.x % M);
+    extern __shared__ double sm[];
+    double* H = sm;                      // [kLR][kLJ]
+    double* wr = H + kLR * kLJ;          // [kLI][8]
+    double* wc = wr + 8 * kLI;           // [kLJ][8]
+    int* r0 = (int*)(wc + 8 * kLJ);      // [kLI]
+    int* q0 = r0 + kLI;                  // [kLJ]
+    const unsigned blk = PASS == 0 ? blockIdx.x : gridDim.x - 1 - blockIdx.x;
+    const int j0 = (int)(blk % jruns) * kLJ, i0 = (int)(blk / jruns % iruns) * ti;
+    const int s = s0 + (int)(blk / jruns / iruns);
     const int64_t c0 = (int64_t)s * ns;
     const int w = (int)min(ns, nout - c0);
-    double wr[8];
-    int r0 = 0;
-    if (!AREA) r0 = lanczos_taps(i, h, M, wr);
-    if (PASS == 0) {
-        long long lo = LLONG_MAX, hi = LLONG_MIN;
-        for (int j = threadIdx.x; j < M; j += kGT) {
-            const long long k = AREA ? area_value(X, nout, h, c0, w, M, i, j)
-                                     : dkey(lanczos_value(X, nout, h, c0, w, M, wr, r0, j));
-            lo = min(lo, k);
-            hi = max(hi, k);
-        }
+    const int ni = min(ti, M - i0), nj = min(kLJ, M - j0);
+    for (int e = (int)threadIdx.x; e < ni + nj; e += kGT) {
+        double t[8];
+        const bool row = e < ni;
+        const int k = row ? lanczos_taps(i0 + e, h, M, t) : lanczos_taps(j0 + e - ni, w, M, t);
+        double* to = row ? wr + 8 * e : wc + 8 * (e - ni);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        for (int a = 0; a < 8; a++) to[a] = t[a];
+        if (row) r0[e] = k;
+        else q0[e - ni] = k;
+    }
+    __syncthreads();
+    const int jj = (int)threadIdx.x % kLJ, g = (int)threadIdx.x / kLJ;
+    const int rb = r0[0], nr = r0[ni - 1] + 8 - rb;  // plane rows rb .. rb + nr - 1 (clamped to the plane)
+    if (jj < nj) {
+        double t[8];
+        int q[8];
+#pragma unroll
+        for (int b = 0; b < 8; b++) {
+            t[b] = wc[8 * jj + b];
+            q[b] = min(max(q0[jj] + b, 0), w - 1);
         }
-        if ((threadIdx.x & 31) == 0) {
-            slo[threadIdx.x >> 5] = lo;
-            shi[threadIdx.x >> 5] = hi;
+        for (int r = g; r < nr; r += kGT / kLJ) {
+            const int32_t* x = X + (int64_t)min(max(rb + r, 0), h - 1) * nout + c0;
+            double row = 0.0;
+#pragma unroll
+            for (int b = 0; b < 8; b++) row = fma(t[b], (double)__ldg(x + q[b]), row);
+            H[r * kLJ + jj] = row;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int k = 1; k < kGT / 32; k++) {
-                lo = min(lo, slo[k]);
-                hi = max(hi, shi[k]);
+    }
+    __syncthreads();
+    long long lo = LLONG_MAX, hi = LLONG_MIN;
+    const double ulo = PASS == 1 ? dval(work[2 * s]) : 0.0, uhi = PASS == 1 ? dval(work[2 * s + 1]) : 0.0;
+    if (jj < nj)
+        for (int i = g; i < ni; i += kGT / kLJ) {
+            const double* Hr = H + (r0[i] - rb) * kLJ + jj;
+            double U = 0.0;
+#pragma unroll
+            for (int a = 0; a < 8; a++) U = fma(wr[8 * i + a], Hr[a * kLJ], U);
+            if (PASS == 0) {
+                lo = min(lo, dkey(U));
+                hi = max(hi, dkey(U));
+            } else {
+                out[((int64_t)s * M + i0 + i) * M + j0 + jj] =
+                    (uint8_t)floor(255.0 * (U - ulo) / (uhi - ulo + 1e-6) + 0.5);
             }
-            lo = min(lo, slo[0]);
-            hi = max(hi, shi[0]);
-            atomicMin(work + 2 * s, lo);
-            atomicMax(work + 2 * s + 1, hi);
         }
-        return;
-    }
-    uint8_t* o = out + ((int64_t)s * M + i) * M;
-    if (AREA) {
-        const long long lo = work[2 * s], hi = work[2 * s + 1];
-        const unsigned long long rng = (unsigned long long)(hi - lo);
-        for (int j = threadIdx.x; j < M; j += kGT) {
-            const long long W = area_value(X, nout, h, c0, w, M, i, j);
-            o[j] = rng == 0 ? (uint8_t)0
-                            : (uint8_t)((510 * (unsigned __int128)(W - lo) + rng) / (2 * (unsigned __int128)rng));
-        }
-    } else {
-        const double lo = dval(work[2 * s]), hi = dval(work[2 * s + 1]);
-        for (int j = threadIdx.x; j < M; j += kGT) {
-            const double U = lanczos_value(X, nout, h, c0, w, M, wr, r0, j);
-            o[j] = (uint8_t)floor(255.0 * (U - lo) / (hi - lo + 1e-6) + 0.5);
-        }
-    }
+    if (PASS == 0) slice_minmax(lo, hi, work + 2 * s);
 }
 
-template <int PASS>
-void launch_pass(bool area, unsigned blocks, cudaStream_t st, const int32_t* X, int h, int64_t nout, int64_t ns,
-                 int s0, int M, long long* work, uint8_t* out)
+// One pass over slices s0 .. s0 + n - 1, all on one path.
+int launch_pass(int pass, bool area, int n, cudaStream_t st, const int32_t* X, int h, int64_t nout, int64_t ns, int s0,
+                int M, long long* work, uint8_t* out)
 {
-    if (area)
-        k_grid<true, PASS><<<blocks, kGT, 0, st>>>(X, h, nout, ns, s0, M, work, out);
-    else
-        k_grid<false, PASS><<<blocks, kGT, 0, st>>>(X, h, nout, ns, s0, M, work, out);
+    if (area) {
+        const int64_t w = ns < nout - (int64_t)s0 * ns ? ns : nout - (int64_t)s0 * ns;
+        const unsigned runs = (unsigned)((M + kGT - 1) / kGT);
+        const int64_t span = (std::min(M, kGT) * w + M - 1) / M + 1;  // columns of a block's run
+        const int cols = (int)std::max<int64_t>(2, (std::min<int64_t>(span, kGCBytes / 4) + 1) & ~1);
+        const size_t smem = (size_t)cols * 4;
+        const unsigned blocks = (unsigned)n * (unsigned)M * runs;
+        if (pass == 0) k_grid_area<0><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s0, M, runs, cols, work, out);
+        else k_grid_area<1><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s0, M, runs, cols, work, out);
+        return af_cuda_check(cudaGetLastError(), "af_grid launch");
+    }
+    // rows per block: as many as their plane rows fit (one row needs 8)
+    const int ti = (int)std::max<int64_t>(1, std::min<int64_t>(kLI, (int64_t)(kLR - 9) * M / h));
+    const unsigned iruns = (unsigned)((M + ti - 1) / ti), jruns = (unsigned)((M + kLJ - 1) / kLJ);
+    const unsigned blocks = (unsigned)n * iruns * jruns;
+    const void* fn = pass == 0 ? (const void*)k_grid_lanczos<0> : (const void*)k_grid_lanczos<1>;
+    if (int rc = af_ensure_smem(fn, kLSmem)) return rc;
+    if (pass == 0) k_grid_lanczos<0><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s0, M, ti, iruns, jruns, work, out);
+    else k_grid_lanczos<1><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s0, M, ti, iruns, jruns, work, out);
+    return af_cuda_check(cudaGetLastError(), "af_grid launch");
 }
 
 }  // namespace
@@ -207,19 +396,12 @@ try {
     const bool area_full = ndm > M && ns > M;
     const bool area_last = ndm > M && last_w > M;
     for (int pass = 0; pass < 2; pass++) {
-        if (nfull > 0) {
-            if (pass == 0)
-                launch_pass<0>(area_full, (unsigned)(nfull * M), st, d_plane, ndm, nout, ns, 0, M, work, d_out);
-            else
-                launch_pass<1>(area_full, (unsigned)(nfull * M), st, d_plane, ndm, nout, ns, 0, M, work, d_out);
-        }
-        if (last_w > 0) {
-            if (pass == 0)
-                launch_pass<0>(area_last, (unsigned)M, st, d_plane, ndm, nout, ns, (int)nfull, M, work, d_out);
-            else
-                launch_pass<1>(area_last, (unsigned)M, st, d_plane, ndm, nout, ns, (int)nfull, M, work, d_out);
-        }
-        if (int rc = af_cuda_check(cudaGetLastError(), "af_grid launch")) return rc;
+        const bool one = nfull > 0 && last_w > 0 && area_full == area_last;  // every slice in one launch
+        if (nfull > 0)
+            if (int rc = launch_pass(pass, area_full, (int)(one ? S : nfull), st, d_plane, ndm, nout, ns, 0, M, work, d_out))
+                return rc;
+        if (last_w > 0 && !one)
+            if (int rc = launch_pass(pass, area_last, 1, st, d_plane, ndm, nout, ns, (int)nfull, M, work, d_out)) return rc;
     }
     return AF_OK;
 } catch (...) {
