@@ -45,8 +45,8 @@ struct Layer {
 
 // Inference batches of at least this many images run the layered tensor-core
 // network; smaller ones the fused one-kernel network (AFGB_CNN_UMMA_MIN
-// overrides at model creation).  Measured on GB300, fused / layered: 0.040 /
-// 0.058 ms at 128 images, 0.074 / 0.070 ms at 256, 0.141 / 0.087 ms at 512.
+// overrides at model creation).  Measured on GB300, fused / layered: 0.025 /
+// 0.041 ms at 152 images, 0.044 / 0.045 ms at 255, 0.076 / 0.064 ms at 512.
 constexpr int kUmmaInferMin = 256;
 
 }  // namespace
@@ -262,12 +262,15 @@ try {
     return af_host_exception("af_model_get_grads");
 }
 
-static int forward(af_model_t m, const __nv_bfloat16* x, int n, const int32_t* y, float* prob, cudaStream_t s)
+// logits: the caller's [n][2], or NULL.
+static int forward(af_model_t m, const __nv_bfloat16* x, int n, const int32_t* y, float* logits, float* prob,
+                   cudaStream_t s)
 {
     const float* P = m->d_params;
+    if (!logits) logits = m->d_logits;
     if (!y && n < m->umma_min)  // small inference batch: one fused kernel
         return nn_forward_fused(x, n, P + m->L[0].woff, P + m->L[0].boff, P + m->L[1].woff, P + m->L[1].boff,
-                                P + m->L[2].woff, P + m->L[2].boff, P + m->fw_off, P + m->fb_off, m->d_logits, prob,
+                                P + m->L[2].woff, P + m->L[2].boff, P + m->fw_off, P + m->fb_off, logits, prob,
                                 s);
     if (!m->packed) {  // the parameters changed since the last packing
         for (int l = 0; l < NL; l++)
@@ -290,7 +293,7 @@ static int forward(af_model_t m, const __nv_bfloat16* x, int n, const int32_t* y
         AF_CUDA(cudaMemsetAsync(m->d_loss, 0, 4, s));
         AF_CUDA(cudaMemsetAsync(m->d_grads, 0, m->nparams * 4, s));
     }
-    return nn_head(m->d_a[NL], n, P + m->fw_off, P + m->fb_off, m->d_logits, prob, y, m->d_loss,
+    return nn_head(m->d_a[NL], n, P + m->fw_off, P + m->fb_off, logits, prob, y, m->d_loss,
                    m->d_grads + m->fw_off, m->d_grads + m->fb_off, m->d_da[NL], s);
 }
 
@@ -328,9 +331,7 @@ extern "C" int af_model_forward(af_model_t m, const uint16_t* d_x, int32_t n, fl
 try {
     if (int rc = check_batch(m, d_x, n)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    if (int rc = forward(m, (const __nv_bfloat16*)d_x, n, nullptr, d_prob, s)) return rc;
-    if (d_logits) AF_CUDA(cudaMemcpyAsync(d_logits, m->d_logits, (size_t)n * 8, cudaMemcpyDeviceToDevice, s));
-    return AF_OK;
+    return forward(m, (const __nv_bfloat16*)d_x, n, nullptr, d_logits, d_prob, s);
 } catch (...) {
     return af_host_exception("af_model_forward");
 }
@@ -341,7 +342,7 @@ try {
     if (int rc = check_batch(m, d_x, n)) return rc;
     if (!d_y) return af_set_error(AF_EINVAL, "af_model_backward: labels NULL");
     cudaStream_t s = (cudaStream_t)stream;
-    if (int rc = forward(m, (const __nv_bfloat16*)d_x, n, d_y, nullptr, s)) return rc;
+    if (int rc = forward(m, (const __nv_bfloat16*)d_x, n, d_y, nullptr, nullptr, s)) return rc;
     if (int rc = backward(m, (const __nv_bfloat16*)d_x, n, s)) return rc;
     if (d_loss) AF_CUDA(cudaMemcpyAsync(d_loss, m->d_loss, 4, cudaMemcpyDeviceToDevice, s));
     return AF_OK;
@@ -408,7 +409,7 @@ try {
         const int32_t k = std::min(m->max_batch, n - i0);
         if (int rc = af_cutouts(p, d_in, nsamp, d_plane, nout, d_cands + i0, k, (uint16_t*)m->d_cut, stream))
             return rc;
-        if (int rc = forward(m, m->d_cut, k, nullptr, d_prob + i0, s)) return rc;
+        if (int rc = forward(m, m->d_cut, k, nullptr, nullptr, d_prob + i0, s)) return rc;
     }
     return AF_OK;
 } catch (...) {
