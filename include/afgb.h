@@ -139,7 +139,8 @@ int af_plan_info(af_plan_t plan, int* nchan, int* ndm, int32_t* dmax, double* ts
  * AFGB_DEDISP_KERNEL=tile|simple|pairs in the environment at plan creation
  * forces the channel tile kernel, the simple kernel, or group rows wherever
  * they apply (without the cost comparison); AFGB_PAIR_GROUP=2|3|4 fixes the
- * group size.  Read-only; no device work.  Not a step of the paper's method. */
+ * group size and AFGB_PAIR_DPW=1|2 the DM rows per consumer warp (blocks of 15
+ * or 30 DM rows).  Read-only; no device work.  Not a step of the paper's method. */
 #define AF_PATH_SIMPLE 0
 #define AF_PATH_TILE 1
 #define AF_PATH_SUBBAND 2

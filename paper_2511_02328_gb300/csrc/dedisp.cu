@@ -298,7 +298,7 @@ try {
     } else if (af_dedisp_uses_pairs(p, 1)) {
         pa = AF_PATH_PAIRS;
         rg = af_pair_ring_depth(p->pairs.shape);
-        sp = p->pairs.tt.spread;
+        sp = p->pairs.spread;
         gr = p->pairs.G;
     } else if (p->tile.ns1 > 0 && !p->force_simple) {
         pa = AF_PATH_TILE;

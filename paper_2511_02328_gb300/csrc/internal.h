@@ -84,12 +84,13 @@ struct af_pair_args {
     const uint16_t* PS;      // rows of the time block
     const int2* chunks;      // per chunk: {row slots, first slot}
     const int32_t* chkoff;   // [nblk + 1] first chunk of each block
-    const int* tabs;         // per chunk: NW x TABW ints, every consumer warp's table for its ring stage
+    const uint16_t* tabs;    // per chunk: DM rows x TABW, every DM row's table of offsets inside a ring stage
     const int2* srec;        // per slot: {window bytes, byte offset inside its stage}
     const int64_t* soff;     // per slot: element offset of its window in PS for the block's first tile
     const int32_t* perm;     // [ndm_pad] plane row, -1 = padding
     int stage_bytes;         // bytes of one ring stage's windows
     int flush;               // rows between folds: flush * 255 * G < 2^16
+    int dpw;                 // DM rows per consumer warp (1 or 2)
     unsigned nblk;
     int64_t T0;              // first output of the time block (a multiple of 8)
     int64_t tend;            // outputs t < tend are written
@@ -104,19 +105,26 @@ struct af_pair_args {
 struct af_pair_tables {
     bool ok = false;               // the plan can use this path
     int G = 2;                     // channels per group (2, 3 or 4)
+    int dpw = 1;                   // DM rows per consumer warp: blocks of 15 or 30 DM rows
     int np = 0, nrows = 0, rwe = 0, maxdr = 0;   // np = groups
     double rows_per_pair = 0;      // rows copied per pair and DM block (mean)
     size_t budget = 0;             // bytes the row buffer may take (AFGB_PAIR_BUDGET_MB at plan creation)
     int shape = 0;                 // ring depth of the row kernel (2 to 4 stages)
     int stage_bytes = 0;           // bytes of one ring stage (windows packed back to back)
-    af_tile_tables tt;             // DM order and block minima for this block shape
+    int nblk = 0, ndm_pad = 0;     // DM blocks, their rows
+    int32_t spread = 0;            // largest delay difference between DMs of one block
     double copy_per_tile = 0;      // bytes of row windows copied per time tile (all DM blocks)
     std::vector<int32_t> h_rb, h_ub, h_rB, h_rspan, h_srow, h_scpart;
+    // until uploaded (when a reservation or a batch first uses the set)
+    std::vector<int32_t> h_rdelta, h_chkoff, h_perm;
+    std::vector<int2> h_gdr, h_chunks, h_srec;
+    std::vector<uint16_t> h_tabs;
+    int32_t* d_perm = nullptr;     // [ndm_pad] plane row of each DM of the blocks, -1 = padding
     int32_t* d_rdelta = nullptr;   // [nrows][G-1] relative delays of each row
     int2* d_gdr = nullptr;         // [groups][G-1] smallest and largest relative delay
     int2* d_chunks = nullptr;      // per chunk: row slots, first slot
     int32_t* d_chkoff = nullptr;   // [nblk + 1]
-    int* d_tabs = nullptr;         // per chunk: every consumer warp's table
+    uint16_t* d_tabs = nullptr;    // per chunk: every DM row's table
     int2* d_srec = nullptr;        // per slot: window bytes, byte offset inside its ring stage
     uint16_t* d_ps = nullptr;      // row buffer
     size_t ps_bytes = 0;
@@ -127,8 +135,7 @@ struct af_pair_tables {
     struct Layout {
         int64_t L = 0, maxlen = 0;     // outputs per time block, longest row
         int4* d_pinfo = nullptr;       // [np] first row, rows, range start ub, range length
-        int2* d_rinfo = nullptr;       // [nrows] row start - ub, row length (rows of a group by start)
-        int* d_gmax = nullptr;         // [np] longest row of each group
+        int4* d_rinfo = nullptr;       // [nrows] row start - ub, row length, largest end so far, smallest start from here
         int64_t* d_rowoff = nullptr;   // [nrows] element offset in the row buffer
         int64_t* d_soff = nullptr;     // per slot: window offset for a time block's first tile
     } lay[2];
@@ -206,7 +213,7 @@ struct af_plan_s {
                                            // comparison (AFGB_DEDISP_KERNEL=pairs)
     int force_group = 0;                   // 2, 3 or 4: only that group size (AFGB_PAIR_GROUP)
     af_pair_tables pairs;                  // group-row path of brute-force plans (the one in use)
-    af_pair_tables alt[2];                 // the other group sizes (3, 4), until a reservation picks
+    af_pair_tables alt[5];                 // the other group sizes and block heights, until a reservation picks
 
     // two-stage subband dedispersion (sb_nsub > 0); `delays` then holds the
     // effective table D[j(m)][c] + R[m][s(c)]

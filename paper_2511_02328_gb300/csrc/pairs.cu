@@ -17,37 +17,52 @@
 // that use it (element e is time T0 + B_g + e, B_g their smallest delay
 // rounded down to 16).
 //
-// Stage 2 (k_pair_tile) is a tile kernel over rows: a block takes NW DM rows
-// (one consumer warp each, DMs ascending) and TTE = 1016 outputs; a producer
-// warp streams the block's row windows (one per block and row) through an
-// NS-deep shared-memory ring, up to 32 windows of whole groups packed back to
-// back per stage, one bulk async copy per window plus one for the chunk's
-// consumer tables of (window, offset) per group, which the host computes once
-// (tiles start at multiples of 8, so no offset depends on the tile).  Lane L
-// of a consumer warp owns outputs 2 (L + 32 m) + k, m < 16, k < 2: one
-// aligned 32-bit shared load brings the two 16-bit samples of a group, so the
-// groups are bucketed by the parity r of the sample offset; one IADD3 adds two
+// Stage 2 (k_pair_tile) is a tile kernel over rows: a block takes 15 or 30 DM
+// rows (15 consumer warps with one or two DMs each, DMs ascending) and TTE = 1016
+// outputs; a producer warp streams the block's row windows (one per block and
+// row) through an NS-deep shared-memory ring, up to 32 windows of whole groups
+// packed back to back per stage, one bulk async copy per window plus one for the
+// chunk's consumer tables of (window, offset) per group, which the host computes
+// once (tiles start at multiples of 8, so no offset depends on the tile).  Lane L
+// of a consumer warp owns outputs 2 (L + 32 m) + k, m < 16, k < 2, of each of its
+// DMs: one aligned 32-bit shared load brings the two 16-bit samples of a group, so
+// the groups are bucketed by the parity r of the sample offset; one IADD3 adds two
 // rows' words into the 16-bit lanes of the bucket's accumulator (at most
-// 65535 / (255 G) rows between folds); a fold re-aligns bucket 1 by one
-// sample (one lane shuffle) into the 32-bit output sums.
+// 65535 / (255 G) rows between folds); a fold re-aligns bucket 1 by one sample (one
+// lane shuffle) into the 32-bit output sums.
+//
+// What bounds stage 2: the consumers' shared loads (2 bytes per DM, group and
+// output) and the window copies from L2 (7.6 TB/s on GB300), which take as long
+// as each other with 15 DM rows per block (4096 channels, 1001 DMs, 215,261
+// outputs, groups of 3: 17.0 ms each alone, 19.2 ms together).  A block of 30 rows
+// copies 0.68 of the bytes per output, since neighbouring DMs share rows; its
+// bucket accumulators fill the registers that 15 rows' accumulators and 32-bit
+// sums took, and the 32-bit sums, touched once per fold, live in tensor memory
+// (which no other part of this kernel uses): 17.2 ms with groups of 3, and groups
+// of 4, whose loads take 13.2 ms alone, 18.8 -> 14.3 ms.
 //
 // Every wait is bounded (the tile kernel's error flag).  The host tables of
-// every group size are built once per plan; a reservation picks the group size
-// by a cost model and sizes the row buffer from a budget.
+// every group size and block height are built once per plan; a reservation picks
+// one by a cost model, uploads it and sizes the row buffer from a budget.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdlib.h>
 
 #include <algorithm>
 #include <array>
+#include <cmath>
+#include <future>
+#include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
 #include "ptx.cuh"
+#include "umma.cuh"
 
 namespace {
 
-constexpr int kPNW = 15;            // DM rows (consumer warps) per block
+constexpr int kPNW = 15;            // consumer warps per block, each with 1 or 2 DM rows (DPW)
 // Ring: up to kPSL row windows per stage (one per producer lane), packed back
 // to back (a stage holds as many whole groups as fit its bytes); the depth is
 // 2, 3 or 4 stages (AFGB_PAIR_STAGES at plan creation, default 3: on the
@@ -55,7 +70,8 @@ constexpr int kPNW = 15;            // DM rows (consumer warps) per block
 constexpr int kPSL = 32;
 constexpr int kPMG = 16;            // 2-sample groups per lane
 constexpr int kPTTE = 1016;         // outputs per tile: a multiple of 8 below 64 * kPMG - 1
-constexpr int kPTABW = 40;          // ints per (stage, warp) table: 2 starts, 2 counts, <= 34 offsets
+constexpr int kPTABW = 40;          // uint16 per (stage, DM row) table: 2 starts, 2 counts, <= 34 offsets / 4
+constexpr int kPTM = 256;           // tensor-memory columns of a block (DPW = 2)
 constexpr uint32_t kPWait = afptx::kMbarWaitPolls;
 constexpr int kET = 4096;           // stage 1: row samples per block
 constexpr int kS1T = 256;
@@ -72,7 +88,8 @@ typedef af_pair_args PairArgs;
 // for every row of the group, the part of those samples inside the row's own
 // range.  pinfo[q] = {first row, rows, ub (the group's first delay rounded down
 // to 16), length of the group's range}; rinfo[g] = {row start - ub (a multiple
-// of 16), row length}; rdelta[g][i-1] = row g's delay of channel Gq+i relative
+// of 16), row length, the largest end of the group's rows up to g, the smallest
+// start of its rows from g on}; rdelta[g][i-1] = row g's delay of channel Gq+i relative
 // to channel Gq; gdr[q][i-1] = the smallest and largest of those over the
 // group's rows.  Channel Gq's window goes to W0, channel Gq+i's (shifted by
 // the smallest delta, longer by the delta range + 4 bytes) to Wi: blocks whose
@@ -80,11 +97,19 @@ typedef af_pair_args PairArgs;
 // window then starts off_i bytes into its buffer), edge blocks byte by byte
 // with zeros outside the rows and for missing channels.  Words at any byte
 // offset are read with a funnel shift (one shift per block and row).
+// A group's rows come in lexicographic order of their tuples, so that a row
+// mostly shares its first delays with the one before: the sums over those
+// channels stay in registers and only the channels from the first difference on
+// are read and widened again (1.36 of 2 per row for groups of 3, 1.61 of 3 for
+// groups of 4 on the 4096-channel workload).  Bound by HBM (groups of 4: 36.9 GB in
+// 5.58 ms, 0.97 of its measured rate; every channel read again for every row: 6.64
+// ms, 15 ALU instructions per 4 samples and row) or, where rows are few or short,
+// by issue.
 template <int G>
-__global__ void __launch_bounds__(kS1T)
+__global__ void __launch_bounds__(kS1T, G == 4 ? 1 : G == 3 ? 5 : 6)
 k_group_rows(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int4* __restrict__ pinfo,
-             const int* __restrict__ gmax, const int2* __restrict__ gdr, const int32_t* __restrict__ rdelta,
-             const int2* __restrict__ rinfo, const int64_t* __restrict__ rowoff, int64_t T0, int etiles, int wstride,
+             const int2* __restrict__ gdr, const int32_t* __restrict__ rdelta,
+             const int4* __restrict__ rinfo, const int64_t* __restrict__ rowoff, int64_t T0, int etiles, int wstride,
              int dshort, uint16_t* __restrict__ PS)
 {
     constexpr int K = G - 1;
@@ -96,23 +121,22 @@ k_group_rows(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int4
     // a time block dshort outputs shorter than the layout's needs every row
     // (and the group's range) dshort samples shorter (dshort a multiple of 16)
     if (e0 >= pi.w - dshort) return;
-    // the rows overlapping [e0, e0 + ET): rows are ordered by start, so they are
-    // those from the first starting after e0 - (longest row) to the first
-    // starting at or after e0 + ET (each still checked below)
+    // the rows overlapping [e0, e0 + ET) lie between the first whose running largest
+    // end passes e0 and the first from which on all start at e0 + ET or later (each
+    // is still checked below)
     int kbeg, kend;
     {
-        const int lo_start = (int)(e0 - __ldg(gmax + q)), hi_start = (int)(e0 + kET);
         int a = 0, b = pi.y;
         while (a < b) {
             const int m = (a + b) >> 1;
-            if (__ldg(rinfo + pi.x + m).x <= lo_start) a = m + 1;
+            if (__ldg(&rinfo[pi.x + m].z) - dshort <= e0) a = m + 1;
             else b = m;
         }
         kbeg = a;
         b = pi.y;
         while (a < b) {
             const int m = (a + b) >> 1;
-            if (__ldg(rinfo + pi.x + m).x < hi_start) a = m + 1;
+            if (__ldg(&rinfo[pi.x + m].w) < e0 + kET) a = m + 1;
             else b = m;
         }
         kend = a;
@@ -166,7 +190,8 @@ k_group_rows(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int4
     // thread tid takes the 4-sample words w = tid + 256 j (j < 4) of the block:
     // consecutive lanes read consecutive shared words (no bank conflicts) and
     // store consecutive 8-byte pieces of a row
-    uint32_t alo[4], ahi[4];
+    // sums over the group's first i + 1 channels at the current delays, two 16-bit lanes a word
+    uint32_t lo[K][4], hi[K][4];
     bool live[4];
     {
         const uint32_t* A32 = reinterpret_cast<const uint32_t*>(sm);
@@ -177,44 +202,78 @@ k_group_rows(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int4
             live[j] = e0 + 4 * w < pi.w - dshort;
             const int p = (off[0] >> 2) + w;
             const uint32_t a = __funnelshift_r(A32[p], A32[p + 1], sh);
-            alo[j] = __byte_perm(a, 0u, 0x4140);  // samples 0, 1 into 16-bit lanes
-            ahi[j] = __byte_perm(a, 0u, 0x4342);  // samples 2, 3
+            lo[0][j] = __byte_perm(a, 0u, 0x4140);  // samples 0, 1 into 16-bit lanes
+            hi[0][j] = __byte_perm(a, 0u, 0x4342);  // samples 2, 3
         }
     }
-    for (int k = kbeg; k < kend; k++) {
-        const int2 ri = __ldg(rinfo + pi.x + k);
-        uint32_t lo[4], hi[4];
+    int prev[K];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            lo[j] = alo[j];
-            hi[j] = ahi[j];
+    for (int i = 0; i < K; i++) prev[i] = INT32_MIN;
+    // a row's record is read while the row before it is summed (groups of 2 have too
+    // little to sum for that: there the loads of several rows overlap as they are)
+    constexpr bool AHEAD = G > 2;
+    int4 ri = __ldg(rinfo + pi.x + kbeg);
+    int64_t ro = __ldg(rowoff + pi.x + kbeg);
+    int dl[K];
+#pragma unroll
+    for (int i = 0; i < K; i++) dl[i] = __ldg(rdelta + (int64_t)(pi.x + kbeg) * K + i);
+    for (int k = kbeg; k < kend; k++) {
+        if (!AHEAD) {
+            const int2 r2 = __ldg(reinterpret_cast<const int2*>(rinfo + pi.x + k));
+            ri.x = r2.x;
+            ri.y = r2.y;
+            ro = __ldg(rowoff + pi.x + k);
+            dl[0] = __ldg(rdelta + pi.x + k);
         }
+        const int start = ri.x, len = ri.y - dshort;
+        uint16_t* row = PS + ro;
+        int d[K];
+#pragma unroll
+        for (int i = 0; i < K; i++) d[i] = dl[i];
+        if (AHEAD && k + 1 < kend) {
+            ri = __ldg(rinfo + pi.x + k + 1);
+            ro = __ldg(rowoff + pi.x + k + 1);
+#pragma unroll
+            for (int i = 0; i < K; i++) dl[i] = __ldg(rdelta + (int64_t)(pi.x + k + 1) * K + i);
+        }
+        if (AHEAD && (start >= e0 + kET || start + len <= e0)) continue;
+        bool change = false;  // a delay so far differs from the last summed row's (the same in every thread)
+        uint32_t l[4], h[4];
 #pragma unroll
         for (int i = 0; i < K; i++) {
+            change = change || d[i] != prev[i];
+            prev[i] = d[i];
+            if (!change && i < K - 1) continue;
             const uint32_t* W32 = reinterpret_cast<const uint32_t*>(sm + kET + 48 + i * wstride);
-            const int pb = off[i + 1] + __ldg(rdelta + (int64_t)(pi.x + k) * K + i) - dmn[i];
+            const int pb = off[i + 1] + d[i] - dmn[i];
             const uint32_t sh = (uint32_t)(pb & 3) * 8u;
 #pragma unroll
             for (int j = 0; j < 4; j++) {
                 const int p = (pb >> 2) + tid + kS1T * j;
                 const uint32_t b = __funnelshift_r(W32[p], W32[p + 1], sh);
-                lo[j] += __byte_perm(b, 0u, 0x4140);
-                hi[j] += __byte_perm(b, 0u, 0x4342);
+                l[j] = lo[i][j] + __byte_perm(b, 0u, 0x4140);
+                h[j] = hi[i][j] + __byte_perm(b, 0u, 0x4342);
+                if (i < K - 1) {
+                    lo[i + 1 < K ? i + 1 : 0][j] = l[j];
+                    hi[i + 1 < K ? i + 1 : 0][j] = h[j];
+                }
             }
         }
-        uint16_t* row = PS + __ldg(rowoff + pi.x + k);
 #pragma unroll
         for (int j = 0; j < 4; j++) {
-            const int64_t rel = e0 + 4 * (tid + kS1T * j) - ri.x;  // sample index within the row
-            if (live[j] && rel >= 0 && rel < ri.y - dshort)
-                *reinterpret_cast<uint2*>(row + rel) = make_uint2(lo[j], hi[j]);
+            const int rel = (int)e0 + 4 * (tid + kS1T * j) - start;  // sample index within the row
+            if (live[j] && (uint32_t)rel < (uint32_t)len)
+                *reinterpret_cast<uint2*>(row + rel) = make_uint2(l[j], h[j]);
         }
     }
 }
 
 // ------------------------------------------------------------------ stage 2
-template <int NW, int NS>
+template <int NS, int DPW>
 struct PairTile {
+    static constexpr int NW = kPNW, ND = NW * DPW;      // consumer warps, DM rows of a block
+    static constexpr uint32_t TB = ND * kPTABW * 2;     // table bytes of a chunk
+
     static __device__ __forceinline__ int2 load_cd(const PairArgs& a, int cbeg, int nchk, int kk)
     {
         return kk < nchk ? __ldg(a.chunks + cbeg + kk) : make_int2(0, 0);
@@ -222,18 +281,16 @@ struct PairTile {
 
     // Chunk c (block-local kk) into stage st: its precomputed table block and
     // one window per row slot, all completing on the stage's full barrier.
-    static __device__ __forceinline__ void produce(const PairArgs& a, uint8_t* smem, int* tab, uint32_t full_bar,
+    static __device__ __forceinline__ void produce(const PairArgs& a, uint8_t* smem, uint16_t* tab, uint32_t full_bar,
                                                    int c, const int2& cd, uint32_t bytes, uint32_t soff,
                                                    int64_t src, int st, int lane)
     {
-        constexpr uint32_t TB = (uint32_t)(NW * kPTABW * 4);
         const uint32_t tot = __reduce_add_sync(0xffffffffu, bytes) + TB;
         __syncwarp();
         afptx::fence_proxy_async();  // the consumers' reads of this stage come before the copies
         if (lane == 0) {
             afptx::mbar_arrive_expect_tx(full_bar, tot);
-            afptx::bulk_g2s(afptx::smem_addr(tab + st * NW * kPTABW), a.tabs + (int64_t)c * NW * kPTABW, TB,
-                            full_bar);
+            afptx::bulk_g2s(afptx::smem_addr(tab + st * ND * kPTABW), a.tabs + (int64_t)c * ND * kPTABW, TB, full_bar);
         }
         __syncwarp();
         if (lane < cd.x && bytes)
@@ -241,33 +298,87 @@ struct PairTile {
                             full_bar);
     }
 
-    // Bucket 1 holds, in lane L group m, samples 2 (L + 32 m) + 1 and + 2: output
-    // k = 0 takes its own upper half, k = 1 the lower half of the next lane's word
-    // (lane 0 of group m + 1 for L = 31).
-    static __device__ __forceinline__ void fold(uint32_t (&A)[2][kPMG], uint32_t (&Wd)[kPMG][2], int lane)
+    // Adds half h (groups 8 h .. 8 h + 7) of the bucket accumulators into the
+    // 32-bit sums w[2 (m - 8 h) + k] and clears them.  Bucket 1 holds, in lane L
+    // group m, samples 2 (L + 32 m) + 1 and + 2: output k = 0 takes its own upper
+    // half, k = 1 the lower half of the next lane's word (lane 0 of group m + 1 for
+    // L = 31).  Halves in descending order: `carry` runs through both.
+    static __device__ __forceinline__ void fold_half(uint32_t (&A)[2][kPMG], int h, uint32_t (&w)[kPMG], uint32_t& carry,
+                                                     int lane)
     {
-        uint32_t carry = 0u;
 #pragma unroll
-        for (int m = kPMG - 1; m >= 0; m--) {
+        for (int i = 7; i >= 0; i--) {
+            const int m = 8 * h + i;
             const uint32_t a0 = A[0][m], a1 = A[1][m];
             const uint32_t lo1 = a1 & 0xFFFFu;
             uint32_t nx = __shfl_down_sync(0xffffffffu, lo1, 1);
             const uint32_t l0 = __shfl_sync(0xffffffffu, lo1, 0);
             if (lane == 31) nx = carry;
             carry = l0;
-            Wd[m][0] += (a0 & 0xFFFFu) + (a1 >> 16);
-            Wd[m][1] += (a0 >> 16) + nx;
+            w[2 * i] += (a0 & 0xFFFFu) + (a1 >> 16);
+            w[2 * i + 1] += (a0 >> 16) + nx;
             A[0][m] = 0u;
             A[1][m] = 0u;
         }
     }
 
+    // The 32-bit sums of a warp's DM rows: registers (one row), or tensor memory
+    // (two rows: lanes 32 (warp % 4) .., 32 columns per row), read, added to and
+    // written back 16 columns at a time.
+    struct Sums {
+        uint32_t r[DPW == 1 ? 2 : 1][kPMG];
+        uint32_t taddr;
+        __device__ __forceinline__ void init(uint32_t tmem, int warp)
+        {
+            if (DPW == 1) {
+#pragma unroll
+                for (int i = 0; i < kPMG; i++) r[0][i] = r[DPW == 1 ? 1 : 0][i] = 0u;
+            } else {
+                taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(64 * (warp >> 2));
+                uint32_t z[16];
+#pragma unroll
+                for (int i = 0; i < 16; i++) z[i] = 0u;
+#pragma unroll
+                for (int c = 0; c < 4; c++) afumma::st_32x32b_x16(taddr + 16 * c, z);
+                afumma::wait_st();
+            }
+        }
+        __device__ __forceinline__ void fold(uint32_t (&A)[2][kPMG], int u, int lane)
+        {
+            uint32_t carry = 0u;
+#pragma unroll
+            for (int h = 1; h >= 0; h--) {
+                if (DPW == 1) {
+                    fold_half(A, h, r[DPW == 1 ? h : 0], carry, lane);
+                } else {
+                    uint32_t w[16];
+                    afumma::ld_32x32b_x16(taddr + 32 * u + 16 * h, w);
+                    afumma::wait_ld();
+                    fold_half(A, h, w, carry, lane);
+                    afumma::st_32x32b_x16(taddr + 32 * u + 16 * h, w);
+                }
+            }
+            if (DPW == 2) afumma::wait_st();
+        }
+        // half h of row u
+        __device__ __forceinline__ void get(int u, int h, uint32_t (&w)[kPMG]) const
+        {
+            if (DPW == 1) {
+#pragma unroll
+                for (int i = 0; i < kPMG; i++) w[i] = r[DPW == 1 ? h : 0][i];
+            } else {
+                afumma::ld_32x32b_x16(taddr + 32 * u + 16 * h, w);
+                afumma::wait_ld();
+            }
+        }
+    };
+
     // DM block jb, outputs t0 .. t0 + TTE - 1 of the time block a.T0.
-    static __device__ __forceinline__ void run(const PairArgs& a, uint8_t* smem, unsigned jb, int64_t t0)
+    static __device__ __forceinline__ void run(const PairArgs& a, uint8_t* smem, unsigned jb, int64_t t0, uint32_t tmem)
     {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        int* tab = (int*)(smem + (size_t)NS * a.stage_bytes);
-        uint64_t* bars = (uint64_t*)(tab + NS * NW * kPTABW);
+        uint16_t* tab = (uint16_t*)(smem + (size_t)NS * a.stage_bytes);
+        uint64_t* bars = (uint64_t*)(tab + NS * ND * kPTABW);
         const uint32_t full0 = afptx::smem_addr(bars), empty0 = full0 + 8 * NS;
         const int cbeg = __ldg(a.chkoff + jb), nchk = __ldg(a.chkoff + jb + 1) - cbeg;
 
@@ -318,15 +429,14 @@ struct PairTile {
             return;
         }
 
-        // ---------------- consumer warps: one DM row each
-        const int drow = (int)jb * NW + warp;
-        uint32_t A[2][kPMG], Wd[kPMG][2];
+        // ---------------- consumer warps: DPW DM rows each
+        uint32_t A[DPW][2][kPMG];
+        Sums sums;
 #pragma unroll
-        for (int m = 0; m < kPMG; m++) {
-            A[0][m] = A[1][m] = 0u;
-            Wd[m][0] = Wd[m][1] = 0u;
-        }
-        const uint32_t lane4 = (uint32_t)lane * 4u;
+        for (int u = 0; u < DPW; u++)
+#pragma unroll
+            for (int m = 0; m < kPMG; m++) A[u][0][m] = A[u][1][m] = 0u;
+        sums.init(tmem, warp);
         int npacc = 0;
         for (int kk = 0; kk < nchk; kk++) {
             const int st = kk % NS;
@@ -334,105 +444,148 @@ struct PairTile {
                 if (lane == 0) atomicExch(a.err, 1);
                 return;
             }
-            const int* tb = tab + (st * NW + warp) * kPTABW;
-            const int4 h = *reinterpret_cast<const int4*>(tb);  // starts 0, 1; counts 0, 1
-            const int npc = h.z + h.w;
-            if (npacc + npc > a.flush) {
-                fold(A, Wd, lane);
-                npacc = 0;
-            }
-            npacc += npc;
+            const uint16_t* tb0 = tab + (st * ND + warp * DPW) * kPTABW;
+            const uint8_t* base = smem + (size_t)st * a.stage_bytes + 4 * lane;
 #pragma unroll
-            for (int r = 0; r < 2; r++) {
-                const int beg = r == 0 ? h.x : h.y;
-                const int n = r == 0 ? h.z : h.w;
-                const int* o = tb + 4 + beg;
-                // the next two rows' offsets one iteration ahead (reads past the
-                // bucket stay inside the table and are never used)
-                int2 nx = *reinterpret_cast<const int2*>(o);
-                int i = 0;
-                for (; i + 2 <= n; i += 2) {
-                    const int2 oo = nx;
-                    nx = *reinterpret_cast<const int2*>(o + i + 2);
-                    const uint8_t* p1 = smem + oo.x + lane4;
-                    const uint8_t* p2 = smem + oo.y + lane4;
-                    uint32_t w1[kPMG], w2[kPMG];
+            for (int u = 0; u < DPW; u++) {
+                const uint16_t* tb = tb0 + u * kPTABW;
+                const uint2 h = *reinterpret_cast<const uint2*>(tb);  // starts 0, 1; counts 0, 1
+                if (u == 0) {  // the chunk's groups: the same number of rows for every DM
+                    const int npc = (int)((h.y & 0xFFFFu) + (h.y >> 16));
+                    if (npacc + npc > a.flush) {
 #pragma unroll
-                    for (int m = 0; m < kPMG; m++) {
-                        w1[m] = *reinterpret_cast<const uint32_t*>(p1 + 128 * m);
-                        w2[m] = *reinterpret_cast<const uint32_t*>(p2 + 128 * m);
+                        for (int v = 0; v < DPW; v++) sums.fold(A[v], v, lane);
+                        npacc = 0;
                     }
-#pragma unroll
-                    for (int m = 0; m < kPMG; m++) A[r][m] += w1[m] + w2[m];
+                    npacc += npc;
                 }
-                if (i < n) {
-                    const uint8_t* p1 = smem + nx.x + lane4;
 #pragma unroll
-                    for (int m = 0; m < kPMG; m++) A[r][m] += *reinterpret_cast<const uint32_t*>(p1 + 128 * m);
+                for (int r = 0; r < 2; r++) {
+                    const int beg = (int)(r == 0 ? h.x & 0xFFFFu : h.x >> 16);
+                    const int n = (int)(r == 0 ? h.y & 0xFFFFu : h.y >> 16);
+                    const uint16_t* o = tb + 4 + beg;
+                    // the next two rows' offsets one iteration ahead (reads past the
+                    // bucket stay inside the table and are never used)
+                    uint32_t nx = *reinterpret_cast<const uint32_t*>(o);
+                    int i = 0;
+                    for (; i + 2 <= n; i += 2) {
+                        const uint32_t oo = nx;
+                        nx = *reinterpret_cast<const uint32_t*>(o + i + 2);
+                        const uint8_t* p1 = base + 4u * (oo & 0xFFFFu);
+                        const uint8_t* p2 = base + 4u * (oo >> 16);
+                        uint32_t w1[kPMG], w2[kPMG];
+#pragma unroll
+                        for (int m = 0; m < kPMG; m++) {
+                            w1[m] = *reinterpret_cast<const uint32_t*>(p1 + 128 * m);
+                            w2[m] = *reinterpret_cast<const uint32_t*>(p2 + 128 * m);
+                        }
+#pragma unroll
+                        for (int m = 0; m < kPMG; m++) A[u][r][m] += w1[m] + w2[m];
+                    }
+                    if (i < n) {
+                        const uint8_t* p1 = base + 4u * (nx & 0xFFFFu);
+#pragma unroll
+                        for (int m = 0; m < kPMG; m++) A[u][r][m] += *reinterpret_cast<const uint32_t*>(p1 + 128 * m);
+                    }
                 }
             }
             __syncwarp();
             if (lane == 0) afptx::mbar_arrive(empty0 + 8 * st);
         }
-        fold(A, Wd, lane);
 
         // ---- outputs and fused row sums
-        const int orow = __ldg(a.perm + drow);
-        long long ssum = 0, ssq = 0;
 #pragma unroll
-        for (int m = 0; m < kPMG; m++) {
+        for (int u = 0; u < DPW; u++) {
+            sums.fold(A[u], u, lane);
+            const int orow = __ldg(a.perm + (int)jb * ND + warp * DPW + u);
+            long long ssum = 0, ssq = 0;
 #pragma unroll
-            for (int k = 0; k < 2; k++) {
-                const int pos = 2 * (lane + 32 * m) + k;
-                const int64_t t = t0 + pos;
-                const uint32_t v = Wd[m][k];
-                if (orow >= 0 && pos < kPTTE && t < a.tend) {
-                    a.Y[(int64_t)orow * a.nout + t] = (int32_t)v;
-                    ssum += (long long)v;
-                    ssq += (long long)v * (long long)v;
+            for (int h = 0; h < 2; h++) {
+                uint32_t w[kPMG];
+                sums.get(u, h, w);
+#pragma unroll
+                for (int i = 0; i < 8; i++) {
+#pragma unroll
+                    for (int k = 0; k < 2; k++) {
+                        const int pos = 2 * (lane + 32 * (8 * h + i)) + k;
+                        const int64_t t = t0 + pos;
+                        const uint32_t v = w[2 * i + k];
+                        if (orow >= 0 && pos < kPTTE && t < a.tend) {
+                            a.Y[(int64_t)orow * a.nout + t] = (int32_t)v;
+                            ssum += (long long)v;
+                            ssq += (long long)v * (long long)v;
+                        }
+                    }
                 }
             }
-        }
-        if (a.stats) {
+            if (a.stats) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                ssum += __shfl_xor_sync(0xffffffffu, ssum, o);
-                ssq += __shfl_xor_sync(0xffffffffu, ssq, o);
-            }
-            if (lane == 0 && orow >= 0) {
-                atomicAdd(reinterpret_cast<unsigned long long*>(&a.stats[orow].sum), (unsigned long long)ssum);
-                atomicAdd(reinterpret_cast<unsigned long long*>(&a.stats[orow].sumsq), (unsigned long long)ssq);
+                for (int o = 16; o > 0; o >>= 1) {
+                    ssum += __shfl_xor_sync(0xffffffffu, ssum, o);
+                    ssq += __shfl_xor_sync(0xffffffffu, ssq, o);
+                }
+                if (lane == 0 && orow >= 0) {
+                    atomicAdd(reinterpret_cast<unsigned long long*>(&a.stats[orow].sum), (unsigned long long)ssum);
+                    atomicAdd(reinterpret_cast<unsigned long long*>(&a.stats[orow].sumsq), (unsigned long long)ssq);
+                }
             }
         }
     }
 };
 
+// Tensor memory of a block with two DM rows per warp: allocated by the producer
+// warp; the address is visible to every thread on return.
+__device__ __forceinline__ uint32_t pair_tmem_alloc(uint32_t* slot)
+{
+    if ((int)threadIdx.x >> 5 == kPNW) {
+        afumma::tmem_alloc(afptx::smem_addr(slot), kPTM);
+        afumma::tmem_relinquish();
+    }
+    afumma::fence_before_sync();
+    __syncthreads();
+    afumma::fence_after_sync();
+    return *slot;
+}
+
+__device__ __forceinline__ void pair_tmem_free(uint32_t tmem)
+{
+    afumma::fence_before_sync();
+    __syncthreads();  // every warp is done with its sums
+    afumma::fence_after_sync();
+    if ((int)threadIdx.x >> 5 == kPNW) afumma::tmem_dealloc(tmem, kPTM);
+}
+
 // Grid = time tiles of the block x DM blocks, DM blocks fastest (a tile's rows
 // stay in L2 while every DM block reads them).
-template <int NW, int NS>
-__global__ void __launch_bounds__((NW + 1) * 32, 1) k_pair_tile(const PairArgs a)
+template <int NS, int DPW>
+__global__ void __launch_bounds__((kPNW + 1) * 32, 1) k_pair_tile(const PairArgs a)
 {
     extern __shared__ __align__(16) uint8_t smem[];
-    PairTile<NW, NS>::run(a, smem, blockIdx.x % a.nblk, a.T0 + (int64_t)(blockIdx.x / a.nblk) * kPTTE);
+    __shared__ uint32_t tslot;
+    const uint32_t tmem = DPW == 2 ? pair_tmem_alloc(&tslot) : 0u;
+    PairTile<NS, DPW>::run(a, smem, blockIdx.x % a.nblk, a.T0 + (int64_t)(blockIdx.x / a.nblk) * kPTTE, tmem);
+    if (DPW == 2) pair_tmem_free(tmem);
 }
 
 // Persistent form over many plans' time blocks (a batch of beams): items
 // (job, DM block, tile) in job order, DM blocks fastest, handed out by an
-// atomic counter; every job carries its own tables and ring-stage size (the
-// shared memory is sized for the largest).  The ring barriers are
-// invalidated and initialised again between items.
-template <int NW, int NS>
-__global__ void __launch_bounds__((NW + 1) * 32, 1)
+// atomic counter; every job carries its own tables, DM rows per warp and
+// ring-stage size (the shared memory is sized for the largest).  The ring
+// barriers are invalidated and initialised again between items.
+template <int NS>
+__global__ void __launch_bounds__((kPNW + 1) * 32, 1)
 k_pair_persistent(const PairArgs* __restrict__ jobs, const long long* __restrict__ first, int njobs,
                   long long total, unsigned long long* counter)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ long long item_s;
+    __shared__ uint32_t tslot;
+    const uint32_t tmem = pair_tmem_alloc(&tslot);
     for (;;) {
         if (threadIdx.x == 0) item_s = (long long)atomicAdd(counter, 1ull);
         __syncthreads();
         const long long item = item_s;
-        if (item >= total) return;
+        if (item >= total) break;
         int lo = 0, hi = njobs - 1;  // the job holding the item: first[j] <= item < first[j + 1]
         while (lo < hi) {
             const int mid = (lo + hi + 1) / 2;
@@ -441,24 +594,29 @@ k_pair_persistent(const PairArgs* __restrict__ jobs, const long long* __restrict
         }
         const PairArgs& a = jobs[lo];
         const long long local = item - __ldg(first + lo);
-        PairTile<NW, NS>::run(a, smem, (unsigned)(local % a.nblk), a.T0 + (local / a.nblk) * kPTTE);
+        const unsigned jb = (unsigned)(local % a.nblk);
+        const int64_t t0 = a.T0 + (local / a.nblk) * kPTTE;
+        if (a.dpw == 2) PairTile<NS, 2>::run(a, smem, jb, t0, tmem);
+        else PairTile<NS, 1>::run(a, smem, jb, t0, tmem);
         __syncthreads();  // every warp is done with the ring before its barriers are reset
         if (threadIdx.x == 0) {
-            const uint32_t bar0 = afptx::smem_addr(smem + (size_t)NS * a.stage_bytes + (size_t)NS * NW * kPTABW * 4);
+            const uint32_t bar0 = afptx::smem_addr(smem + (size_t)NS * a.stage_bytes) +
+                                  (uint32_t)(NS * kPNW * a.dpw * kPTABW * 2);
             for (int s = 0; s < 2 * NS; s++) afptx::mbar_inval(bar0 + 8 * s);
         }
     }
+    pair_tmem_free(tmem);
 }
 
-size_t tables_smem(int ns) { return (size_t)ns * kPNW * kPTABW * 4 + 2 * (size_t)ns * 8; }
+size_t tables_smem(int ns, int dpw) { return (size_t)ns * kPNW * dpw * kPTABW * 2 + 2 * (size_t)ns * 8; }
 int rows_wstride(int maxdr) { return (int)r16(kET + maxdr + 4 + 4 + 48); }
 size_t rows_smem(int maxdr, int G) { return (size_t)kET + 48 + (size_t)(G - 1) * rows_wstride(maxdr); }
 
-const void* tile_kernel(int ns)
+typedef void (*TileKernel)(const PairArgs);
+TileKernel tile_kernel(int ns, int dpw)
 {
-    return ns == 4 ? (const void*)k_pair_tile<kPNW, 4>
-         : ns == 3 ? (const void*)k_pair_tile<kPNW, 3>
-                   : (const void*)k_pair_tile<kPNW, 2>;
+    if (dpw == 2) return ns == 4 ? k_pair_tile<4, 2> : ns == 3 ? k_pair_tile<3, 2> : k_pair_tile<2, 2>;
+    return ns == 4 ? k_pair_tile<4, 1> : ns == 3 ? k_pair_tile<3, 1> : k_pair_tile<2, 1>;
 }
 
 size_t pair_budget()
@@ -470,13 +628,17 @@ size_t pair_budget()
 }
 
 // Rates measured on GB300 at 2070 MHz (4096-channel workload, 1001 DMs, 3-deep
-// ring): stage 2 moves shared-memory bytes (consumer loads + row-window
-// copies) at about 40 / 37 / 31 TB/s for groups of 2 / 3 / 4 channels (fewer
-// groups per chunk and more frequent folds as groups grow); stage 1 moves row
-// bytes + input at about 6.9 / 6.5 / 5.4 TB/s of HBM; the channel tile kernel
-// adds about 17.7 T samples/s.
+// ring).  Stage 2 with its copies (its consumers) left out in a throw-away
+// build: 24.8 / 17.0 / 13.2 ms of shared loads (17.3 / 17.0 / 17.2 ms of window
+// copies, L2 to shared memory) for groups of 2 / 3 / 4 channels in blocks of 15 DM
+// rows; both together 24.8 / 19.2 / 18.8 ms, and in blocks of 30 rows, which copy
+// 0.65 / 0.68 / 0.72 of the bytes, 25.0 / 17.2 / 14.3 ms.  Stage 1 moves row bytes +
+// input at about 6.6 TB/s of HBM; the channel tile kernel adds about 17.7 T samples/s.
 constexpr double kTileAddps = 17.7e12;
-inline double smem_rate(int G) { return G == 4 ? 31e12 : G == 3 ? 37e12 : 40e12; }
+constexpr double kBlockStart = 4.5e-6;  // a stage-2 block's first copies and its stores, per 15 DM rows
+constexpr double kRowRate = 6.5e12;
+inline double load_rate(int G) { return G == 4 ? 33.6e12 : G == 3 ? 34.7e12 : 35.7e12; }
+inline double copy_rate(int G) { return G == 4 ? 7.0e12 : 7.6e12; }
 inline double row_rate(int G) { return G == 4 ? 5.2e12 : G == 3 ? 6.2e12 : 6.5e12; }
 
 }  // namespace
@@ -486,7 +648,7 @@ int af_pair_ring_depth(int ns) { return ns; }
 
 void af_pairs_free(af_pair_tables* T)
 {
-    af_tile_tables_free(&T->tt);
+    cudaFree(T->d_perm);
     cudaFree(T->d_rdelta);
     cudaFree(T->d_gdr);
     cudaFree(T->d_chunks);
@@ -495,7 +657,6 @@ void af_pairs_free(af_pair_tables* T)
     cudaFree(T->d_srec);
     for (auto& l : T->lay) {
         cudaFree(l.d_pinfo);
-        cudaFree(l.d_gmax);
         cudaFree(l.d_rinfo);
         cudaFree(l.d_rowoff);
         cudaFree(l.d_soff);
@@ -505,11 +666,11 @@ void af_pairs_free(af_pair_tables* T)
     *T = af_pair_tables();
 }
 
-// Host tables of channel groups of G (2 or 4) channels (once per plan).
-// Leaves T->ok false, and returns AF_OK, when the plan is not suited: a block
-// whose group needs more than a stage of rows, a delta range beyond the
-// stage-1 window, more than 8 rows per group and block, or windows that fit
-// no ring shape.
+// Host tables of channel groups of G (2 to 4) channels and dpw DM rows per
+// consumer warp (once per plan; no CUDA calls).  Leaves T->ok false when the
+// plan is not suited: a block whose group needs more than a stage of rows, a
+// delta range beyond the stage-1 window, more than 8 rows per group and 15 DM
+// rows, or windows that fit no ring shape.
 //
 // Group q holds channels G q .. G q + G - 1 (fewer in the last group); a row
 // is one tuple of delays relative to the group's first channel,
@@ -525,15 +686,12 @@ void af_pairs_free(af_pair_tables* T)
 // for the time block's first tile.
 typedef std::array<int32_t, 3> Key;
 
-static int build_groups(af_plan_t p, int G, af_pair_tables* T)
+static void build_groups(af_plan_t p, int G, int dpw, int optin, const std::vector<int>& order, af_pair_tables* T)
 {
-    af_pairs_free(T);
-    const int nchan = p->nchan, ndm = p->ndm, NW = kPNW, K = G - 1;
-    std::vector<int32_t> dsort, dmin;
-    if (int rc = af_tile_tables_build(p->delays.data(), p->dms.data(), ndm, nchan, NW, 8, p->device, &T->tt, &dsort,
-                                      &dmin))
-        return rc;
-    const int nblk = T->tt.nblk;
+    const int nchan = p->nchan, ndm = p->ndm, NW = kPNW * dpw, K = G - 1;  // NW: DM rows of a block
+    const int nblk = (ndm + NW - 1) / NW;
+    // plane row of a block's w-th DM, ascending (the last one repeated as padding)
+    auto dm_of = [&](int j, int w) { return order[std::min(j * NW + w, ndm - 1)]; };
     const int ng = (nchan + G - 1) / G;
     const int32_t* D = p->delays.data();
     auto key_of = [&](const int32_t* row, int c0) {
@@ -542,9 +700,8 @@ static int build_groups(af_plan_t p, int G, af_pair_tables* T)
             if (c0 + i < nchan) k[i - 1] = row[c0 + i] - row[c0];
         return k;
     };
-    // rows of a group are stored in order of their start B_g (so that the rows
-    // a stretch of samples overlaps are contiguous); rlook maps a tuple to its
-    // row (per group, sorted by tuple)
+    // rows of a group are stored in lexicographic order of their tuples (stage 1
+    // keeps partial sums from one to the next); rlook finds a tuple's row
     std::vector<int32_t> rb(ng + 1, 0), rdelta, rB, rspan, ub(ng);
     std::vector<std::pair<Key, int32_t>> rlook;
     std::vector<int2> gdr((size_t)ng * K);
@@ -570,7 +727,6 @@ static int build_groups(af_plan_t p, int G, af_pair_tables* T)
             rows.push_back(Row{v[d].first, B, v[e - 1].second - B});
             d = e;
         }
-        std::stable_sort(rows.begin(), rows.end(), [](const Row& a, const Row& b) { return a.B < b.B; });
         const size_t n0 = rB.size();
         for (const Row& r : rows) {
             rlook.push_back(std::make_pair(r.key, (int32_t)rB.size()));
@@ -578,9 +734,8 @@ static int build_groups(af_plan_t p, int G, af_pair_tables* T)
             rB.push_back(r.B);
             rspan.push_back(r.span);
         }
-        std::sort(rlook.begin() + n0, rlook.end());
         rb[q + 1] = (int32_t)rB.size();
-        ub[q] = rB[n0];
+        ub[q] = *std::min_element(rB.begin() + n0, rB.end());
         for (int i = 0; i < K; i++) {
             int32_t lo = INT32_MAX, hi = INT32_MIN;
             for (const Row& r : rows) {
@@ -596,71 +751,72 @@ static int build_groups(af_plan_t p, int G, af_pair_tables* T)
     for (int j = 0; j < nblk; j++)
         for (int c = 0; c < nchan; c += G) {
             int32_t hi = INT32_MIN;
-            for (int w = 0; w < NW; w++) hi = std::max(hi, dsort[(size_t)(j * NW + w) * nchan + c]);
-            spread = std::max(spread, hi - dmin[(size_t)j * nchan + c]);
+            int32_t lo = INT32_MAX;
+            for (int w = 0; w < NW; w++) {
+                const int32_t v0 = D[(size_t)dm_of(j, w) * nchan + c];
+                hi = std::max(hi, v0);
+                lo = std::min(lo, v0);
+            }
+            spread = std::max(spread, hi - lo);
         }
-    int optin = 0;
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
     const int64_t rwe = r8((int64_t)spread + 1031);
-    if (spread >= (1 << 20) || maxdr > kMaxDr) return AF_OK;
+    if (spread >= (1 << 20) || maxdr > kMaxDr) return;
     int NS = 3;
     if (const char* e = getenv("AFGB_PAIR_STAGES")) NS = std::min(4, std::max(2, atoi(e)));
     // one stage: up to kPSL windows back to back; the widest window must fit
     // (16 bytes stay free for the static shared memory of the persistent form)
-    const int stage_bytes = (int)(((size_t)optin - tables_smem(NS) - 16) / NS) & ~15;
-    if (2 * rwe > stage_bytes) return AF_OK;
+    const int stage_bytes = (int)(((size_t)optin - tables_smem(NS, dpw) - 16) / NS) & ~15;
+    if (2 * rwe > stage_bytes) return;
     // chunks of whole groups, at most kPSL windows and stage_bytes each, per block; their tables
     struct Ent {
-        int slot[kPNW];
-        int e[kPNW];
+        int slot[2 * kPNW];
+        int e[2 * kPNW];
     };
     std::vector<Ent> ents;
     std::vector<int2> chunks;
     std::vector<int32_t> chkoff(nblk + 1, 0), srow, scpart;
     std::vector<int2> srec;  // per slot: window bytes, offset inside its stage
-    std::vector<int> tabs;
+    std::vector<uint16_t> tabs;
     std::vector<Key> dq(NW), S;
     std::vector<int32_t> d0(NW), sdm;
-    int open_slots = 0, open_bytes = 0, first_slot = 0, kloc = 0;
+    int open_slots = 0, open_bytes = 0, first_slot = 0;
     std::vector<int> sbyt, soffs;  // slot bytes and stage offsets of the open group
     auto flush = [&]() {
         if (ents.empty()) return;
-        const int st = kloc % NS;
         const size_t base = tabs.size();
         tabs.resize(base + (size_t)NW * kPTABW, 0);
         for (int w = 0; w < NW; w++) {
-            int* tb = tabs.data() + base + (size_t)w * kPTABW;
+            uint16_t* tb = tabs.data() + base + (size_t)w * kPTABW;
             int cnt[2] = {0, 0};
             for (const Ent& en : ents) cnt[en.e[w] & 1]++;
             int pos[2] = {0, (cnt[0] + 1) & ~1};  // bucket starts even: offsets load in pairs
-            tb[0] = pos[0];
-            tb[1] = pos[1];
-            tb[2] = cnt[0];
-            tb[3] = cnt[1];
+            tb[0] = (uint16_t)pos[0];
+            tb[1] = (uint16_t)pos[1];
+            tb[2] = (uint16_t)cnt[0];
+            tb[3] = (uint16_t)cnt[1];
             for (const Ent& en : ents) {
                 const int r = en.e[w] & 1;
-                tb[4 + pos[r]++] = st * stage_bytes + srec[first_slot + en.slot[w]].y + 2 * (en.e[w] - r);
+                // bytes from the stage's start, a multiple of 4 below 2^18
+                tb[4 + pos[r]++] = (uint16_t)((srec[first_slot + en.slot[w]].y + 2 * (en.e[w] - r)) / 4);
             }
         }
         chunks.push_back(make_int2(open_slots, first_slot));
         ents.clear();
         open_slots = 0;
         open_bytes = 0;
-        kloc++;
     };
     for (int j = 0; j < nblk; j++) {
-        kloc = 0;
         for (int q = 0; q < ng; q++) {
             const int c0 = G * q;
             for (int w = 0; w < NW; w++) {
-                const int32_t* row = dsort.data() + (size_t)(j * NW + w) * nchan;
+                const int32_t* row = D + (size_t)dm_of(j, w) * nchan;
                 d0[w] = row[c0];
                 dq[w] = key_of(row, c0);
             }
             S.assign(dq.begin(), dq.end());
             std::sort(S.begin(), S.end());
             S.erase(std::unique(S.begin(), S.end()), S.end());
-            if ((int)S.size() > kPSL) return AF_OK;
+            if ((int)S.size() > kPSL) return;
             // one window per (block, row): from the smallest delay of the block's DMs on that row
             sdm.assign(S.size(), 0);
             sbyt.assign(S.size(), 0);
@@ -676,7 +832,7 @@ static int build_groups(af_plan_t p, int G, af_pair_tables* T)
                 sbyt[k] = (int)(2 * r8((int64_t)(hi - lo) + 1031));
                 gbytes += sbyt[k];
             }
-            if (gbytes > stage_bytes) return AF_OK;
+            if (gbytes > stage_bytes) return;
             if (open_slots + (int)S.size() > kPSL || open_bytes + gbytes > stage_bytes) flush();
             if (ents.empty()) first_slot = (int)srec.size();
             for (size_t k = 0; k < S.size(); k++) {
@@ -699,13 +855,14 @@ static int build_groups(af_plan_t p, int G, af_pair_tables* T)
         flush();
         chkoff[j + 1] = (int32_t)chunks.size();
     }
-    // rows copied per group and block: beyond 8 the copies alone outweigh the
-    // loads they save (the reservation weighs the rest)
+    // rows copied per group and block: beyond 8 for 15 DM rows the copies alone
+    // outweigh the loads they save (the reservation weighs the rest)
     const double rows_per_group = (double)srec.size() / ((double)nblk * ng);
-    if (rows_per_group > 8.0) return AF_OK;
+    if (rows_per_group > 8.0 * dpw) return;
     double copy = 0;
     for (const int2& r : srec) copy += r.x;
     T->G = G;
+    T->dpw = dpw;
     T->np = ng;
     T->nrows = (int)rB.size();
     T->rwe = (int)rwe;
@@ -715,47 +872,89 @@ static int build_groups(af_plan_t p, int G, af_pair_tables* T)
     T->shape = NS;
     T->stage_bytes = stage_bytes;
     T->copy_per_tile = copy;
-    T->h_rb = rb;
-    T->h_ub = ub;
-    T->h_rB = rB;
-    T->h_rspan = rspan;
-    T->h_srow = srow;
-    T->h_scpart = scpart;
-    cudaError_t e;
-    auto up = [&](void** d, const void* h, size_t n) {
-        if ((e = cudaMalloc(d, n)) != cudaSuccess) return false;
-        return (e = cudaMemcpy(*d, h, n, cudaMemcpyHostToDevice)) == cudaSuccess;
+    T->nblk = nblk;
+    T->ndm_pad = nblk * NW;
+    T->spread = spread;
+    T->h_rb = std::move(rb);
+    T->h_ub = std::move(ub);
+    T->h_rB = std::move(rB);
+    T->h_rspan = std::move(rspan);
+    T->h_srow = std::move(srow);
+    T->h_scpart = std::move(scpart);
+    T->h_rdelta = std::move(rdelta);
+    T->h_gdr = std::move(gdr);
+    T->h_chunks = std::move(chunks);
+    T->h_chkoff = std::move(chkoff);
+    T->h_tabs = std::move(tabs);
+    T->h_srec = std::move(srec);
+    T->h_perm.assign(T->ndm_pad, -1);
+    for (int i = 0; i < ndm; i++) T->h_perm[i] = order[i];
+    T->ok = true;
+}
+
+// Device copies of a table set and its layouts' arrays (once, when a
+// reservation or a batch first uses the set; the host copies go).
+static int upload_groups(af_pair_tables* T)
+{
+    if (T->d_tabs) return AF_OK;
+    cudaError_t e = cudaSuccess;
+    auto up = [&](auto** d, auto& h) {
+        if (e == cudaSuccess) e = cudaMalloc(d, h.size() * sizeof(h[0]));
+        if (e == cudaSuccess) e = cudaMemcpy(*d, h.data(), h.size() * sizeof(h[0]), cudaMemcpyHostToDevice);
     };
-    if (!up((void**)&T->d_rdelta, rdelta.data(), rdelta.size() * 4) ||
-        !up((void**)&T->d_gdr, gdr.data(), gdr.size() * sizeof(int2)) ||
-        !up((void**)&T->d_chunks, chunks.data(), chunks.size() * sizeof(int2)) ||
-        !up((void**)&T->d_chkoff, chkoff.data(), chkoff.size() * 4) ||
-        !up((void**)&T->d_tabs, tabs.data(), tabs.size() * 4) ||
-        !up((void**)&T->d_srec, srec.data(), srec.size() * sizeof(int2))) {
-        af_pairs_free(T);
+    up(&T->d_rdelta, T->h_rdelta);
+    up(&T->d_gdr, T->h_gdr);
+    up(&T->d_chunks, T->h_chunks);
+    up(&T->d_chkoff, T->h_chkoff);
+    up(&T->d_srec, T->h_srec);
+    up(&T->d_perm, T->h_perm);
+    for (auto& l : T->lay)
+        if (e != cudaSuccess || (e = cudaMalloc(&l.d_pinfo, (size_t)T->np * sizeof(int4))) != cudaSuccess ||
+            (e = cudaMalloc(&l.d_rinfo, (size_t)T->nrows * sizeof(int4))) != cudaSuccess ||
+            (e = cudaMalloc(&l.d_rowoff, (size_t)T->nrows * 8)) != cudaSuccess ||
+            (e = cudaMalloc(&l.d_soff, T->h_srow.size() * 8)) != cudaSuccess)
+            break;
+    up(&T->d_tabs, T->h_tabs);
+    if (e != cudaSuccess) {  // nothing half done: the set can be tried again
+        auto drop = [](auto*& d) {
+            cudaFree(d);
+            d = nullptr;
+        };
+        drop(T->d_rdelta), drop(T->d_gdr), drop(T->d_chunks), drop(T->d_chkoff), drop(T->d_srec), drop(T->d_perm);
+        drop(T->d_tabs);
+        for (auto& l : T->lay) drop(l.d_pinfo), drop(l.d_rinfo), drop(l.d_rowoff), drop(l.d_soff);
         return af_cuda_check(e, "group tables");
     }
-    for (auto& l : T->lay)
-        if ((e = cudaMalloc(&l.d_pinfo, (size_t)ng * sizeof(int4))) != cudaSuccess ||
-            (e = cudaMalloc(&l.d_gmax, (size_t)ng * sizeof(int))) != cudaSuccess ||
-            (e = cudaMalloc(&l.d_rinfo, (size_t)T->nrows * sizeof(int2))) != cudaSuccess ||
-            (e = cudaMalloc(&l.d_rowoff, (size_t)T->nrows * 8)) != cudaSuccess ||
-            (e = cudaMalloc(&l.d_soff, srow.size() * 8)) != cudaSuccess) {
-            af_pairs_free(T);
-            return af_cuda_check(e, "group tables");
-        }
-    T->ok = true;
+    auto gone = [](auto& h) { std::remove_reference_t<decltype(h)>().swap(h); };
+    gone(T->h_rdelta), gone(T->h_gdr), gone(T->h_chunks), gone(T->h_chkoff), gone(T->h_srec), gone(T->h_perm);
+    gone(T->h_tabs);
     return AF_OK;
 }
 
-// Groups of 2, 3 and 4 channels, all kept until a reservation picks one.
+// Groups of 2, 3 and 4 channels in blocks of 15 and of 30 DM rows, all kept until
+// a reservation picks one; each set is built by its own host thread.
+// (AFGB_PAIR_DPW=1|2 keeps to blocks of 15 or of 30.)
 int af_pairs_build(af_plan_t p)
 {
-    if (int rc = build_groups(p, 2, &p->pairs)) return rc;
-    if (p->nchan >= 8) {
-        if (int rc = build_groups(p, 3, &p->alt[0])) return rc;
-        if (int rc = build_groups(p, 4, &p->alt[1])) return rc;
-    }
+    int optin = 0;
+    AF_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
+    std::vector<int> order(p->ndm);  // plane rows by ascending DM
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->dms[x] < p->dms[y]; });
+    int only = 0;
+    if (const char* e = getenv("AFGB_PAIR_DPW")) only = atoi(e);
+    std::vector<std::future<void>> jobs;
+    const bool threads = (int64_t)p->ndm * p->nchan > 20000;  // a thread takes longer to start than a smaller set
+    int k = 0;
+    for (int G = 2; G <= (p->nchan >= 8 ? 4 : 2); G++)
+        for (int dpw = 1; dpw <= 2; dpw++) {
+            if (only == 3 - dpw) continue;
+            af_pair_tables* T = k == 0 ? &p->pairs : &p->alt[k - 1];
+            k++;
+            jobs.push_back(std::async(threads ? std::launch::async : std::launch::deferred,
+                                      [=, &order] { build_groups(p, G, dpw, optin, order, T); }));
+        }
+    for (auto& j : jobs) j.get();
     return AF_OK;
 }
 
@@ -798,6 +997,7 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
     af_pair_tables* T = &p->pairs;
     af_pair_tables::Layout& ly = T->lay[k];
     if (ly.L == L) return AF_OK;
+    if (int rc = upload_groups(T)) return rc;
     const int64_t need = rows_elems(T, L);
     if (ly.L || (size_t)need * 2 > T->ps_bytes)
         if (int rc = af_cuda_check(cudaDeviceSynchronize(), "pair layout")) return rc;
@@ -810,22 +1010,21 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
         T->ps_bytes = (size_t)need * 2;
     }
     std::vector<int64_t> rowoff(T->nrows), soff(T->h_srow.size());
-    std::vector<int4> pinfo(T->np);
-    std::vector<int> gmax(T->np);
-    std::vector<int2> rinfo(T->nrows);
+    std::vector<int4> pinfo(T->np), rinfo(T->nrows);
     int64_t off = 0, maxlen = 0;
     for (int q = 0; q < T->np; q++) {
-        int64_t end = 0, longest = 0;
-        for (int g = T->h_rb[q]; g < T->h_rb[q + 1]; g++) {
+        const int g0 = T->h_rb[q], g1 = T->h_rb[q + 1];
+        int64_t end = 0;
+        for (int g = g0; g < g1; g++) {
             const int64_t len = row_len(T, g, L);
             rowoff[g] = off;
             off += len;
-            rinfo[g] = make_int2(T->h_rB[g] - T->h_ub[q], (int)len);
-            end = std::max(end, (int64_t)rinfo[g].x + len);
-            longest = std::max(longest, len);
+            const int start = T->h_rB[g] - T->h_ub[q];
+            end = std::max(end, (int64_t)start + len);
+            rinfo[g] = make_int4(start, (int)len, (int)end, start);
         }
-        pinfo[q] = make_int4(T->h_rb[q], T->h_rb[q + 1] - T->h_rb[q], T->h_ub[q], (int)end);
-        gmax[q] = (int)longest;
+        for (int g = g1 - 2; g >= g0; g--) rinfo[g].w = std::min(rinfo[g].w, rinfo[g + 1].w);
+        pinfo[q] = make_int4(g0, g1 - g0, T->h_ub[q], (int)end);
         maxlen = std::max(maxlen, end);
     }
     for (size_t i = 0; i < soff.size(); i++) soff[i] = rowoff[T->h_srow[i]] + T->h_scpart[i];
@@ -835,22 +1034,59 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
         (e = cudaMemcpy(ly.d_soff, soff.data(), soff.size() * 8, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(ly.d_pinfo, pinfo.data(), pinfo.size() * sizeof(int4), cudaMemcpyHostToDevice)) !=
             cudaSuccess ||
-        (e = cudaMemcpy(ly.d_rinfo, rinfo.data(), rinfo.size() * sizeof(int2), cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemcpy(ly.d_gmax, gmax.data(), gmax.size() * sizeof(int), cudaMemcpyHostToDevice)) != cudaSuccess)
+        (e = cudaMemcpy(ly.d_rinfo, rinfo.data(), rinfo.size() * sizeof(int4), cudaMemcpyHostToDevice)) != cudaSuccess)
         return af_cuda_check(e, "pair layout");
     ly.L = L;
     ly.maxlen = maxlen;
     return AF_OK;
 }
 
-// Predicted time (s) of group rows T in time blocks of L outputs on nout outputs.
+// Predicted time (s) of group rows T in time blocks of L outputs on nout
+// outputs.  A stage-2 block takes the 6-norm of its shared loads' and its window
+// copies' times at the rates above (they overlap, not quite), and a launch whole
+// waves of one block per SM: blocks of 30 DM rows are faster by up to a quarter
+// on many waves and slower where 15 rows fill the last wave better (2128 channels,
+// 609 DMs, 22 tiles: 902 blocks of 15 in 0.62 ms, 462 of 30 in 0.75 ms).
 static double rows_cost(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L)
 {
+    const double nsm = p->num_sms > 0 ? p->num_sms : 152;
+    const double loads = 2.0 * kPNW * T->dpw * T->np * 64.0 * kPMG / (load_rate(T->G) / nsm);
+    const double copies = T->copy_per_tile / T->nblk / (copy_rate(T->G) / nsm);
+    const double block = std::pow(std::pow(loads, 6) + std::pow(copies, 6), 1.0 / 6) + kBlockStart * T->dpw;
+    auto waves = [&](int64_t outs) {
+        return std::ceil((double)((outs + kPTTE - 1) / kPTTE) * T->nblk / nsm);
+    };
+    const int64_t full = nout / L, rest = nout - full * L;
+    const double s2 = block * ((double)full * waves(L) + (rest > 0 ? waves(rest) : 0.0));
+    // stage 1: HBM, and a block's window loads (1 ns per channel and block of the whole GPU)
+    double blocks1 = 0;
+    for (int q = 0; q < T->np; q++) {
+        int64_t end = 0;
+        for (int g = T->h_rb[q]; g < T->h_rb[q + 1]; g++)
+            end = std::max(end, (int64_t)T->h_rB[g] - T->h_ub[q] + row_len(T, g, L));
+        blocks1 += (double)((end + kET - 1) / kET);
+    }
+    const double times = (double)full + (rest > 0 ? (double)rest / L : 0.0);
+    const double s1 = times * (2.0 * (double)rows_elems(T, L) / kRowRate + blocks1 * 4e-9 * T->G) +
+                      (double)p->nchan * (double)(nout + p->dmax) / kRowRate + 8e-6;
+    return s1 + s2;
+}
+
+// The same at throughput alone, neither side's launches, waves or latencies
+// counted, as the channel tile kernel's time below is: what decides between the two.
+static double rows_rate_cost(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L)
+{
     const double tiles = (double)((nout + kPTTE - 1) / kPTTE), blocks = (double)((nout + L - 1) / L);
-    const double s2 = (2.0 * T->tt.ndm_pad * T->np * (double)nout + tiles * T->copy_per_tile) / smem_rate(T->G);
+    const double rate = T->G == 4 ? 31e12 : T->G == 3 ? 37e12 : 40e12;  // loads + copies, blocks of 15 DM rows
+    const double s2 = (2.0 * T->ndm_pad * T->np * (double)nout + tiles * T->copy_per_tile) / rate;
     const double s1 = (blocks * 2.0 * (double)rows_elems(T, L) + (double)p->nchan * (double)(nout + p->dmax)) /
                       row_rate(T->G);
     return s1 + s2;
+}
+
+static bool rows_beat_tile(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L)
+{
+    return rows_rate_cost(p, T, nout, L) < (double)p->ndm * p->nchan * (double)nout / kTileAddps;
 }
 
 // Gives up a table set's row buffer and layouts (after the device is idle).
@@ -868,35 +1104,44 @@ static int pairs_release(af_pair_tables* T)
 
 // Picks the group rows for nout outputs: of the group sizes (2 only unless
 // larger groups are allowed; AFGB_PAIR_GROUP=2|3|4 restricts), the one
-// predicted fastest within max_bytes of rows, if it beats the channel tile
+// predicted fastest within max_bytes of rows, if any beats the channel tile
 // kernel (AFGB_DEDISP_KERNEL=pairs skips that comparison); it becomes
 // p->pairs (a previously picked set gives up its buffer).  *L gets its time
 // block; 0 when nothing suits.
-// The candidate (0: p->pairs, 1, 2: p->alt) and time block the pick would
+// The candidate (0: p->pairs, k: p->alt[k - 1]) and time block the pick would
 // take, or -1; changes nothing.
 static int pairs_choose(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L)
 {
     *L = 0;
-    const af_pair_tables* cand[3] = {&p->pairs, &p->alt[0], &p->alt[1]};
-    int best = -1;
-    double best_t = 0;
-    int64_t best_L = 0;
-    for (int k = 0; k < 3; k++) {
-        const af_pair_tables* T = cand[k];
+    // two predictions: the block model's fastest set is taken where it beats by 3.5 %
+    // (over 22 plans its error on the ratio of two sets was below that where it would
+    // have chosen wrongly) the set of 15-row blocks that moves the fewest bytes
+    int best = -1, plain = -1;
+    double best_t = 0, plain_t = 0, plain_model = 0;
+    int64_t Ls[6] = {};
+    bool beats = false;
+    for (int k = 0; k < 6; k++) {
+        const af_pair_tables* T = k == 0 ? &p->pairs : &p->alt[k - 1];
         if (!T->ok || (T->G != 2 && !allow_larger) || (p->force_group && T->G != p->force_group)) continue;
-        const int64_t Lk = block_len(T, nout, max_bytes);
-        if (Lk <= 0) continue;
-        const double t = rows_cost(p, T, nout, Lk);
+        Ls[k] = block_len(T, nout, max_bytes);
+        if (Ls[k] <= 0) continue;
+        beats = beats || rows_beat_tile(p, T, nout, Ls[k]);
+        const double t = rows_cost(p, T, nout, Ls[k]), r = rows_rate_cost(p, T, nout, Ls[k]);
         if (best < 0 || t < best_t) {
             best = k;
             best_t = t;
-            best_L = Lk;
+        }
+        if (T->dpw == 1 && (plain < 0 || r < plain_t)) {
+            plain = k;
+            plain_t = r;
+            plain_model = t;
         }
     }
     if (best < 0) return -1;
+    if (plain >= 0 && best_t > 0.965 * plain_model) best = plain;
     const bool tile = p->tile.ns1 > 0;  // else the one-thread-per-output kernel
-    if (!p->force_pairs && tile && best_t >= (double)p->ndm * p->nchan * (double)nout / kTileAddps) return -1;
-    *L = best_L;
+    if (!p->force_pairs && tile && !beats) return -1;
+    *L = Ls[best];
     return best;
 }
 
@@ -905,9 +1150,8 @@ int af_pairs_pick(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes
     const int best = pairs_choose(p, nout, allow_larger, max_bytes, L);
     if (best < 0) return AF_OK;
     if (best > 0) {
-        af_pair_tables* cand[3] = {&p->pairs, &p->alt[0], &p->alt[1]};
         if (int rc = pairs_release(&p->pairs)) return rc;
-        std::swap(p->pairs, *cand[best]);
+        std::swap(p->pairs, p->alt[best - 1]);
     }
     return AF_OK;
 }
@@ -917,8 +1161,7 @@ size_t af_pairs_workspace(af_plan_t p, int64_t nout)
     int64_t L = 0;
     const int best = pairs_choose(p, nout, true, SIZE_MAX, &L);
     if (best < 0) return 0;
-    const af_pair_tables* cand[3] = {&p->pairs, &p->alt[0], &p->alt[1]};
-    return 2 * (size_t)rows_elems(cand[best], L);
+    return 2 * (size_t)rows_elems(best == 0 ? &p->pairs : &p->alt[best - 1], L);
 }
 
 // Reserves the picked group rows: the row buffer and the layouts of
@@ -989,8 +1232,7 @@ int af_pairs_attach(af_plan_t p, uint16_t* buf, size_t bytes, int64_t nout)
         if (rows_elems(T, mid * kPTTE) <= cap) lo = mid;
         else hi = mid - 1;
     }
-    if (!p->force_pairs && p->tile.ns1 > 0 &&
-        rows_cost(p, T, nout, lo * kPTTE) >= (double)p->ndm * p->nchan * (double)nout / kTileAddps)
+    if (!p->force_pairs && p->tile.ns1 > 0 && !rows_beat_tile(p, T, nout, lo * kPTTE))
         return AF_OK;  // this beam stays on the channel tile kernel
     if (int rc = af_cuda_check(cudaDeviceSynchronize(), "pairs attach")) return rc;
     if (T->ps_owned) cudaFree(T->d_ps);
@@ -1021,15 +1263,15 @@ int af_launch_pairs_rows(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int la
     const unsigned long long g1 = (unsigned long long)T->np * etiles;
     if (g1 > 0x7fffffffULL) return af_set_error(AF_EINVAL, "pairs: problem too large for one grid");
     if (T->G == 4)
-        k_group_rows<4><<<(unsigned)g1, kS1T, s1, s>>>(d_in, nsamp, p->nchan, ly.d_pinfo, ly.d_gmax, T->d_gdr, T->d_rdelta,
+        k_group_rows<4><<<(unsigned)g1, kS1T, s1, s>>>(d_in, nsamp, p->nchan, ly.d_pinfo, T->d_gdr, T->d_rdelta,
                                                       ly.d_rinfo, ly.d_rowoff, T0, etiles, rows_wstride(T->maxdr),
                                                       dshort, T->d_ps);
     else if (T->G == 3)
-        k_group_rows<3><<<(unsigned)g1, kS1T, s1, s>>>(d_in, nsamp, p->nchan, ly.d_pinfo, ly.d_gmax, T->d_gdr, T->d_rdelta,
+        k_group_rows<3><<<(unsigned)g1, kS1T, s1, s>>>(d_in, nsamp, p->nchan, ly.d_pinfo, T->d_gdr, T->d_rdelta,
                                                       ly.d_rinfo, ly.d_rowoff, T0, etiles, rows_wstride(T->maxdr),
                                                       dshort, T->d_ps);
     else
-        k_group_rows<2><<<(unsigned)g1, kS1T, s1, s>>>(d_in, nsamp, p->nchan, ly.d_pinfo, ly.d_gmax, T->d_gdr, T->d_rdelta,
+        k_group_rows<2><<<(unsigned)g1, kS1T, s1, s>>>(d_in, nsamp, p->nchan, ly.d_pinfo, T->d_gdr, T->d_rdelta,
                                                       ly.d_rinfo, ly.d_rowoff, T0, etiles, rows_wstride(T->maxdr),
                                                       dshort, T->d_ps);
     return af_cuda_check(cudaGetLastError(), "group rows launch");
@@ -1052,36 +1294,29 @@ int af_pairs_block_args(af_plan_t p, int64_t nout, int layout, int64_t T0, int32
     a.tabs = T->d_tabs;
     a.srec = T->d_srec;
     a.soff = ly.d_soff;
-    a.perm = T->tt.d_perm;
+    a.perm = T->d_perm;
     a.stage_bytes = T->stage_bytes;
     a.flush = 65535 / (255 * T->G);
-    a.nblk = (unsigned)T->tt.nblk;
+    a.dpw = T->dpw;
+    a.nblk = (unsigned)T->nblk;
     a.T0 = T0;
     a.tend = std::min(nout, T0 + L);
     a.nout = nout;
     a.Y = d_plane;
     a.stats = d_stats;
     a.err = p->d_err;
-    *items = (long long)((std::min(L, nout - T0) + kPTTE - 1) / kPTTE) * (long long)T->tt.nblk;
+    *items = (long long)((std::min(L, nout - T0) + kPTTE - 1) / kPTTE) * (long long)T->nblk;
     return AF_OK;
 }
 
-size_t af_pairs_stage2_smem(af_plan_t p, int ns) { return (size_t)ns * p->pairs.stage_bytes + tables_smem(ns); }
+size_t af_pairs_stage2_smem(af_plan_t p, int ns) { return (size_t)ns * p->pairs.stage_bytes + tables_smem(ns, p->pairs.dpw); }
 
 int af_launch_pairs_persistent(int ns, size_t smem, int grid, const af_pair_args* d_jobs, const long long* d_first,
                                int njobs, long long total, unsigned long long* d_counter, cudaStream_t s)
 {
-    const void* fn = ns == 4   ? (const void*)k_pair_persistent<kPNW, 4>
-                     : ns == 3 ? (const void*)k_pair_persistent<kPNW, 3>
-                               : (const void*)k_pair_persistent<kPNW, 2>;
-    if (int rc = af_ensure_smem(fn, smem)) return rc;
-    const dim3 blk((kPNW + 1) * 32);
-    if (ns == 4)
-        k_pair_persistent<kPNW, 4><<<grid, blk, smem, s>>>(d_jobs, d_first, njobs, total, d_counter);
-    else if (ns == 3)
-        k_pair_persistent<kPNW, 3><<<grid, blk, smem, s>>>(d_jobs, d_first, njobs, total, d_counter);
-    else
-        k_pair_persistent<kPNW, 2><<<grid, blk, smem, s>>>(d_jobs, d_first, njobs, total, d_counter);
+    const auto fn = ns == 4 ? k_pair_persistent<4> : ns == 3 ? k_pair_persistent<3> : k_pair_persistent<2>;
+    if (int rc = af_ensure_smem((const void*)fn, smem)) return rc;
+    fn<<<grid, (kPNW + 1) * 32, smem, s>>>(d_jobs, d_first, njobs, total, d_counter);
     return af_cuda_check(cudaGetLastError(), "persistent pair tile launch");
 }
 
@@ -1097,15 +1332,10 @@ int af_launch_pairs_block(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int64
     long long items = 0;
     if (int rc = af_pairs_block_args(p, nout, layout, T0, d_plane, d_stats, &a, &items, Lb)) return rc;
     const size_t s2 = af_pairs_stage2_smem(p, T->shape);
-    if (int rc = af_ensure_smem(tile_kernel(T->shape), s2)) return rc;
+    const TileKernel fn = tile_kernel(T->shape, T->dpw);
+    if (int rc = af_ensure_smem((const void*)fn, s2)) return rc;
     if ((unsigned long long)items > 0x7fffffffULL) return af_set_error(AF_EINVAL, "pairs: problem too large for one grid");
-    const dim3 grid2((unsigned)items), blk2((kPNW + 1) * 32);
-    if (T->shape == 4)
-        k_pair_tile<kPNW, 4><<<grid2, blk2, s2, s>>>(a);
-    else if (T->shape == 3)
-        k_pair_tile<kPNW, 3><<<grid2, blk2, s2, s>>>(a);
-    else
-        k_pair_tile<kPNW, 2><<<grid2, blk2, s2, s>>>(a);
+    fn<<<(unsigned)items, (kPNW + 1) * 32, s2, s>>>(a);
     return af_cuda_check(cudaGetLastError(), "pair tile launch");
 }
 

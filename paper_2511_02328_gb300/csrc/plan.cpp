@@ -146,8 +146,7 @@ static void free_plan(af_plan_t p)
     cudaFree(p->d_delays);
     af_tile_tables_free(&p->tile);
     af_pairs_free(&p->pairs);
-    af_pairs_free(&p->alt[0]);
-    af_pairs_free(&p->alt[1]);
+    for (af_pair_tables& t : p->alt) af_pairs_free(&t);
     af_sb_free(p);
     cudaFree(p->d_err);
     cudaFree(p->d_stats);
