@@ -179,7 +179,7 @@ int af_launch_pairs_block(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int64
 // (its input, outputs + Dmax, is copied before any work), each next one six
 // times the previous (its input arrives while the previous one runs), at most
 // cap_tiles each.
-std::vector<int64_t> af_search_block_tiles(int64_t nout, int64_t cap_tiles);
+std::vector<int64_t> af_search_block_tiles(af_plan_t p, int64_t nout, int64_t cap_tiles);
 int af_pair_tile_outputs();
 int af_pair_ring_depth(int shape);
 // Row-buffer bytes of a full-length single time block, and the use of a row

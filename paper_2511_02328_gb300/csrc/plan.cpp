@@ -773,7 +773,7 @@ try {
         // rest of the copy.
         const int ly = p->pairs.lay[1].L > 0 ? 1 : 0;
         const int64_t tte = af_pair_tile_outputs();
-        const std::vector<int64_t> blocks = af_search_block_tiles(nout, p->pairs.lay[ly].L / tte);
+        const std::vector<int64_t> blocks = af_search_block_tiles(p, nout, p->pairs.lay[ly].L / tte);
         AF_CUDA(cudaEventRecord(p->ws_ev[0], s));
         AF_CUDA(cudaStreamWaitEvent(p->ws_copy, p->ws_ev[0], 0));
         AF_CUDA(cudaMemsetAsync(p->d_stats, 0, (size_t)p->ndm * sizeof(af_rowstats_t), s));
