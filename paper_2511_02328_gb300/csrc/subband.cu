@@ -11,7 +11,7 @@
 // delays D[j(m)][c] + R[m][s(c)].
 //
 // Stage 1 is the tile kernel of tile.cuh in subband mode: rows = coarse DMs
-// (11 per block), channels streamed subband by subband, one scratch row
+// (14 per block), channels streamed subband by subband, one scratch row
 // stored per (row, subband).  Its table delays are staggered per (row,
 // subband) so that a block's delay spread is the within-subband dispersion
 // only (see tile.cuh).
@@ -33,8 +33,13 @@
 
 namespace {
 
-constexpr int kSbNW = 11;  // stage-1 block shape (rows x 128-output groups)
-constexpr int kSbM = 8;
+// stage-1 block shape (rows x 128-output groups).  4096 channels, 126 coarse
+// rows, 64 subbands, 262144 samples, both stages: 14 x 6 8.42 ms, 11 x 8 8.58,
+// 9 x 10 8.64, 10 x 10 8.25; 2802 channels, 24 rows, 55424 samples: 0.36, 0.41,
+// 0.40 and 0.40 ms.  15 consumer and producer warps hide more latency and the
+// shorter tile leaves less of the last wave idle.
+constexpr int kSbNW = 14;
+constexpr int kSbM = 6;
 constexpr int kS2Threads = 256;
 constexpr int kS2BufBytes = 24576;       // target bytes per stage-2 buffer
 constexpr int64_t kScratchBudget = (int64_t)1 << 30;  // default stage-1 scratch
@@ -184,6 +189,12 @@ void s2_geometry(af_plan_t p, int* rw, int* sc, size_t* smem)
     *smem = 2 * (size_t)(*sc) * (size_t)(*rw) * es + 16 + (rbytes <= (size_t)kS2RBytes ? rbytes : 0);
 }
 
+const void* s1_fn(bool i16)
+{
+    return i16 ? (const void*)aftile::k_tile_sb<kSbNW, kSbM, aftile::kSub16>
+               : (const void*)aftile::k_tile_sb<kSbNW, kSbM, aftile::kSub32>;
+}
+
 template <typename T>
 const void* s2_fn(int n0)
 {
@@ -206,6 +217,40 @@ void s2_launch(int n0, unsigned grid, size_t smem, cudaStream_t s, const T* I, i
     case 16: Stage2<T, 16>::launch(grid, smem, s, I, ipitch, nsub, n0, ndm, R, rw, sc, v0, lcur, nout, vtiles, Y, stats, err); break;
     default: Stage2<T, 32>::launch(grid, smem, s, I, ipitch, nsub, n0, ndm, R, rw, sc, v0, lcur, nout, vtiles, Y, stats, err); break;
     }
+}
+
+// Stage-1 tiles of a time block of l outputs.
+int64_t s1_tiles(af_plan_t p, int64_t l)
+{
+    constexpr int TTE = aftile::tte_of(kSbM);
+    return (l + p->sb_rmax + p->sb.maxstag + TTE - 1) / TTE;
+}
+
+// Outputs per time block, at most the plan's sb_L: of the lengths whose stage-1
+// blocks fill whole waves of one per SM, and sb_L itself, the one with the
+// fewest waves in total (the longest of these: each block recomputes the
+// residual and stagger overlap).  11 x 8 blocks, 4096 channels: 9.14 ms with
+// blocks of sb_L (6 waves for 5.4), 8.58 ms so.
+int64_t time_block(af_plan_t p, int64_t nout)
+{
+    constexpr int TTE = aftile::tte_of(kSbM);
+    const int64_t nsm = p->num_sms > 0 ? p->num_sms : 152, nblk = p->sb.tile.nblk;
+    const int64_t over = p->sb_rmax + p->sb.maxstag;
+    auto waves = [&](int64_t l) { return (s1_tiles(p, l) * nblk + nsm - 1) / nsm; };
+    auto total = [&](int64_t l) {
+        const int64_t rest = nout % l;
+        return nout / l * waves(l) + (rest ? waves(rest) : 0);
+    };
+    int64_t best = std::min(p->sb_L, nout), cost = total(best);
+    for (int64_t k = waves(best) - 1; k >= 1 && best > 4096; k--) {
+        const int64_t l = (k * nsm / nblk * TTE - over) / 256 * 256;
+        if (l < 4096 || 2 * l < best) break;
+        if (total(l) < cost) {
+            best = l;
+            cost = total(l);
+        }
+    }
+    return best;
 }
 
 }  // namespace
@@ -248,7 +293,7 @@ int af_sb_prepare(af_plan_t p)
             }
             for (int w = 0; w < kSbNW; w++) {
                 const int r = std::min(b * kSbNW + w, nc - 1);
-                const int32_t st = Dc[(size_t)r * nchan + top[s]] - lo;
+                const int32_t st = (Dc[(size_t)r * nchan + top[s]] - lo) & ~3;  // aligned stores in stage 1
                 stag[(size_t)(b * kSbNW + w) * nsub + s] = st;
                 maxstag = std::max(maxstag, st);
             }
@@ -297,8 +342,7 @@ int af_sb_prepare(af_plan_t p)
         (err = cudaMalloc(&p->sb.d_I, ibytes)) != cudaSuccess)
         return af_cuda_check(err, "af_plan_subband: device tables / scratch");
     if (p->sb.tile.fits)
-        if (int rc = af_ensure_smem((const void*)aftile::k_tile_sb<kSbNW, kSbM>, af_tile_smem(kSbNW, p->sb.tile.rw)))
-            return rc;
+        if (int rc = af_ensure_smem(s1_fn(p->sb.i16), af_tile_smem(kSbNW, p->sb.tile.rw))) return rc;
     return af_ensure_smem(p->sb.i16 ? s2_fn<uint16_t>(p->sb_n0) : s2_fn<uint32_t>(p->sb_n0), s2smem);
 }
 
@@ -309,17 +353,17 @@ int af_launch_subband(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int64_t n
         if (int rc = af_cuda_check(cudaMemsetAsync(d_stats, 0, (size_t)p->ndm * sizeof(af_rowstats_t), s),
                                    "subband stats reset"))
             return rc;
-    constexpr int TTE = aftile::tte_of(kSbM);
     int rw, sc;
     size_t s2smem;
     s2_geometry(p, &rw, &sc, &s2smem);
     const int64_t tv = tv_of(p->sb_n0);
     const size_t s1smem = af_tile_smem(kSbNW, p->sb.tile.rw);
-    if (int rc = af_ensure_smem((const void*)aftile::k_tile_sb<kSbNW, kSbM>, s1smem)) return rc;
+    if (int rc = af_ensure_smem(s1_fn(p->sb.i16), s1smem)) return rc;
     if (int rc = af_ensure_smem(p->sb.i16 ? s2_fn<uint16_t>(p->sb_n0) : s2_fn<uint32_t>(p->sb_n0), s2smem)) return rc;
 
-    for (int64_t v0 = 0; v0 < nout; v0 += p->sb_L) {
-        const int64_t lcur = std::min(p->sb_L, nout - v0);
+    const int64_t L = time_block(p, nout);
+    for (int64_t v0 = 0; v0 < nout; v0 += L) {
+        const int64_t lcur = std::min(L, nout - v0);
         aftile::TileArgs a;
         a.X = d_in;
         a.nsamp = nsamp;
@@ -332,7 +376,7 @@ int af_launch_subband(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int64_t n
         a.nout = 0;
         a.rw = p->sb.tile.rw;
         a.li = lcur + p->sb_rmax;
-        a.tiles = (unsigned)((a.li + p->sb.maxstag + TTE - 1) / TTE);
+        a.tiles = (unsigned)s1_tiles(p, lcur);
         a.nblk = (unsigned)p->sb.tile.nblk;
         a.Y = nullptr;
         a.stats = nullptr;
@@ -342,7 +386,6 @@ int af_launch_subband(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int64_t n
         a.sbfirst = p->sb.d_first;
         a.stag = p->sb.d_stag;
         a.I = p->sb.d_I;
-        a.i16 = p->sb.i16 ? 1 : 0;
         a.ipitch = p->sb.ipitch;
         a.tbase = v0;
         const unsigned long long nb1 = (unsigned long long)a.tiles * a.nblk;
@@ -350,7 +393,10 @@ int af_launch_subband(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int64_t n
         const unsigned long long nb2 = (unsigned long long)vtiles * p->sb_ncoarse;
         if (nb1 > 0x7fffffffULL || nb2 > 0x7fffffffULL)
             return af_set_error(AF_EINVAL, "subband dedisperse: problem too large for one grid");
-        aftile::k_tile_sb<kSbNW, kSbM><<<(unsigned)nb1, (kSbNW + 1) * 32, s1smem, s>>>(a);
+        if (p->sb.i16)
+            aftile::k_tile_sb<kSbNW, kSbM, aftile::kSub16><<<(unsigned)nb1, (kSbNW + 1) * 32, s1smem, s>>>(a);
+        else
+            aftile::k_tile_sb<kSbNW, kSbM, aftile::kSub32><<<(unsigned)nb1, (kSbNW + 1) * 32, s1smem, s>>>(a);
         if (int rc = af_cuda_check(cudaGetLastError(), "subband stage 1 launch")) return rc;
         if (p->sb.i16)
             s2_launch<uint16_t>(p->sb_n0, (unsigned)nb2, s2smem, s, (const uint16_t*)p->sb.d_I, p->sb.ipitch,
