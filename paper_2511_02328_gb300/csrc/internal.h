@@ -135,7 +135,7 @@ struct af_pair_tables {
     struct Layout {
         int64_t L = 0, maxlen = 0;     // outputs per time block, longest row
         int4* d_pinfo = nullptr;       // [np] first row, rows, range start ub, range length
-        int4* d_rinfo = nullptr;       // [nrows] row start - ub, row length, largest end so far, smallest start from here
+        int2* d_rinfo = nullptr;       // [nrows] row start - ub, row length
         int64_t* d_rowoff = nullptr;   // [nrows] element offset in the row buffer
         int64_t* d_soff = nullptr;     // per slot: window offset for a time block's first tile
     } lay[2];

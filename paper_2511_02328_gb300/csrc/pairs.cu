@@ -88,32 +88,41 @@ typedef af_pair_args PairArgs;
 // for every row of the group, the part of those samples inside the row's own
 // range.  pinfo[q] = {first row, rows, ub (the group's first delay rounded down
 // to 16), length of the group's range}; rinfo[g] = {row start - ub (a multiple
-// of 16), row length, the largest end of the group's rows up to g, the smallest
-// start of its rows from g on}; rdelta[g][i-1] = row g's delay of channel Gq+i relative
+// of 16), row length}; rdelta[g][i-1] = row g's delay of channel Gq+i relative
 // to channel Gq; gdr[q][i-1] = the smallest and largest of those over the
 // group's rows.  Channel Gq's window goes to W0, channel Gq+i's (shifted by
 // the smallest delta, longer by the delta range + 4 bytes) to Wi: blocks whose
 // windows lie inside the input rows copy them with aligned 16-byte loads (a
-// window then starts off_i bytes into its buffer), edge blocks byte by byte
-// with zeros outside the rows and for missing channels.  Words at any byte
+// window then starts off_i bytes into its buffer), edge blocks the same with
+// zeros outside the rows and for missing channels (byte by byte a row's last
+// block alone took 20 us).  Words at any byte
 // offset are read with a funnel shift (one shift per block and row).
 // A group's rows come in lexicographic order of their tuples, so that a row
 // mostly shares its first delays with the one before: the sums over those
 // channels stay in registers and only the channels from the first difference on
 // are read and widened again (1.36 of 2 per row for groups of 3, 1.61 of 3 for
 // groups of 4 on the 4096-channel workload).  Bound by HBM (groups of 4: 36.9 GB in
-// 5.58 ms, 0.97 of its measured rate; every channel read again for every row: 6.64
-// ms, 15 ALU instructions per 4 samples and row) or, where rows are few or short,
-// by issue.
+// 5.34 ms, its measured rate; every channel read again for every row: 6.64 ms, 15
+// ALU instructions per 4 samples and row) or, where rows are few or short, by
+// issue.  With every row waiting for its own record, and edge windows copied byte
+// by byte, 3508 channels, 1287 DMs, 19024 outputs took 258 us in groups of 4, 137 so;
+// 271 channels, 543 DMs, 22053 outputs 53 us, 25 so.  8 - G blocks per SM: one
+// block more spills or is slower (G = 4: 1.00 to 1.27 ms), one less up to 1.13 times
+// slower.
 template <int G>
-__global__ void __launch_bounds__(kS1T, G == 4 ? 1 : G == 3 ? 5 : 6)
+__global__ void __launch_bounds__(kS1T, 8 - G)
 k_group_rows(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int4* __restrict__ pinfo,
              const int2* __restrict__ gdr, const int32_t* __restrict__ rdelta,
-             const int4* __restrict__ rinfo, const int64_t* __restrict__ rowoff, int64_t T0, int etiles, int wstride,
+             const int2* __restrict__ rinfo, const int64_t* __restrict__ rowoff, int64_t T0, int etiles, int wstride,
              int dshort, uint16_t* __restrict__ PS)
 {
     constexpr int K = G - 1;
     extern __shared__ __align__(16) uint8_t sm[];
+    __shared__ int64_t s_ro[kS1T];
+    __shared__ int2 s_ri[kS1T];
+    __shared__ int s_dl[K][kS1T];
+    __shared__ int s_cnt[kS1T / 32];
+    __shared__ uint8_t s_list[kS1T];
     const int tid = threadIdx.x;
     const int q = blockIdx.x / etiles;
     const int64_t e0 = (int64_t)(blockIdx.x % etiles) * kET;
@@ -121,27 +130,38 @@ k_group_rows(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int4
     // a time block dshort outputs shorter than the layout's needs every row
     // (and the group's range) dshort samples shorter (dshort a multiple of 16)
     if (e0 >= pi.w - dshort) return;
-    // the rows overlapping [e0, e0 + ET) lie between the first whose running largest
-    // end passes e0 and the first from which on all start at e0 + ET or later (each
-    // is still checked below)
-    int kbeg, kend;
-    {
-        int a = 0, b = pi.y;
-        while (a < b) {
-            const int m = (a + b) >> 1;
-            if (__ldg(&rinfo[pi.x + m].z) - dshort <= e0) a = m + 1;
-            else b = m;
+    // The records of the group's rows in shared memory, kS1T rows a pass, and the
+    // list of those that overlap [e0, e0 + ET): one load per thread, instead of
+    // every row's sum waiting for its own record.
+    bool over = false;
+    auto load_records = [&](int kb) {
+        over = false;
+        if (kb + tid < pi.y) {
+            const int g = pi.x + kb + tid;
+            const int2 r = __ldg(rinfo + g);
+            s_ri[tid] = make_int2(r.x, r.y - dshort);
+            s_ro[tid] = __ldg(rowoff + g);
+#pragma unroll
+            for (int i = 0; i < K; i++) s_dl[i][tid] = __ldg(rdelta + (int64_t)g * K + i);
+            over = r.x < e0 + kET && r.x + r.y - dshort > e0;
         }
-        kbeg = a;
-        b = pi.y;
-        while (a < b) {
-            const int m = (a + b) >> 1;
-            if (__ldg(&rinfo[pi.x + m].w) < e0 + kET) a = m + 1;
-            else b = m;
+    };
+    // ends with a barrier; returns the list's length
+    auto list_records = [&]() {
+        const unsigned bal = __ballot_sync(0xffffffffu, over);
+        if ((tid & 31) == 0) s_cnt[tid >> 5] = __popc(bal);
+        __syncthreads();
+        int n = 0, at = 0;
+#pragma unroll
+        for (int w = 0; w < kS1T / 32; w++) {
+            if (w == (tid >> 5)) at = n;
+            n += s_cnt[w];
         }
-        kend = a;
-    }
-    if (kbeg >= kend) return;
+        if (over) s_list[at + __popc(bal & ((1u << (tid & 31)) - 1u))] = (uint8_t)tid;
+        __syncthreads();
+        return n;
+    };
+    load_records(0);
     const int c0 = G * q;
     const int64_t u0 = T0 + pi.z + e0;
     int dmn[K], bw[K], off[K + 1];
@@ -169,24 +189,29 @@ k_group_rows(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int4
             for (int k = tid; k < ni; k += kS1T) wi[k] = __ldg(gi + k);
         }
     } else {
-        off[0] = 0;
-        for (int k = tid; k < kET + 4; k += kS1T) {
-            const int64_t u = u0 + k;
-            sm[k] = (u >= 0 && u < nsamp) ? __ldg(x0 + k) : (uint8_t)0;
-        }
-#pragma unroll
-        for (int i = 0; i < K; i++) {
-            off[i + 1] = 0;
-            const bool have = c0 + 1 + i < nchan;
-            const uint8_t* xi = X + (int64_t)(have ? c0 + 1 + i : c0) * nsamp + u0 + dmn[i];
-            uint8_t* wi = sm + kET + 48 + i * wstride;
-            for (int k = tid; k < bw[i] + 4; k += kS1T) {
-                const int64_t u = u0 + dmn[i] + k;
-                wi[k] = (have && u >= 0 && u < nsamp) ? __ldg(xi + k) : (uint8_t)0;
+        // the same 16-byte pieces; those outside the row (or of a missing channel) are
+        // zero, the one that straddles an end is copied byte by byte
+        auto edge = [&](uint8_t* w, int c, int64_t u, int bytes) {
+            const bool have = c < nchan;
+            const uint8_t* x = X + (int64_t)(have ? c : c0) * nsamp + u;
+            const int o = (int)((uintptr_t)x & 15);
+            const int n = (o + bytes + 15) >> 4;
+            for (int k = tid; k < n; k += kS1T) {
+                const int64_t s = u - o + 16 * k;
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (have && s >= 0 && s + 16 <= nsamp) v = __ldg(reinterpret_cast<const uint4*>(x - o) + k);
+                reinterpret_cast<uint4*>(w)[k] = v;
+                if (have && s < nsamp && s + 16 > 0 && (s < 0 || s + 16 > nsamp))
+                    for (int i = (int)max((int64_t)0, -s); i < (int)min((int64_t)16, nsamp - s); i++)
+                        w[16 * k + i] = __ldg(x - o + 16 * k + i);
             }
-        }
+            return o;
+        };
+        off[0] = edge(sm, c0, u0, kET + 4);
+#pragma unroll
+        for (int i = 0; i < K; i++) off[i + 1] = edge(sm + kET + 48 + i * wstride, c0 + 1 + i, u0 + dmn[i], bw[i] + 4);
     }
-    __syncthreads();
+    int nrec = list_records();  // its barriers also complete the windows
     // thread tid takes the 4-sample words w = tid + 256 j (j < 4) of the block:
     // consecutive lanes read consecutive shared words (no bank conflicts) and
     // store consecutive 8-byte pieces of a row
@@ -209,34 +234,24 @@ k_group_rows(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int4
     int prev[K];
 #pragma unroll
     for (int i = 0; i < K; i++) prev[i] = INT32_MIN;
-    // a row's record is read while the row before it is summed (groups of 2 have too
-    // little to sum for that: there the loads of several rows overlap as they are)
-    constexpr bool AHEAD = G > 2;
-    int4 ri = __ldg(rinfo + pi.x + kbeg);
-    int64_t ro = __ldg(rowoff + pi.x + kbeg);
-    int dl[K];
-#pragma unroll
-    for (int i = 0; i < K; i++) dl[i] = __ldg(rdelta + (int64_t)(pi.x + kbeg) * K + i);
-    for (int k = kbeg; k < kend; k++) {
-        if (!AHEAD) {
-            const int2 r2 = __ldg(reinterpret_cast<const int2*>(rinfo + pi.x + k));
-            ri.x = r2.x;
-            ri.y = r2.y;
-            ro = __ldg(rowoff + pi.x + k);
-            dl[0] = __ldg(rdelta + pi.x + k);
+    for (int kb = 0, k = 0; kb < pi.y; k++) {
+        if (k == nrec) {  // the same in every thread: the next pass
+            kb += kS1T;
+            k = -1;
+            nrec = 0;
+            if (kb < pi.y) {
+                __syncthreads();  // every thread is done with the records before
+                load_records(kb);
+                nrec = list_records();
+            }
+            continue;
         }
-        const int start = ri.x, len = ri.y - dshort;
-        uint16_t* row = PS + ro;
+        const int rec = s_list[k];
+        const int start = s_ri[rec].x, len = s_ri[rec].y;
+        uint16_t* row = PS + s_ro[rec];
         int d[K];
 #pragma unroll
-        for (int i = 0; i < K; i++) d[i] = dl[i];
-        if (AHEAD && k + 1 < kend) {
-            ri = __ldg(rinfo + pi.x + k + 1);
-            ro = __ldg(rowoff + pi.x + k + 1);
-#pragma unroll
-            for (int i = 0; i < K; i++) dl[i] = __ldg(rdelta + (int64_t)(pi.x + k + 1) * K + i);
-        }
-        if (AHEAD && (start >= e0 + kET || start + len <= e0)) continue;
+        for (int i = 0; i < K; i++) d[i] = s_dl[i][rec];
         bool change = false;  // a delay so far differs from the last summed row's (the same in every thread)
         uint32_t l[4], h[4];
 #pragma unroll
@@ -632,13 +647,20 @@ size_t pair_budget()
 // build: 24.8 / 17.0 / 13.2 ms of shared loads (17.3 / 17.0 / 17.2 ms of window
 // copies, L2 to shared memory) for groups of 2 / 3 / 4 channels in blocks of 15 DM
 // rows; both together 24.8 / 19.2 / 18.8 ms, and in blocks of 30 rows, which copy
-// 0.65 / 0.68 / 0.72 of the bytes, 25.0 / 17.2 / 14.3 ms.  Stage 1 moves row bytes +
-// input at about 6.6 TB/s of HBM; the channel tile kernel adds about 17.7 T samples/s.
+// 0.65 / 0.68 / 0.72 of the bytes, 25.0 / 17.2 / 14.3 ms.  The rates below are fitted
+// to both stages' times of 70 plans (128 to 4096 channels, 64 to 1495 DMs, 11 k to
+// 215 k outputs; the fit's errors are 6 and 7 %); the channel tile kernel adds about
+// 17.7 T samples/s.
 constexpr double kTileAddps = 17.7e12;
-constexpr double kBlockStart = 4.5e-6;  // a stage-2 block's first copies and its stores, per 15 DM rows
-constexpr double kRowRate = 6.5e12;
-inline double load_rate(int G) { return G == 4 ? 33.6e12 : G == 3 ? 34.7e12 : 35.7e12; }
-inline double copy_rate(int G) { return G == 4 ? 7.0e12 : 7.6e12; }
+constexpr double kBlockStart = 4.6e-6;  // a stage-2 block's first copies and its stores, per 15 DM rows
+constexpr double kBlockNorm = 6.4;      // how far a block's loads and copies overlap
+constexpr double kRowRead = 4.7e12;     // stage 2: rows from HBM, overlapping the blocks (6.2-norm)
+inline double load_rate(int G) { return G == 4 ? 37.1e12 : G == 3 ? 37.2e12 : 37.5e12; }
+inline double copy_rate(int G) { return G == 4 ? 6.8e12 : G == 3 ? 7.2e12 : 7.7e12; }
+// stage 1: a launch, a block of the whole GPU, a row's part of one block (8 KB
+// written), and a row of the group that has the most, one after another
+constexpr double kRowsLaunch = 5.6e-6, kRowPart = 1.1e-9, kRowSerial = 0.37e-6;
+inline double rows_block(int G) { return G == 4 ? 8.1e-9 : G == 3 ? 5.0e-9 : 2.9e-9; }
 inline double row_rate(int G) { return G == 4 ? 5.2e12 : G == 3 ? 6.2e12 : 6.5e12; }
 
 }  // namespace
@@ -910,7 +932,7 @@ static int upload_groups(af_pair_tables* T)
     up(&T->d_perm, T->h_perm);
     for (auto& l : T->lay)
         if (e != cudaSuccess || (e = cudaMalloc(&l.d_pinfo, (size_t)T->np * sizeof(int4))) != cudaSuccess ||
-            (e = cudaMalloc(&l.d_rinfo, (size_t)T->nrows * sizeof(int4))) != cudaSuccess ||
+            (e = cudaMalloc(&l.d_rinfo, (size_t)T->nrows * sizeof(int2))) != cudaSuccess ||
             (e = cudaMalloc(&l.d_rowoff, (size_t)T->nrows * 8)) != cudaSuccess ||
             (e = cudaMalloc(&l.d_soff, T->h_srow.size() * 8)) != cudaSuccess)
             break;
@@ -1010,7 +1032,8 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
         T->ps_bytes = (size_t)need * 2;
     }
     std::vector<int64_t> rowoff(T->nrows), soff(T->h_srow.size());
-    std::vector<int4> pinfo(T->np), rinfo(T->nrows);
+    std::vector<int4> pinfo(T->np);
+    std::vector<int2> rinfo(T->nrows);
     int64_t off = 0, maxlen = 0;
     for (int q = 0; q < T->np; q++) {
         const int g0 = T->h_rb[q], g1 = T->h_rb[q + 1];
@@ -1021,9 +1044,8 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
             off += len;
             const int start = T->h_rB[g] - T->h_ub[q];
             end = std::max(end, (int64_t)start + len);
-            rinfo[g] = make_int4(start, (int)len, (int)end, start);
+            rinfo[g] = make_int2(start, (int)len);
         }
-        for (int g = g1 - 2; g >= g0; g--) rinfo[g].w = std::min(rinfo[g].w, rinfo[g + 1].w);
         pinfo[q] = make_int4(g0, g1 - g0, T->h_ub[q], (int)end);
         maxlen = std::max(maxlen, end);
     }
@@ -1034,7 +1056,7 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
         (e = cudaMemcpy(ly.d_soff, soff.data(), soff.size() * 8, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(ly.d_pinfo, pinfo.data(), pinfo.size() * sizeof(int4), cudaMemcpyHostToDevice)) !=
             cudaSuccess ||
-        (e = cudaMemcpy(ly.d_rinfo, rinfo.data(), rinfo.size() * sizeof(int4), cudaMemcpyHostToDevice)) != cudaSuccess)
+        (e = cudaMemcpy(ly.d_rinfo, rinfo.data(), rinfo.size() * sizeof(int2), cudaMemcpyHostToDevice)) != cudaSuccess)
         return af_cuda_check(e, "pair layout");
     ly.L = L;
     ly.maxlen = maxlen;
@@ -1042,33 +1064,38 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
 }
 
 // Predicted time (s) of group rows T in time blocks of L outputs on nout
-// outputs.  A stage-2 block takes the 6-norm of its shared loads' and its window
+// outputs.  A stage-2 block takes the 6.4-norm of its shared loads' and its window
 // copies' times at the rates above (they overlap, not quite), and a launch whole
 // waves of one block per SM: blocks of 30 DM rows are faster by up to a quarter
 // on many waves and slower where 15 rows fill the last wave better (2128 channels,
-// 609 DMs, 22 tiles: 902 blocks of 15 in 0.62 ms, 462 of 30 in 0.75 ms).
+// 609 DMs, 22 tiles: 902 blocks of 15 in 0.62 ms, 462 of 30 in 0.75 ms).  Stage 1
+// is its blocks and the row pieces they write, or, where they are few, the group
+// with the most rows.
 static double rows_cost(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L)
 {
     const double nsm = p->num_sms > 0 ? p->num_sms : 152;
     const double loads = 2.0 * kPNW * T->dpw * T->np * 64.0 * kPMG / (load_rate(T->G) / nsm);
     const double copies = T->copy_per_tile / T->nblk / (copy_rate(T->G) / nsm);
-    const double block = std::pow(std::pow(loads, 6) + std::pow(copies, 6), 1.0 / 6) + kBlockStart * T->dpw;
+    const double block = std::pow(std::pow(loads, kBlockNorm) + std::pow(copies, kBlockNorm), 1.0 / kBlockNorm) + kBlockStart * T->dpw;
     auto waves = [&](int64_t outs) {
         return std::ceil((double)((outs + kPTTE - 1) / kPTTE) * T->nblk / nsm);
     };
     const int64_t full = nout / L, rest = nout - full * L;
-    const double s2 = block * ((double)full * waves(L) + (rest > 0 ? waves(rest) : 0.0));
-    // stage 1: HBM, and a block's window loads (1 ns per channel and block of the whole GPU)
+    const double times = (double)full + (rest > 0 ? (double)rest / L : 0.0);
+    const double s2 = std::pow(std::pow(block * ((double)full * waves(L) + (rest > 0 ? waves(rest) : 0.0)), 6.2) +
+                                   std::pow(times * 2.0 * (double)rows_elems(T, L) / kRowRead, 6.2),
+                               1.0 / 6.2);
     double blocks1 = 0;
+    int most = 0;
     for (int q = 0; q < T->np; q++) {
         int64_t end = 0;
         for (int g = T->h_rb[q]; g < T->h_rb[q + 1]; g++)
             end = std::max(end, (int64_t)T->h_rB[g] - T->h_ub[q] + row_len(T, g, L));
         blocks1 += (double)((end + kET - 1) / kET);
+        most = std::max(most, T->h_rb[q + 1] - T->h_rb[q]);
     }
-    const double times = (double)full + (rest > 0 ? (double)rest / L : 0.0);
-    const double s1 = times * (2.0 * (double)rows_elems(T, L) / kRowRate + blocks1 * 4e-9 * T->G) +
-                      (double)p->nchan * (double)(nout + p->dmax) / kRowRate + 8e-6;
+    const double all = blocks1 * rows_block(T->G) + (double)rows_elems(T, L) / kET * kRowPart;
+    const double s1 = times * (kRowsLaunch + std::cbrt(std::pow(all, 3) + std::pow(most * kRowSerial, 3)));
     return s1 + s2;
 }
 
@@ -1113,11 +1140,11 @@ static int pairs_release(af_pair_tables* T)
 static int pairs_choose(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L)
 {
     *L = 0;
-    // two predictions: the block model's fastest set is taken where it beats by 3.5 %
-    // (over 22 plans its error on the ratio of two sets was below that where it would
-    // have chosen wrongly) the set of 15-row blocks that moves the fewest bytes
-    int best = -1, plain = -1;
-    double best_t = 0, plain_t = 0, plain_model = 0;
+    // the set the model predicts fastest: over 70 plans 0.1 % slower on average than
+    // the set that measured fastest, at most 3.2 % (the set of 15-row blocks that moves
+    // the fewest bytes, over 47 of them: 6.6 % and 29 %)
+    int best = -1;
+    double best_t = 0;
     int64_t Ls[6] = {};
     bool beats = false;
     for (int k = 0; k < 6; k++) {
@@ -1126,19 +1153,13 @@ static int pairs_choose(af_plan_t p, int64_t nout, bool allow_larger, size_t max
         Ls[k] = block_len(T, nout, max_bytes);
         if (Ls[k] <= 0) continue;
         beats = beats || rows_beat_tile(p, T, nout, Ls[k]);
-        const double t = rows_cost(p, T, nout, Ls[k]), r = rows_rate_cost(p, T, nout, Ls[k]);
+        const double t = rows_cost(p, T, nout, Ls[k]);
         if (best < 0 || t < best_t) {
             best = k;
             best_t = t;
         }
-        if (T->dpw == 1 && (plain < 0 || r < plain_t)) {
-            plain = k;
-            plain_t = r;
-            plain_model = t;
-        }
     }
     if (best < 0) return -1;
-    if (plain >= 0 && best_t > 0.965 * plain_model) best = plain;
     const bool tile = p->tile.ns1 > 0;  // else the one-thread-per-output kernel
     if (!p->force_pairs && tile && !beats) return -1;
     *L = Ls[best];
