@@ -342,12 +342,13 @@ __global__ void __launch_bounds__(kThreads) k_tconv(const typename Op::Args args
                     afptx::fence_proxy_async();
                     afptx::mbar_arrive(full0 + 8 * s);
                 }
-                op.unpool_finish(t, lane, acc);
+                op.unpool_finish(t, lane, acc, xv);
             }
             ok = afumma::wait_or_abort(tfull0, 0u, abort) && ok;
             if (!epi_sync_any(!ok || *abort)) {
                 afumma::fence_after_sync();
-                op.final(tmem, quarter, lane);
+                if constexpr (Op::UNPOOL) op.unpool_add(tid - 64, xv);
+                op.final(sm + Op::RB, tmem, quarter, lane);
             }
         }
     }
@@ -427,7 +428,7 @@ struct ConvOp {
                              afumma::smem_desc(res + (uint32_t)s * 2 * LBO_B, LBO_B, 128), idesc, s != 0);
         }
     }
-    __device__ void final(uint32_t, int, int) const {}
+    __device__ void final(uint8_t*, uint32_t, int, int) const {}
     // Thread = tile row r = 32 quarter + lane, pixel (y0 + r / W, r % W).
     __device__ void epilogue(int tile, uint32_t tmem, int quarter, int lane, float* xv, uint32_t* xq) const
     {
@@ -708,16 +709,22 @@ struct WgradOp {
             *reinterpret_cast<uint4*>(st + zb * PLANE_Z + (r * W + x) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
-    // The bias gradient: the lanes of a warp with one block reduce, then one
-    // atomic per channel and warp.
-    __device__ void unpool_finish(int t, int lane, float (&acc)[8]) const
+    // The bias gradient: the lanes of a warp with one block reduce into xv
+    // [4 warps][COUT]; after a barrier, one coalesced addition per block (one per
+    // warp and channel block kept the L2 busy for 15 of the kernel's 38 us on 256
+    // images).
+    __device__ void unpool_finish(int t, int lane, float (&acc)[8], float* xv) const
     {
 #pragma unroll
         for (int j = 0; j < 8; j++) {
 #pragma unroll
             for (int o = 16; o >= ZB; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-            if (lane < ZB) atomicAdd(a.db + (t % ZB) * 8 + j, acc[j]);  // t % ZB = lane % ZB
+            if (lane < ZB) xv[(t >> 5) * COUT + lane * 8 + j] = acc[j];  // t % ZB = lane % ZB
         }
+    }
+    __device__ void unpool_add(int t, const float* xv) const
+    {
+        if (t < COUT) atomicAdd(a.db + t, xv[t] + xv[COUT + t] + xv[2 * COUT + t] + xv[3 * COUT + t]);
     }
     // copies 0 .. 3 CB - 1: the shifted copies of X; then one per dZ block
     __device__ void copy(int c, uint32_t st, int tile, uint32_t bar) const
@@ -772,9 +779,20 @@ struct WgradOp {
         }
     }
     __device__ void epilogue(int, uint32_t, int, int, float*, uint32_t*) const {}
-    // Row o = 32 quarter + lane of the accumulator: its columns into grad.
-    __device__ void final(uint32_t tmem, int quarter, int lane) const
+    // The accumulator into grad by way of shared memory (the ring is free by now):
+    // laid out there as the gradient is, rows of FROW floats, then added in
+    // runs of consecutive addresses.  A block's sums meet every other block's at
+    // the same addresses, and the L2 takes the additions to one 32-byte sector
+    // one after another: straight from the accumulator (a lane per row, a float
+    // at a time) they took most of the kernels' time on 256 images (third layer
+    // 61 us, 17 so; first layer 61 us, 38 so, 21 with the bias gradient below).
+    static constexpr int FROW = CIN * 9 + (CIN > 2 ? 4 : 0);  // pads to an odd number of 16-byte pieces
+    static_assert((uint32_t)COUT * FROW * 4 <= (uint32_t)NS * SSTAGE, "the gradient fits the ring");
+    __device__ void final(uint8_t* ring, uint32_t tmem, int quarter, int lane) const
     {
+        float* F = reinterpret_cast<float*>(ring);
+        const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16);
+        const int o = 32 * quarter + lane;
         if constexpr (SWAP) {
             // row m = 32 quarter + lane: row shift j = m / 8 of a block's copies
             // (tap dy = j % (R + 2), dx = j / (R + 2)), channel m % 8; columns:
@@ -782,7 +800,6 @@ struct WgradOp {
             const int m = 32 * quarter + lane, j = m >> 3, dx = j / (R + 2), dy = j - dx * (R + 2);
             const bool real = dy < 3 && dx < 3;
             const int t = 3 * dy + dx;
-            const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16);
 #pragma unroll 1
             for (int k = 0; k < NMMA; k++)
 #pragma unroll 1
@@ -793,40 +810,39 @@ struct WgradOp {
                     if (!real) continue;
                     const int i = 8 * k + (m & 7);
 #pragma unroll
-                    for (int jj = 0; jj < 16; jj++)
-                        atomicAdd(a.grad + ((int64_t)(c0 + jj) * 9 + t) * CIN + i, __uint_as_float(v[jj]));
+                    for (int jj = 0; jj < 16; jj++) F[(c0 + jj) * FROW + t * CIN + i] = __uint_as_float(v[jj]);
                 }
-            return;
-        }
-        if (32 * quarter >= COUT) return;  // warp-uniform: no real rows in this quarter
-        const int o = 32 * quarter + lane;
-        const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16);
+        } else if (32 * quarter < COUT) {  // warp-uniform: real rows in this quarter
 #pragma unroll 1
-        for (int c0 = 0; c0 < NCOL; c0 += 16) {
-            uint32_t v[16];
-            afumma::ld_32x32b_x16(taddr + (uint32_t)c0, v);
-            afumma::wait_ld();
-            if (o >= COUT) continue;
-#pragma unroll
-            for (int jj = 0; jj < 16; jj++) {
-                const int col = c0 + jj;
-                int t, i;
+            for (int c0 = 0; c0 < NCOL; c0 += 16) {
+                uint32_t v[16];
+                afumma::ld_32x32b_x16(taddr + (uint32_t)c0, v);
+                afumma::wait_ld();
+                if (o >= COUT) continue;
                 if constexpr (CB == 1) {
-                    const int dy = col >> 3, dx = (col & 7) >> 1;
-                    i = col & 1;
-                    if (dy >= 3 || dx >= 3) continue;
-                    t = 3 * dy + dx;
-                } else if constexpr (TAPN) {
-                    const int k = col / NPM, r = col - k * NPM, j = r >> 3, dx = j / (R + 2), dy = j - dx * (R + 2);
-                    i = 8 * k + (r & 7);
-                    if (dy >= 3 || dx >= 3 || i >= CIN) continue;
-                    t = 3 * dy + dx;
+                    // columns 8 dy + 2 dx + c
+#pragma unroll
+                    for (int jj = 0; jj < 16; jj++) {
+                        const int dy = (c0 + jj) >> 3, q = jj & 7;
+                        if (dy < 3 && q < 6) F[o * FROW + 6 * dy + q] = __uint_as_float(v[jj]);
+                    }
                 } else {
-                    t = col / NPM;
-                    i = col - t * NPM;
+                    // columns t CIN + i, the gradient's own order
+                    static_assert(!TAPN || CB == 1, "taps along N only here");
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        *reinterpret_cast<uint4*>(F + o * FROW + c0 + 4 * q) =
+                            make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
                 }
-                atomicAdd(a.grad + ((int64_t)o * 9 + t) * CIN + i, __uint_as_float(v[jj]));
             }
+        }
+        epi_sync();
+        constexpr int ROW4 = CIN > 2 ? CIN * 9 / 4 : 1, TOTAL = CIN > 2 ? COUT * ROW4 : COUT * FROW / 4;
+        static_assert(CIN > 2 ? CIN * 9 % 4 == 0 : COUT * FROW % 4 == 0, "whole 16-byte pieces");
+        for (int e = 32 * quarter + lane; e < TOTAL; e += 128) {
+            const int row = CIN > 2 ? e / ROW4 : 0, q = e - row * ROW4;
+            const float4 v = *reinterpret_cast<const float4*>(F + (CIN > 2 ? row * FROW + 4 * q : 4 * e));
+            atomicAdd(reinterpret_cast<float4*>(a.grad) + e, v);
         }
     }
 };
@@ -839,29 +855,48 @@ struct WgradOp {
 // W[o][8 - t][i].  cbk = channel blocks of K per tap (1: the first layer's
 // column-expanded input, two K steps of rows (0, 1) and (1, 2), the repeated
 // row 1 with zero weights).
-__global__ void k_tpack(const float* __restrict__ w, int cin, int cout, int cbk, int nrows, int dgrad, int total,
-                        __nv_bfloat16* __restrict__ out)
+// One launch packs every layer that needs it and clears the gradients (five
+// packs and two clears of about 3 us each, and the gaps between them, were 20
+// of a 219-us training step of 256 images).
+struct PackJob {
+    const float* w;      // NULL: clear out (total floats)
+    void* out;
+    int cin, cout, cbk, nrows, dgrad, total, first;  // first: the job's first block
+};
+constexpr int kMaxPack = 6;
+struct PackJobs {
+    PackJob job[kMaxPack];
+    int n;
+};
+__global__ void __launch_bounds__(256) k_tpack(const PackJobs jobs)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= total) return;
-    const int k = e & 7, row = (e >> 3) % nrows, kc = (e / (8 * nrows)) & 1, s = e / (16 * nrows);
+    int j = 0;
+    while (j + 1 < jobs.n && (int)blockIdx.x >= jobs.job[j + 1].first) j++;
+    const PackJob& p = jobs.job[j];
+    const int e = ((int)blockIdx.x - p.first) * 256 + (int)threadIdx.x;
+    if (e >= p.total) return;
+    if (!p.w) {
+        reinterpret_cast<float*>(p.out)[e] = 0.f;
+        return;
+    }
+    const int k = e & 7, row = (e >> 3) % p.nrows, kc = (e / (8 * p.nrows)) & 1, s = e / (16 * p.nrows);
     int t, c;
-    if (cbk == 1) {
+    if (p.cbk == 1) {
         // column-expanded input: K half kc of step s is row dy = s + kc (step 1's
         // first half repeats row 1 with zero weights), channel k = (dx, c)
         const int dy = s + kc;
         t = (s == 1 && kc == 0) || k >= 6 ? -1 : 3 * dy + (k >> 1);
         c = k & 1;
     } else {
-        t = s / (cbk / 2);
-        c = (2 * (s % (cbk / 2)) + kc) * 8 + k;
+        t = s / (p.cbk / 2);
+        c = (2 * (s % (p.cbk / 2)) + kc) * 8 + k;
     }
     float v = 0.f;
     if (t >= 0) {
-        if (!dgrad && c < cin) v = w[((int64_t)row * 9 + t) * cin + c];
-        if (dgrad && c < cout) v = w[((int64_t)c * 9 + (8 - t)) * cin + row];
+        if (!p.dgrad && c < p.cin) v = p.w[((int64_t)row * 9 + t) * p.cin + c];
+        if (p.dgrad && c < p.cout) v = p.w[((int64_t)c * 9 + (8 - t)) * p.cin + row];
     }
-    out[e] = __float2bfloat16(v);
+    reinterpret_cast<__nv_bfloat16*>(p.out)[e] = __float2bfloat16(v);
 }
 
 // ------------------------------------------------------------ host side
@@ -938,13 +973,27 @@ size_t nn_tpack_bytes(int layer, int dgrad)
     return layer == 1 ? Dg1::STEPS * 2 * Dg1::LBO_B : layer == 2 ? Dg2::STEPS * 2 * Dg2::LBO_B : 0;
 }
 
-int nn_tpack(int layer, int dgrad, const float* w, __nv_bfloat16* out, cudaStream_t s)
+int nn_tpack(const float* const (&w)[3], __nv_bfloat16* const (&fwd)[3], __nv_bfloat16* const (&dgrad)[3],
+             float* clear, int64_t nclear, cudaStream_t s)
 {
-    if (layer < 0 || layer > 2 || (dgrad && layer == 0)) return af_set_error(AF_EINVAL, "conv pack: layer %d", layer);
-    const int cin = kCin[layer], cout = kCout[layer];
-    const int cbk = dgrad ? cout / 8 : (cin < 8 ? 1 : cin / 8), nrows = dgrad ? cin : cout;  // cbk 1: expanded
-    const int total = (int)(nn_tpack_bytes(layer, dgrad) / 2);
-    k_tpack<<<(total + 255) / 256, 256, 0, s>>>(w, cin, cout, cbk, nrows, dgrad, total, out);
+    PackJobs jobs;
+    jobs.n = 0;
+    int blocks = 0;
+    auto add = [&](PackJob p) {
+        p.first = blocks;
+        blocks += (p.total + 255) / 256;
+        jobs.job[jobs.n++] = p;
+    };
+    for (int l = 0; l < 3; l++) {
+        const int cin = kCin[l], cout = kCout[l];
+        if (fwd[l])  // cbk 1: expanded
+            add(PackJob{w[l], fwd[l], cin, cout, cin < 8 ? 1 : cin / 8, cout, 0, (int)(nn_tpack_bytes(l, 0) / 2), 0});
+        if (l > 0 && dgrad[l])
+            add(PackJob{w[l], dgrad[l], cin, cout, cout / 8, cin, 1, (int)(nn_tpack_bytes(l, 1) / 2), 0});
+    }
+    if (clear) add(PackJob{nullptr, clear, 0, 0, 0, 1, 0, (int)nclear, 0});
+    if (!jobs.n) return AF_OK;
+    k_tpack<<<blocks, 256, 0, s>>>(jobs);
     return af_cuda_check(cudaGetLastError(), "conv pack");
 }
 
@@ -987,7 +1036,8 @@ int nn_tconv_dgrad(int layer, const __nv_bfloat16* dz, int n, const __nv_bfloat1
 int nn_tconv_wgrad(int layer, const __nv_bfloat16* dz, const __nv_bfloat16* x, int n, float* grad, int* err,
                    cudaStream_t s)
 {
-    if (layer < 0 || layer > 2 || n < 1 || !x || !dz || ((uintptr_t)x & 15) || ((uintptr_t)dz & 15))
+    if (layer < 0 || layer > 2 || n < 1 || !x || !dz || ((uintptr_t)x & 15) || ((uintptr_t)dz & 15) ||
+        ((uintptr_t)grad & 15))
         return af_set_error(AF_EINVAL, "conv weight gradient: layer %d / alignment", layer);
     const int W = kW[layer], tiles = n * (W / (128 / W));
 #define AF_TW(L, Op)                                                      \
@@ -1005,7 +1055,8 @@ int nn_tconv_wgrad(int layer, const __nv_bfloat16* dz, const __nv_bfloat16* x, i
 int nn_tconv_wgrad_unpool(const __nv_bfloat16* dp, const uint8_t* idx, const __nv_bfloat16* x, int n, float* grad,
                           float* db, int* err, cudaStream_t s)
 {
-    if (n < 1 || !x || !dp || !idx || !db || ((uintptr_t)x & 15) || ((uintptr_t)dp & 15) || ((uintptr_t)idx & 7))
+    if (n < 1 || !x || !dp || !idx || !db || ((uintptr_t)x & 15) || ((uintptr_t)dp & 15) || ((uintptr_t)idx & 7) ||
+        ((uintptr_t)grad & 15))
         return af_set_error(AF_EINVAL, "conv weight gradient (unpool): argument / alignment");
     const int W = kW[0], tiles = n * (W / (128 / W));
     typename Wg0u::Args a{x, nullptr, grad, n, err, dp, idx, db};

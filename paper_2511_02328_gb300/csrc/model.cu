@@ -65,14 +65,14 @@ struct af_model_s {
     __nv_bfloat16* d_da[NL + 1] = {};  // gradients w.r.t. d_a[l] (l >= 1)
     __nv_bfloat16* d_dz[NL] = {};      // gradients w.r.t. the pre-pool ReLU outputs (layers 1, 2)
     float* d_logits = nullptr;
-    float* d_loss = nullptr;
+    float* d_loss = nullptr;           // after d_grads, cleared with them
     int* d_err = nullptr;              // raised by a bounded tensor-core wait that ran out
     __nv_bfloat16* d_cut = nullptr;    // cut-outs for af_classify
     int umma_min = 0;                  // inference batches of at least this size use the tensor-core layers
     // d_wt holds the packed form of the current d_params (set by a forward pass
     // that packed them, on the stream where packed_ev is recorded; cleared by
     // every call that changes the parameters)
-    bool packed = false;
+    bool packed = false, packed_d = false;  // d_wt, d_wd
     cudaEvent_t packed_ev = nullptr;
 };
 
@@ -95,7 +95,6 @@ static void free_model(af_model_t m)
     }
     cudaFree(m->d_err);
     cudaFree(m->d_logits);
-    cudaFree(m->d_loss);
     cudaFree(m->d_cut);
     if (m->packed_ev) cudaEventDestroy(m->packed_ev);
     delete m;
@@ -156,7 +155,8 @@ try {
         if (e == cudaSuccess) e = cudaMalloc((void**)p, bytes);
     };
     A(&m->d_params, off * 4);
-    A(&m->d_grads, off * 4);
+    A(&m->d_grads, (off + 1) * 4);
+    m->d_loss = m->d_grads + off;
     A(&m->d_m, off * 4);
     A(&m->d_v, off * 4);
     for (int l = 0; l < NL; l++) {
@@ -171,7 +171,6 @@ try {
     }
     A(&m->d_err, 16);
     A(&m->d_logits, (size_t)n * 2 * 4);
-    A(&m->d_loss, 16);
     A(&m->d_cut, (size_t)n * 64 * 64 * 2 * 2);
     if (e == cudaSuccess) e = cudaMemset(m->d_err, 0, 16);
     if (e == cudaSuccess) e = cudaMemset(m->d_m, 0, off * 4);
@@ -240,7 +239,7 @@ static int copy_params(af_model_t m, float* dst, const float* src, int64_t n, cu
 extern "C" int af_model_set_params(af_model_t m, const float* h, int64_t n)
 try {
     if (!m || !h) return af_set_error(AF_EINVAL, "af_model_set_params: NULL argument");
-    m->packed = false;
+    m->packed = m->packed_d = false;
     return copy_params(m, m->d_params, h, n, cudaMemcpyHostToDevice, "af_model_set_params");
 } catch (...) {
     return af_host_exception("af_model_set_params");
@@ -272,14 +271,25 @@ static int forward(af_model_t m, const __nv_bfloat16* x, int n, const int32_t* y
         return nn_forward_fused(x, n, P + m->L[0].woff, P + m->L[0].boff, P + m->L[1].woff, P + m->L[1].boff,
                                 P + m->L[2].woff, P + m->L[2].boff, P + m->fw_off, P + m->fb_off, logits, prob,
                                 s);
-    if (!m->packed) {  // the parameters changed since the last packing
-        for (int l = 0; l < NL; l++)
-            if (int rc = nn_tpack(l, 0, P + m->L[l].woff, m->d_wt[l], s)) return rc;
+    // what the parameters' last change left unpacked, and clear gradients, in one launch
+    const bool pack = !m->packed, pack_d = y && !m->packed_d;
+    if (m->packed || m->packed_d) AF_CUDA(cudaStreamWaitEvent(s, m->packed_ev, 0));  // on this or another stream
+    if (pack || y) {
+        const float* w[NL];
+        __nv_bfloat16 *fwd[NL], *dgrad[NL];
+        for (int l = 0; l < NL; l++) {
+            w[l] = P + m->L[l].woff;
+            fwd[l] = pack ? m->d_wt[l] : nullptr;
+            dgrad[l] = pack_d ? m->d_wd[l] : nullptr;
+        }
+        // the loss follows the gradients
+        if (int rc = nn_tpack(w, fwd, dgrad, y ? m->d_grads : nullptr, m->nparams + 1, s)) return rc;
+    }
+    if (pack || pack_d) {
         if (!m->packed_ev) AF_CUDA(cudaEventCreateWithFlags(&m->packed_ev, cudaEventDisableTiming));
         AF_CUDA(cudaEventRecord(m->packed_ev, s));
         m->packed = true;
-    } else {
-        AF_CUDA(cudaStreamWaitEvent(s, m->packed_ev, 0));  // packed on this or another stream
+        m->packed_d = m->packed_d || pack_d;
     }
     const __nv_bfloat16* a = x;  // the first layer expands its columns itself
     for (int l = 0; l < NL; l++) {
@@ -288,10 +298,6 @@ static int forward(af_model_t m, const __nv_bfloat16* x, int n, const int32_t* y
                                   s))
             return rc;
         a = m->d_a[l + 1];
-    }
-    if (y) {
-        AF_CUDA(cudaMemsetAsync(m->d_loss, 0, 4, s));
-        AF_CUDA(cudaMemsetAsync(m->d_grads, 0, m->nparams * 4, s));
     }
     return nn_head(m->d_a[NL], n, P + m->fw_off, P + m->fb_off, logits, prob, y, m->d_loss,
                    m->d_grads + m->fw_off, m->d_grads + m->fb_off, m->d_da[NL], s);
@@ -310,10 +316,7 @@ static int backward(af_model_t m, const __nv_bfloat16* x, int n, cudaStream_t s)
             return rc;
         const __nv_bfloat16* a = l ? m->d_a[l] : x;
         if (int rc = nn_tconv_wgrad(l, m->d_dz[l], a, n, m->d_grads + L.woff, m->d_err, s)) return rc;
-        if (l > 0) {
-            if (int rc = nn_tpack(l, 1, m->d_params + L.woff, m->d_wd[l], s)) return rc;
-            if (int rc = nn_tconv_dgrad(l, m->d_dz[l], n, m->d_wd[l], m->d_da[l], m->d_err, s)) return rc;
-        }
+        if (int rc = nn_tconv_dgrad(l, m->d_dz[l], n, m->d_wd[l], m->d_da[l], m->d_err, s)) return rc;
     }
     return AF_OK;
 }
@@ -356,7 +359,7 @@ try {
     if (!(lr > 0.0f) || !isfinite(lr)) return af_set_error(AF_EINVAL, "af_train_step: bad learning rate");
     if (int rc = af_model_backward(m, d_x, d_y, n, d_loss, stream)) return rc;
     m->step++;
-    m->packed = false;
+    m->packed = m->packed_d = false;
     return nn_adam(m->d_params, m->d_grads, m->d_m, m->d_v, m->nparams, lr, m->step, (cudaStream_t)stream);
 } catch (...) {
     return af_host_exception("af_train_step");
@@ -462,7 +465,7 @@ try {
     const size_t got = fread(buf.data(), 4, buf.size(), f);
     fclose(f);
     if (got != buf.size()) return af_set_error(AF_EINVAL, "af_model_load: truncated checkpoint");
-    m->packed = false;
+    m->packed = m->packed_d = false;
     AF_CUDA(cudaMemcpy(m->d_params, buf.data(), m->nparams * 4, cudaMemcpyHostToDevice));
     AF_CUDA(cudaMemcpy(m->d_m, buf.data() + m->nparams, m->nparams * 4, cudaMemcpyHostToDevice));
     AF_CUDA(cudaMemcpy(m->d_v, buf.data() + 2 * m->nparams, m->nparams * 4, cudaMemcpyHostToDevice));

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "internal.h"
 #include "nn.h"
 
@@ -76,48 +78,98 @@ __global__ void __launch_bounds__(256) k_pool_back(const __nv_bfloat16* __restri
 // channel-blocked: channel c at block c / 8, lane c % 8),
 // logits = g fw^T + fb, softmax; with labels, the mean cross-entropy and its
 // gradients (dfw, dfb accumulated, da3 written as bf16).
-__global__ void k_head(const __nv_bfloat16* __restrict__ a3, int n, const float* __restrict__ fw,
-                       const float* __restrict__ fb, float* __restrict__ logits, float* __restrict__ prob,
-                       const int32_t* __restrict__ y, float* __restrict__ loss, float* __restrict__ dfw,
-                       float* __restrict__ dfb, __nv_bfloat16* __restrict__ da3)
+//
+// A block of 256 threads takes kHeadS samples a pass, 64 threads (one per
+// channel) each, and adds its share of the parameter gradients once at the end:
+// the L2 takes additions to one address one after another, so one set of 131 per
+// sample took 40 us for 4096 samples (18.7 so; 256 samples 7.7 and 5.6 us).
+// Activations come and their gradients go in 16-byte pieces by way of shared
+// memory.
+constexpr int kHeadS = 4;
+constexpr int kHeadRow = 64 * 8 + 8;  // elements of a channel block in shared memory, padded against bank conflicts
+__global__ void __launch_bounds__(64 * kHeadS) k_head(const __nv_bfloat16* __restrict__ a3, int n,
+                                                      const float* __restrict__ fw, const float* __restrict__ fb,
+                                                      float* __restrict__ logits, float* __restrict__ prob,
+                                                      const int32_t* __restrict__ y, float* __restrict__ loss,
+                                                      float* __restrict__ dfw, float* __restrict__ dfb,
+                                                      __nv_bfloat16* __restrict__ da3)
 {
-    const int s = blockIdx.x;
-    const int ch = threadIdx.x;  // 64 threads
-    __shared__ float g[64], lg[2];
-    const __nv_bfloat16* a = a3 + ((int64_t)s * 8 + ch / 8) * 64 * 8 + ch % 8;
-    float acc = 0.f;
-    for (int q = 0; q < 64; q++) acc += __bfloat162float(a[q * 8]);
-    g[ch] = acc / 64.f;
-    __syncthreads();
-    if (ch < 2) {
-        float v = fb[ch];
-        for (int i = 0; i < 64; i++) v += g[i] * fw[ch * 64 + i];
-        lg[ch] = v;
-    }
-    __syncthreads();
-    const float mx = fmaxf(lg[0], lg[1]);
-    const float e0 = expf(lg[0] - mx), e1 = expf(lg[1] - mx);
-    const float p0 = e0 / (e0 + e1), p1 = e1 / (e0 + e1);
-    if (ch == 0) {
-        logits[2 * s] = lg[0];
-        logits[2 * s + 1] = lg[1];
-        if (prob) prob[s] = p1;
+    __shared__ __align__(16) __nv_bfloat16 act[kHeadS][8 * kHeadRow];
+    __shared__ __align__(16) __nv_bfloat16 dv[kHeadS][64];
+    __shared__ float g[kHeadS][64], lg[kHeadS][2], w[128], sum[kHeadS][131];
+    const int grp = threadIdx.x >> 6, ch = threadIdx.x & 63;
+    if (threadIdx.x < 128) w[threadIdx.x] = fw[threadIdx.x];
+    float s0 = 0.f, s1 = 0.f, sl = 0.f, sb0 = 0.f, sb1 = 0.f;  // this thread's shares of dfw, loss, dfb
+    const float inv = 1.f / (float)n;
+    for (int first = blockIdx.x * kHeadS; first < n; first += gridDim.x * kHeadS) {
+        const int s = first + grp;
+        const bool real = s < n;
+        const uint4* src = reinterpret_cast<const uint4*>(a3 + (int64_t)s * 4096);
+        if (real)
+#pragma unroll
+            for (int k = 0; k < 8; k++)  // piece 64 k + ch: channel block k, pixel ch
+                *reinterpret_cast<uint4*>(&act[grp][k * kHeadRow + ch * 8]) = __ldg(src + 64 * k + ch);
+        __syncthreads();
+        if (real) {
+            const __nv_bfloat16* a = &act[grp][(ch / 8) * kHeadRow + ch % 8];
+            float acc = 0.f;
+#pragma unroll 16
+            for (int q = 0; q < 64; q++) acc += __bfloat162float(a[q * 8]);
+            g[grp][ch] = acc / 64.f;
+        }
+        __syncthreads();
+        if (real && ch < 2) {
+            float v = fb[ch];
+#pragma unroll 16
+            for (int i = 0; i < 64; i++) v += g[grp][i] * w[ch * 64 + i];
+            lg[grp][ch] = v;
+        }
+        __syncthreads();
+        if (real) {
+            const float l0 = lg[grp][0], l1 = lg[grp][1], mx = fmaxf(l0, l1);
+            const float e0 = expf(l0 - mx), e1 = expf(l1 - mx);
+            const float p0 = e0 / (e0 + e1), p1 = e1 / (e0 + e1);
+            if (ch == 0) {
+                logits[2 * s] = l0;
+                logits[2 * s + 1] = l1;
+                if (prob) prob[s] = p1;
+            }
+            if (y) {
+                const int lab = y[s];
+                const float d0 = (p0 - (lab == 0 ? 1.f : 0.f)) * inv, d1 = (p1 - (lab == 1 ? 1.f : 0.f)) * inv;
+                if (ch == 0) {
+                    sl += -logf(lab == 1 ? p1 : p0) * inv;
+                    sb0 += d0;
+                    sb1 += d1;
+                }
+                s0 += d0 * g[grp][ch];
+                s1 += d1 * g[grp][ch];
+                dv[grp][ch] = __float2bfloat16((d0 * w[ch] + d1 * w[64 + ch]) / 64.f);
+            }
+        }
+        if (!y) continue;
+        __syncthreads();
+        if (real) {
+            uint4* dst = reinterpret_cast<uint4*>(da3 + (int64_t)s * 4096);
+#pragma unroll
+            for (int k = 0; k < 8; k++) dst[64 * k + ch] = *reinterpret_cast<const uint4*>(&dv[grp][8 * k]);
+        }
     }
     if (!y) return;
-    const int lab = y[s];
-    const float inv = 1.f / (float)n;
-    const float d0 = (p0 - (lab == 0 ? 1.f : 0.f)) * inv, d1 = (p1 - (lab == 1 ? 1.f : 0.f)) * inv;
+    sum[grp][ch] = s0;
+    sum[grp][64 + ch] = s1;
     if (ch == 0) {
-        atomicAdd(loss, -logf(lab == 1 ? p1 : p0) * inv);
-        atomicAdd(dfb, d0);
-        atomicAdd(dfb + 1, d1);
+        sum[grp][128] = sl;
+        sum[grp][129] = sb0;
+        sum[grp][130] = sb1;
     }
-    atomicAdd(dfw + ch, d0 * g[ch]);
-    atomicAdd(dfw + 64 + ch, d1 * g[ch]);
-    const float dg = (d0 * fw[ch] + d1 * fw[64 + ch]) / 64.f;
-    const __nv_bfloat16 v = __float2bfloat16(dg);
-    __nv_bfloat16* d = da3 + ((int64_t)s * 8 + ch / 8) * 64 * 8 + ch % 8;
-    for (int q = 0; q < 64; q++) d[q * 8] = v;
+    __syncthreads();
+    if (threadIdx.x < 131) {
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < kHeadS; k++) v += sum[k][threadIdx.x];
+        atomicAdd(threadIdx.x < 128 ? dfw + threadIdx.x : threadIdx.x == 128 ? loss : dfb + (threadIdx.x - 129), v);
+    }
 }
 
 // Adam on fp32 master weights (Kingma & Ba 2015, bias-corrected).
@@ -164,7 +216,11 @@ int nn_pool_back(const __nv_bfloat16* dp, const uint8_t* idx, int n, int H, int 
 int nn_head(const __nv_bfloat16* a3, int n, const float* fw, const float* fb, float* logits, float* prob,
             const int32_t* y, float* loss, float* dfw, float* dfb, __nv_bfloat16* da3, cudaStream_t s)
 {
-    k_head<<<n, 64, 0, s>>>(a3, n, fw, fb, logits, prob, y, loss, dfw, dfb, da3);
+    int dev = 0, nsm = 0;
+    AF_CUDA(cudaGetDevice(&dev));
+    AF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int blocks = std::min((n + kHeadS - 1) / kHeadS, 2 * nsm);
+    k_head<<<blocks, 64 * kHeadS, 0, s>>>(a3, n, fw, fb, logits, prob, y, loss, dfw, dfb, da3);
     return af_cuda_check(cudaGetLastError(), "head");
 }
 

@@ -42,7 +42,10 @@ int nn_tconv_wgrad(int layer, const __nv_bfloat16* dz, const __nv_bfloat16* x, i
 int nn_tconv_wgrad_unpool(const __nv_bfloat16* dp, const uint8_t* idx, const __nv_bfloat16* x, int n, float* grad,
                           float* db, int* err, cudaStream_t s);
 size_t nn_tpack_bytes(int layer, int dgrad);
-int nn_tpack(int layer, int dgrad, const float* w, __nv_bfloat16* out, cudaStream_t s);
+// Packs w[l] into fwd[l] and dgrad[l] (l >= 1), where not NULL, and clears nclear
+// floats at `clear` (NULL: none), in one launch.
+int nn_tpack(const float* const (&w)[3], __nv_bfloat16* const (&fwd)[3], __nv_bfloat16* const (&dgrad)[3],
+             float* clear, int64_t nclear, cudaStream_t s);
 // 2x2 max-pool backward on channel-blocked tensors (dz [n][c/8][H][W][8] from
 // the pooled gradient and the argmax bytes, both [n][c/8][H/2][W/2][8]); adds
 // the bias gradient (sum of dz over pixels) into db.
