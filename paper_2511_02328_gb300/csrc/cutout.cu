@@ -19,6 +19,7 @@
 
 #include "internal.h"
 #include "nn.h"
+#include "tile.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -28,57 +29,147 @@ constexpr int S = 64;
 constexpr int kCl = 8;                 // CTAs per candidate (one thread-block cluster)
 constexpr int T = 256, NWARP = T / 32; // threads per CTA; warp w of CTA r owns image rows 8 r + w of both images
 constexpr int CH = 512;                // DM-time: window positions per chunk, 16 per lane
-constexpr int CHF = 496;               // frequency-time: positions per chunk, 16 per lane of lanes 0..30
-constexpr int kG = 6;                  // channels whose loads are issued together
+constexpr int CHF = 508;               // frequency-time: positions per chunk (the last word's bytes shift out)
+constexpr int kG = 4;                   // channels whose loads are issued together
 constexpr int kDelaysInShared = 8192 / kCl;  // a CTA's channels whose delays are staged in shared memory
+constexpr int kSortMax = 4096;         // candidates up to which clusters take them widest first
+constexpr int kRow = CH / 16 * 20;     // staged chunk: 16 positions every 20 words (no bank conflicts)
 
-// Adds u[0..15], the column sums of window positions q0 .. q0 + 15 (q0 = the
-// lane's first position), into the warp's 64 bins (bin j = positions
-// [j b, (j+1) b); positions from 64 b on belong to no bin): one shared atomic
-// per bin the lane's positions touch.
-__device__ __forceinline__ void add_bins(const int32_t* u, int q0, int b, unsigned long long* wb)
+// Adds the column sums of window positions q0 .. q0 + 15 (q0 = the lane's first
+// position, st = the warp's staged chunk) into the warp's 64 bins (bin j =
+// positions [j b, (j+1) b); positions from 64 b on belong to no bin): one addition
+// per bin the lane's positions touch.  A bin is two 32-bit words, sums of acc's low
+// 20 bits and of the rest: 32-bit shared additions are one instruction, 64-bit ones
+// a compare-and-swap loop that every lane of a wide bin takes part in.  fit: at
+// most 2048 additions per bin, so neither word overflows; else the bin is one
+// 64-bit word.  One copy of the code: the unrolled kernel otherwise misses its
+// instruction cache.
+__device__ __noinline__ void add_bins(const int32_t* st, int lane, int q0, int b, unsigned long long* wb, bool fit)
 {
     int bin = q0 / b, edge = (bin + 1) * b;
-    long long acc = 0;  // added as two's complement: plane values may be negative
-#pragma unroll
-    for (int jj = 0; jj < 16; jj++) {
-        if (q0 + jj == edge) {  // entering the next bin
-            if (bin < S && acc) atomicAdd(wb + bin, (unsigned long long)acc);
-            acc = 0;
-            bin++;
-            edge += b;
+    long long acc = 0;  // two's complement: plane values may be negative
+    auto put = [&]() {
+        if (bin < S && acc) {
+            if (fit) {
+                int* w = reinterpret_cast<int*>(wb + bin);
+                atomicAdd(w, (int)(acc & 0xFFFFF));
+                if (acc >> 20) atomicAdd(w + 1, (int)(acc >> 20));
+            } else {
+                atomicAdd(wb + bin, (unsigned long long)acc);
+            }
         }
-        acc += u[jj];
+    };
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const int4 u4 = *reinterpret_cast<const int4*>(st + lane * 20 + 4 * q);
+        const int u[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+        for (int jj = 0; jj < 4; jj++) {
+            if (q0 + 4 * q + jj == edge) {  // entering the next bin
+                put();
+                acc = 0;
+                bin++;
+                edge += b;
+            }
+            acc += u[jj];
+        }
     }
-    if (bin < S && acc) atomicAdd(wb + bin, (unsigned long long)acc);
+    put();
 }
 
-// Realigns a warp's 16-byte blocks: lane l holds own = the aligned block at
-// aa + 16 l; its 16 bytes start m bytes in (m warp-uniform), so they are the
-// bytes m .. m + 15 of own followed by lane l + 1's block (a shuffle), funnel-
-// shifted.  Lane 31's result is not used.
-__device__ __forceinline__ uint4 realign16(const uint4 own, int m)
+// One channel's words into the sums of bucket Q.  The comment keeps the compiler
+// from merging the four into one indexed access (which puts the sums in memory).
+template <int Q>
+__device__ __forceinline__ void add_bucket(uint32_t (&A)[4][4], uint32_t (&O)[4][4], const uint32_t (&w)[4])
 {
-    uint4 nx;
-    nx.x = __shfl_down_sync(0xffffffffu, own.x, 1);
-    nx.y = __shfl_down_sync(0xffffffffu, own.y, 1);
-    nx.z = __shfl_down_sync(0xffffffffu, own.z, 1);
-    nx.w = __shfl_down_sync(0xffffffffu, own.w, 1);
-    const uint32_t sh = 8u * (uint32_t)(m & 3);
-    switch (m >> 2) {  // warp-uniform
-    case 0:
-        return make_uint4(__funnelshift_r(own.x, own.y, sh), __funnelshift_r(own.y, own.z, sh),
-                          __funnelshift_r(own.z, own.w, sh), __funnelshift_r(own.w, nx.x, sh));
-    case 1:
-        return make_uint4(__funnelshift_r(own.y, own.z, sh), __funnelshift_r(own.z, own.w, sh),
-                          __funnelshift_r(own.w, nx.x, sh), __funnelshift_r(nx.x, nx.y, sh));
-    case 2:
-        return make_uint4(__funnelshift_r(own.z, own.w, sh), __funnelshift_r(own.w, nx.x, sh),
-                          __funnelshift_r(nx.x, nx.y, sh), __funnelshift_r(nx.y, nx.z, sh));
-    default:
-        return make_uint4(__funnelshift_r(own.w, nx.x, sh), __funnelshift_r(nx.x, nx.y, sh),
-                          __funnelshift_r(nx.y, nx.z, sh), __funnelshift_r(nx.z, nx.w, sh));
+    asm volatile("// bucket %0" ::"n"(Q));
+#pragma unroll
+    for (int m = 0; m < 4; m++) {
+        A[Q][m] += w[m];
+        O[Q][m] += __byte_perm(w[m], 0u, 0x4341);
     }
+}
+
+// One channel's words into the sums of the bucket of its byte offset sh (the
+// same in every lane).
+__device__ __forceinline__ void add_words(uint32_t (&A)[4][4], uint32_t (&O)[4][4], const uint32_t (&w)[4], int sh)
+{
+    if (sh & 2) {
+        if (sh & 1) add_bucket<3>(A, O, w);
+        else add_bucket<2>(A, O, w);
+    } else {
+        if (sh & 1) add_bucket<1>(A, O, w);
+        else add_bucket<0>(A, O, w);
+    }
+}
+
+// Adds nc channels' words: channel k's window starts at x + k * nsamp + dl[k],
+// x including the lane's 4 * lane bytes.  INNER: every word lies inside the input;
+// else words outside it (which hold no position that counts) are replaced by its
+// first or last.
+template <bool INNER>
+__device__ __forceinline__ void add_channels(uint32_t (&A)[4][4], uint32_t (&O)[4][4], const uint8_t* x, int64_t nsamp,
+                                             const int32_t* dl, int nc, const uint8_t* first, const uint8_t* last)
+{
+    auto load = [&](uint32_t (&w)[4], int dc) {
+        const uint8_t* a = x + dc;
+        const int sh = (int)((uintptr_t)a & 3);
+        a -= sh;
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const uint8_t* am = a + 128 * m;
+            if (!INNER) am = am < first ? first : am > last ? last : am;
+            w[m] = __ldg(reinterpret_cast<const uint32_t*>(am));
+        }
+        x += nsamp;
+        return sh;
+    };
+    int c = 0;
+#pragma unroll 1
+    for (; c + kG <= nc; c += kG) {
+        uint32_t w[kG][4];
+        int sh[kG];
+#pragma unroll
+        for (int k = 0; k < kG; k++) sh[k] = load(w[k], dl[c + k]);
+#pragma unroll
+        for (int k = 0; k < kG; k++) add_words(A, O, w[k], sh[k]);
+    }
+#pragma unroll 1
+    for (; c < nc; c++) {
+        uint32_t w[4];
+        const int sh = load(w, dl[c]);
+        add_words(A, O, w, sh);
+    }
+}
+
+// Position of window position q of a chunk in the staged chunk.
+__device__ __forceinline__ int staged(int q) { return q + (q >> 4) * 4; }
+
+// The candidate of rank `rank` when all n are taken widest first (by the widths'
+// binary order of magnitude, then by index).  Every thread of the CTA calls it.
+__device__ int ranked(const af_cand_t* __restrict__ cands, int n, int rank, int* hist, int* found)
+{
+    if (threadIdx.x < 32) hist[threadIdx.x] = 0;
+    __syncthreads();
+    auto cls = [&](int i) { return __clz(max(1, cands[i].width)); };  // small for wide
+    for (int i = threadIdx.x; i < n; i += T) atomicAdd(&hist[cls(i)], 1);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        int k = 0, left = rank;
+        while (left >= hist[k]) left -= hist[k++];
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + (int)threadIdx.x;
+            const unsigned m = __ballot_sync(0xffffffffu, i < n && cls(min(i, n - 1)) == k);
+            const int c = __popc(m);
+            if (left < c) {
+                if (((m >> threadIdx.x) & 1u) && __popc(m & ((1u << threadIdx.x) - 1u)) == left) *found = i;
+                break;
+            }
+            left -= c;
+        }
+    }
+    __syncthreads();
+    return *found;
 }
 
 // One cluster of kCl CTAs per candidate; CTA r computes DM-time rows and
@@ -86,31 +177,39 @@ __device__ __forceinline__ uint4 realign16(const uint4 own, int m)
 // Window positions q in [0, 64 b) are samples start + q, start = t - 32 b;
 // samples outside [0, nout) count 0.  A warp walks its rows in chunks, lane l
 // holding positions 16 l .. 16 l + 15 of the chunk (512 positions for the
-// DM-time row, 496 for the frequency-time row, whose lane 31 only supplies
-// the block after lane 30's): for the frequency-time row it adds the row's
-// channels in 16-bit lanes -- one aligned 16-byte load per channel and lane,
-// kG channels' loads issued together, realigned by a shuffle and funnel shifts
-// and masked to the positions that count (byte loads when the input rows are
-// not whole 16-byte blocks) -- then folds the 16 column sums into the warp's
-// bins.  The images' minimum and maximum are reduced over the cluster through
+// DM-time row, 508 for the frequency-time row).  DM-time values are loaded 32
+// consecutive at a time and staged in shared memory.  The frequency-time row adds
+// its channels as the dedispersion tile kernel does: aligned 32-bit words (four per
+// lane and channel, kG channels' loads issued together), bucketed by the byte the
+// window starts at, A += w and O += the odd bytes, the buckets folded once per
+// chunk; positions that do not count are cleared after the fold.  Then the chunk
+// is added into the warp's bins.  The images' minimum and maximum are reduced over the cluster through
 // distributed shared memory; every CTA of a cluster takes the same path (one
 // candidate), so both cluster barriers are reached by all of them.
+// Bound by the loads' latency.  256 candidates of widths 1 to 256, 4096 channels,
+// cut out and classified: 477 us (880 to 920 with 16-byte loads realigned by shuffles
+// and masked per channel, 64-bit bins and plane values loaded 64 bytes apart);
+// 3 CTAs per SM with 4 channels in flight a warp: 473, 2 with 8: 479, 4 with 2: 539.
+// Clusters take the widest candidates first, so that no long one starts last: in
+// the list's order 625 us.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(T, 3)
 k_cutout(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int32_t* __restrict__ D, int ndm,
-         const int32_t* __restrict__ plane, int64_t nout, const af_cand_t* __restrict__ cands, bool vec,
+         const int32_t* __restrict__ plane, int64_t nout, const af_cand_t* __restrict__ cands, int n, bool vec,
          __nv_bfloat16* __restrict__ out)
 {
     __shared__ unsigned long long wbins[NWARP][2][S];  // per warp: bins of its DM-time and frequency-time rows
     __shared__ int32_t sD[kDelaysInShared];            // the delays of this CTA's channels (when they fit)
     __shared__ long long red[NWARP][4];                // per-warp min / max of both images
+    __shared__ __align__(16) int32_t stage[NWARP][kRow];
+    __shared__ int hist[32], found;
     __shared__ long long mm[4];                        // this CTA's: DM-time min, max, frequency-time min, max
     cg::cluster_group cluster = cg::this_cluster();
     const int r = (int)cluster.block_rank();
-    const int cand = blockIdx.x / kCl;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cand = n <= kSortMax ? ranked(cands, n, (int)(blockIdx.x / kCl), hist, &found) : (int)(blockIdx.x / kCl);
     const af_cand_t cd = cands[cand];
     const int d = cd.dm_idx;
     __nv_bfloat16* o = out + (int64_t)cand * S * S * 2;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = NWARP * r + warp;  // image row of this warp (both images)
     if (d < 0 || d >= ndm) {  // not a row of this plan: zero cut-outs (the whole cluster returns here)
         for (int e = threadIdx.x; e < NWARP * S * 2; e += T) o[NWARP * r * S * 2 + e] = __float2bfloat16(0.f);
@@ -127,108 +226,91 @@ k_cutout(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int32_t*
     for (int e = lane; e < 2 * S; e += 32) (&wbins[warp][0][0])[e] = 0ull;
     __syncthreads();
 
+    // the bins' two 32-bit words hold every sum
+    const bool fit = b <= 2048 && (int64_t)gsz * 255 * b < (int64_t)1 << 31;
+    int32_t* st = stage[warp];
     // DM-time row: plane row d - 32 + row (0 outside the plan)
     const int pr = d - 32 + row;
     if (pr >= 0 && pr < ndm) {
         const int32_t* yr = plane + (int64_t)pr * nout;
         for (int p0 = 0; p0 < span; p0 += CH) {
-            const int q0 = p0 + 16 * lane;
-            int32_t u[16];
+            if (start + p0 + CH <= 0 || start + p0 >= nout) continue;  // no position counts
 #pragma unroll
-            for (int jj = 0; jj < 16; jj++) {
-                const int64_t sm = start + q0 + jj;
-                u[jj] = q0 + jj < span && sm >= 0 && sm < nout ? __ldg(yr + sm) : 0;
+            for (int jj = 0; jj < CH / 32; jj++) {
+                const int q = p0 + 32 * jj + lane;
+                const int64_t sm = start + q;
+                st[staged(32 * jj + lane)] = q < span && sm >= 0 && sm < nout ? __ldg(yr + sm) : 0;
             }
-            add_bins(u, q0, b, wbins[warp][0]);
+            __syncwarp();
+            add_bins(st, lane, p0 + 16 * lane, b, wbins[warp][0], fit);
+            __syncwarp();
         }
     }
-    // frequency-time row: channels row * gsz .. (row + 1) * gsz; lane 31
-    // holds no positions (it supplies lane 30's next block)
-    const int64_t total = (int64_t)nchan * nsamp;  // input bytes (a multiple of 16 when vec)
+    // frequency-time row: channels row * gsz .. (row + 1) * gsz
+    const int64_t last_word = (int64_t)nchan * nsamp - 4;  // nchan is a multiple of 64: whole words
+    const int32_t* dl = dsh ? sD + (row * gsz - cb) : D + (int64_t)d * nchan + row * gsz;  // the row's delays
     for (int p0 = 0; p0 < span; p0 += CHF) {
-        const int q0 = p0 + 16 * lane;
-        const int64_t s0 = start + q0;  // sample of the lane's first position
-        const bool mine = lane < 31;
-        // bytes of the lane's positions that count: inside the window and the plane's time range
-        uint32_t keep[4];
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            uint32_t k4 = 0;
-#pragma unroll
-            for (int bb = 0; bb < 4; bb++) {
-                const int jj = 4 * q + bb;
-                if (mine && q0 + jj < span && s0 + jj >= 0 && s0 + jj < nout) k4 |= 0xFFu << (8 * bb);
-            }
-            keep[q] = k4;
-        }
-        int32_t u[16];  // column sums, at most 255 * nchan / 64
-#pragma unroll
-        for (int jj = 0; jj < 16; jj++) u[jj] = 0;
-        for (int c0 = row * gsz; c0 < (row + 1) * gsz; c0 += 256) {  // 16-bit lanes hold 256 channels
-            const int c1 = min(c0 + 256, (row + 1) * gsz);
-            uint32_t E[4] = {0u, 0u, 0u, 0u}, O[4] = {0u, 0u, 0u, 0u};
+        const int64_t s0 = start + p0;  // sample of the chunk's first position
+        if (s0 + CHF <= 0 || s0 >= nout) continue;  // no position counts
+        const bool inner = s0 >= 3 && s0 + CH <= nout;  // every word of every channel lies inside its row
+        const bool full = s0 >= 0 && s0 + CHF <= nout && p0 + CHF <= span;  // every position counts
+        for (int c0 = 0; c0 < gsz; c0 += 256) {  // 16-bit lanes hold 256 channels
+            const int nc = min(256, gsz - c0);
+            const uint8_t* x = X + (int64_t)(row * gsz + c0) * nsamp + s0;
+            uint32_t u[4][4];  // column sums of positions 4 (lane + 32 m) + k, at most 255 * 256
             if (vec) {
-                for (int c = c0; c < c1; c += kG) {
-                    // the loads of kG channels first: the lane's aligned block
-                    // wherever it lies inside the input (a block holding a byte
-                    // that counts always does; the others are masked out)
-                    uint4 own[kG];
-                    int mk[kG];
+                uint32_t A[4][4], O[4][4];
 #pragma unroll
-                    for (int k = 0; k < kG; k++) {
-                        mk[k] = 0;
-                        own[k] = make_uint4(0u, 0u, 0u, 0u);
-                        if (c + k < c1) {
-                            const int32_t dc = dsh ? sD[c + k - cb] : __ldg(D + (int64_t)d * nchan + c + k);
-                            const int64_t a = (int64_t)(c + k) * nsamp + dc + s0;
-                            mk[k] = (int)(a & 15);  // the same in every lane
-                            const int64_t aa = a - mk[k];
-                            if (aa >= 0 && aa + 16 <= total) own[k] = __ldg(reinterpret_cast<const uint4*>(X + aa));
+                for (int q = 0; q < 4; q++)
+#pragma unroll
+                    for (int m = 0; m < 4; m++) A[q][m] = O[q][m] = 0u;
+                if (inner) add_channels<true>(A, O, x + 4 * lane, nsamp, dl + c0, nc, X, X + last_word);
+                else add_channels<false>(A, O, x + 4 * lane, nsamp, dl + c0, nc, X, X + last_word);
+#pragma unroll
+                for (int m = 0; m < 4; m++)
+#pragma unroll
+                    for (int k = 0; k < 4; k++) u[m][k] = 0u;
+                aftile::Tile<1, 4>::fold(A, O, u, lane);
+            } else {  // byte by byte
+#pragma unroll
+                for (int m = 0; m < 4; m++)
+#pragma unroll
+                    for (int k = 0; k < 4; k++) u[m][k] = 0u;
+#pragma unroll 1
+                for (int c = 0; c < nc; c++, x += nsamp)
+#pragma unroll
+                    for (int m = 0; m < 4; m++)
+#pragma unroll
+                        for (int k = 0; k < 4; k++) {
+                            const int p = 4 * (lane + 32 * m) + k;
+                            if (s0 + p >= 0 && s0 + p < nout) u[m][k] += __ldg(x + dl[c0 + c] + p);
                         }
-                    }
-#pragma unroll
-                    for (int k = 0; k < kG; k++)
-                        if (c + k < c1) {  // warp-uniform
-                            const uint4 v = realign16(own[k], mk[k]);
-                            const uint32_t w[4] = {v.x & keep[0], v.y & keep[1], v.z & keep[2], v.w & keep[3]};
-#pragma unroll
-                            for (int q = 0; q < 4; q++) {
-                                E[q] += w[q] & 0x00FF00FFu;
-                                O[q] += __byte_perm(w[q], 0u, 0x4341);
-                            }
-                        }
-                }
-            } else {
-                for (int c = c0; c < c1; c++) {
-                    const int32_t dc = dsh ? sD[c - cb] : __ldg(D + (int64_t)d * nchan + c);
-                    const int64_t a = (int64_t)c * nsamp + dc + s0;  // the lane's first byte (in the input where valid)
-#pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        uint32_t acc = 0;
-#pragma unroll
-                        for (int bb = 0; bb < 4; bb++)
-                            if ((keep[q] >> (8 * bb)) & 1u) acc |= (uint32_t)__ldg(X + a + 4 * q + bb) << (8 * bb);
-                        E[q] += acc & 0x00FF00FFu;
-                        O[q] += __byte_perm(acc, 0u, 0x4341);
-                    }
-                }
             }
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-                u[4 * q + 0] += (int32_t)(E[q] & 0xFFFFu);
-                u[4 * q + 1] += (int32_t)(O[q] & 0xFFFFu);
-                u[4 * q + 2] += (int32_t)(E[q] >> 16);
-                u[4 * q + 3] += (int32_t)(O[q] >> 16);
+            for (int m = 0; m < 4; m++) {
+                const int p = 4 * (lane + 32 * m);
+                if (!full) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++)
+                        if (p + k >= CHF || p0 + p + k >= span || s0 + p + k < 0 || s0 + p + k >= nout) u[m][k] = 0u;
+                } else if (p >= CHF) {
+                    u[m][0] = u[m][1] = u[m][2] = u[m][3] = 0u;
+                }
+                *reinterpret_cast<uint4*>(st + staged(p)) = make_uint4(u[m][0], u[m][1], u[m][2], u[m][3]);
             }
+            __syncwarp();
+            add_bins(st, lane, p0 + 16 * lane, b, wbins[warp][1], fit);
+            __syncwarp();
         }
-        if (mine) add_bins(u, q0, b, wbins[warp][1]);
     }
     __syncwarp();
     long long bins[2][2];  // [DM-time, frequency-time][column 2 lane + h]
 #pragma unroll
     for (int k = 0; k < 2; k++) {
-        bins[k][0] = (long long)wbins[warp][k][2 * lane];
-        bins[k][1] = (long long)wbins[warp][k][2 * lane + 1];
+        for (int h = 0; h < 2; h++) {
+            const long long w = (long long)wbins[warp][k][2 * lane + h];
+            bins[k][h] = fit ? ((w >> 32) << 20) + (long long)(uint32_t)w : w;
+        }
     }
 
     // min / max of both images: warp, CTA, then the cluster (distributed shared memory)
@@ -284,8 +366,7 @@ int nn_cutouts(const uint8_t* X, int64_t nsamp, int nchan, const int32_t* D, int
 {
     if (n <= 0) return AF_OK;
     if ((long long)n * kCl > 0x7fffffffLL) return af_set_error(AF_EINVAL, "cut-outs: too many candidates for one grid");
-    // 16-byte loads: the input 16-byte aligned with rows of whole 16-byte blocks
-    const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0 && nsamp % 16 == 0;
-    k_cutout<<<(unsigned)n * kCl, T, 0, s>>>(X, nsamp, nchan, D, ndm, plane, nout, cands, vec, out);
+    const bool vec = (reinterpret_cast<uintptr_t>(X) & 3) == 0;  // 32-bit loads
+    k_cutout<<<(unsigned)n * kCl, T, 0, s>>>(X, nsamp, nchan, D, ndm, plane, nout, cands, n, vec, out);
     return af_cuda_check(cudaGetLastError(), "cut-out launch");
 }
