@@ -1028,7 +1028,12 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
         cudaFree(T->d_ps);
         T->d_ps = nullptr;
         T->ps_bytes = 0;
-        if (cudaError_t e = cudaMalloc(&T->d_ps, (size_t)need * 2)) return af_cuda_check(e, "group rows");
+        if (cudaError_t e = cudaMalloc(&T->d_ps, (size_t)need * 2)) {
+            cudaGetLastError();  // the failed allocation is reported here, not by the next launch
+            T->d_ps = nullptr;
+            T->lay[0].L = T->lay[1].L = 0;  // nothing is reserved any more
+            return af_cuda_check(e, "group rows");
+        }
         T->ps_bytes = (size_t)need * 2;
     }
     std::vector<int64_t> rowoff(T->nrows), soff(T->h_srow.size());
@@ -1185,9 +1190,25 @@ size_t af_pairs_workspace(af_plan_t p, int64_t nout)
     return 2 * (size_t)rows_elems(best == 0 ? &p->pairs : &p->alt[best - 1], L);
 }
 
-// Reserves the picked group rows: the row buffer and the layouts of
-// af_dedisperse and (with `search`) af_search.  Nothing when none suits.
-int af_pairs_reserve(af_plan_t p, int64_t nout, bool search, bool allow_larger, size_t max_bytes)
+size_t af_pairs_lean_bytes(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes)
+{
+    size_t bytes = 0;
+    double best = 0;
+    for (int k = 0; k < 6; k++) {
+        const af_pair_tables* T = k == 0 ? &p->pairs : &p->alt[k - 1];
+        if (!T->ok || T->dpw != 1 || (T->G != 2 && !allow_larger) || (p->force_group && T->G != p->force_group)) continue;
+        const int64_t L = block_len(T, nout, max_bytes);
+        if (L <= 0) continue;
+        const double r = rows_rate_cost(p, T, nout, L);
+        if (!bytes || r < best) {
+            best = r;
+            bytes = 2 * (size_t)rows_elems(T, L);
+        }
+    }
+    return bytes;
+}
+
+static int reserve_once(af_plan_t p, int64_t nout, bool search, bool allow_larger, size_t max_bytes)
 {
     int64_t best_L = 0;
     if (int rc = af_pairs_pick(p, nout, allow_larger, max_bytes, &best_L)) return rc;
@@ -1203,6 +1224,17 @@ int af_pairs_reserve(af_plan_t p, int64_t nout, bool search, bool allow_larger, 
         if (int rc = pairs_layout(p, 1, Lmax)) return rc;
     }
     return AF_OK;
+}
+
+// Reserves the picked group rows: the row buffer and the layouts of
+// af_dedisperse and (with `search`) af_search.  Nothing when none suits.  Where the
+// device cannot hold the fastest set's buffer, the fastest within the lean one.
+int af_pairs_reserve(af_plan_t p, int64_t nout, bool search, bool allow_larger, size_t max_bytes)
+{
+    const int rc = reserve_once(p, nout, search, allow_larger, max_bytes);
+    if (rc != AF_ENOMEM) return rc;
+    const size_t lean = af_pairs_lean_bytes(p, nout, allow_larger, max_bytes);
+    return lean ? reserve_once(p, nout, search, allow_larger, std::min(lean, max_bytes)) : rc;
 }
 
 std::vector<int64_t> af_search_block_tiles(af_plan_t p, int64_t nout, int64_t cap_tiles)

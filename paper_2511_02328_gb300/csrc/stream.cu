@@ -331,13 +331,22 @@ try {
                               (size_t)s->ndm * sizeof(af_rowstats_t) + (size_t)s->cap * sizeof(af_cand_t) + 64;
     const size_t beam_bytes = (size_t)s->nchan * (size_t)std::max<int64_t>(s->dmax, 1);
     size_t budget = cfg->hbm_budget;
-    // the group-row buffer, where the plan uses group rows: the fastest group
-    // size whose buffer the budget holds next to the beam state and one slot
+    // the group-row buffer, where the plan uses group rows: the fastest set whose
+    // buffer the budget holds next to the beam state and as many slots as the lean
+    // set's buffer leaves (a larger one would trade slots for speed: 2 for 6 on 19
+    // beams of 4096 channels in 64 GiB)
     size_t rows = 0;
+    int nslots = cfg->max_slots > 0 ? cfg->max_slots : 4;
     if (p->pairs.ok && !p->force_tile && !p->force_simple) {
         const size_t fixed = beam_bytes * s->nbeams + slot_bytes;
         if (!budget || budget > fixed) {
-            if ((rc = af_pairs_reserve(p, s->hop, false, true, budget ? budget - fixed : SIZE_MAX))) {
+            size_t room = budget ? budget - fixed : SIZE_MAX;
+            const size_t lean = budget ? af_pairs_lean_bytes(p, s->hop, true, room) : 0;
+            if (lean) {
+                const size_t slots = std::min((size_t)nslots, 1 + (room - lean) / slot_bytes);
+                room -= (slots - 1) * slot_bytes;
+            }
+            if ((rc = af_pairs_reserve(p, s->hop, false, true, room))) {
                 free_stream(s);
                 return rc;
             }
@@ -349,7 +358,6 @@ try {
         free_stream(s);
         return af_set_error(AF_EINVAL, "af_stream_open: DM grid too coarse for the tile kernel");
     }
-    int nslots = cfg->max_slots > 0 ? cfg->max_slots : 4;
     if (budget) {
         if (budget < beam_bytes * s->nbeams + slot_bytes + rows) {
             free_stream(s);
