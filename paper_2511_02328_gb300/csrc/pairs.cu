@@ -1239,15 +1239,15 @@ int af_pairs_reserve(af_plan_t p, int64_t nout, bool search, bool allow_larger, 
 
 std::vector<int64_t> af_search_block_tiles(af_plan_t p, int64_t nout, int64_t cap_tiles)
 {
-    // the dedispersion consumes input ~5 times slower than a pinned host copy
-    // delivers it, and the copy starts before the first block: each block can
-    // be 6 times the previous one and still find its input in place when the
-    // previous one ends (on the 4096-channel workload: blocks of 6, 36 and 170
-    // tiles; a median call of 25.43 ms, against 25.81 ms growing by 4 and
-    // 25.90 ms growing by 8).  A block's tiles are rounded to whole waves of
-    // stage-2 blocks, one per SM: without that a block of 18 tiles x 34 DM
-    // blocks takes 5 waves for 4.03 of work (1024 channels, 262144 samples,
-    // 1001 DMs: a host search of 3.95 ms, 3.79 ms with whole waves).
+    // the dedispersion consumes input about 4 times slower than a pinned host copy
+    // delivers it, and the copy starts before the first block: each block can be 4
+    // times the previous one and still find its input in place when the previous
+    // one ends.  262144 samples, 4096 channels, 1001 DMs: a call of 21.9 ms growing
+    // by 4 or by 3, 23.4 by 6; 512 channels, 400 DMs, 131072 samples: 1.30 and 1.37
+    // ms; 1024 channels, 1001 DMs: 3.64 and 3.60 ms.  A block's tiles are rounded to
+    // whole waves of stage-2 blocks, one per SM: without that a block of 18 tiles x
+    // 34 DM blocks takes 5 waves for 4.03 of work (that last call: 3.95 ms growing by
+    // 6, 3.79 ms with whole waves, before stage 1's present form).
     const int64_t tiles = (nout + kPTTE - 1) / kPTTE;
     const int64_t nsm = p->num_sms > 0 ? p->num_sms : 152, nblk = std::max(1, p->pairs.nblk);
     cap_tiles = std::max<int64_t>(1, cap_tiles);
@@ -1261,7 +1261,7 @@ std::vector<int64_t> af_search_block_tiles(af_plan_t p, int64_t nout, int64_t ca
         const int64_t t = std::min(std::min(whole_waves(b), cap_tiles), tiles - done);
         out.push_back(t);
         done += t;
-        b = 6 * t;
+        b = 4 * t;
     }
     return out;
 }
