@@ -215,10 +215,7 @@ SB_N0, SB_NSUB = 8, 64
 # DRAM read + write bytes of one stage-2 group-row tile launch (k_pair_tile) on this workload, from an ncu
 # capture of the same kernel (dram__bytes_read.sum + dram__bytes_write.sum); None until captured, and reset
 # to None whenever the kernel changes
-PAIR_TILE_TRAFFIC = {   # keyed by channels per row: (bytes per launch, basis), from a capture of the current kernel
-    3: (3.64e10, "ncu dram__bytes read+write of k_pair_tile<15,3> on rows of 3 channels at 2^16 samples (3.26 GB, "
-                 "19 output tiles), scaled by the output tiles to this 2^18-sample launch (212 tiles)"),
-}
+PAIR_TILE_TRAFFIC = {}  # keyed by channels per row: (bytes per launch, basis), from a capture of the current kernel
 
 
 def match_pulses(cands, pulses, dms):
@@ -993,7 +990,7 @@ def main():
         performed = stage["row_bytes"] / 2 * (G - 1) + plan.ndm * ngroups * nout
         s1_ach = s1_bytes / (stage["rows_ms"] * 1e-3) / 1e9
         roofline = {
-            "bound": "smem", "kernel": "k_pair_tile<15,%d> (stage 2 of the group-row dedispersion, %d channels "
+            "bound": "smem", "kernel": "k_pair_tile, ring of %d (stage 2 of the group-row dedispersion, %d channels "
                                        "per row)" % (kern["ring"], G),
             "achieved": s2_ach, "peak": smem_peak, "unit": "TB/s", "frac": s2_ach / smem_peak,
             "traffic": traffic, "traffic_basis": traffic_basis,
@@ -1016,8 +1013,9 @@ def main():
                              "performed_frac_of_measured_int32_add_rate": performed / (ms_dedisp * 1e-3) / add_rate,
                              "measured_int32_add_rate": add_rate,
                              "note": "effective = the brute-force sum's ndm x nchan x nout additions per second "
-                                     "(the metric); performed = the additions the two stages execute: (G - 1) per "
-                                     "row sample in stage 1 + one per (DM, channel group, output) in stage 2",
+                                     "(the metric); performed = the additions the two stages execute: at most (G - 1) "
+                                     "per row sample in stage 1 (rows that share their first delays share those sums) "
+                                     "+ one per (DM, channel group, output) in stage 2",
                              "hbm": {"achieved": hbm_ach, "peak": hbm_peak, "unit": "GB/s",
                                      "frac": hbm_ach / hbm_peak, "basis": "of measured"}},
         }

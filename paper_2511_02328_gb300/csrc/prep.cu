@@ -2,12 +2,14 @@
 // square-law time downsampling and the zero-DM filter.
 //
 //   out[c][k] = min( sqrt(V * S / N), V ),  S = sum of bin k (N samples), V = 255,
-//   rounded half up, exactly: floor((isqrt(floor(4 V S / N)) + 1) / 2), evaluated
-//   as max r with r^2 N <= 4 V S from a float estimate and two integer tests.
+//   rounded half up, exactly: floor((isqrt(floor(4 V S / N)) + 1) / 2) (below).
 //
-// One block per (channel, run of TB bins): the block's input span is read
-// with coalesced loads into shared memory, then every thread sums its bins
-// there.  HBM-bound: nchan * nsamp bytes read, nchan * nsamp / D written.
+// Downsampling by 4, 8, 16 or 32 of rows of whole 16-byte pieces takes its bins straight
+// from 16-byte loads (k_downsample4); any other factor or alignment goes through
+// shared memory, one block per (channel, run of bins).  HBM-bound: nchan * nsamp
+// bytes read, nchan * nsamp / D written.  The zero-DM filter of up to 4096 channels
+// holds a tile of every channel in the shared memory of a thread-block cluster and
+// reads the input once; wider inputs are read twice.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
