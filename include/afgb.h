@@ -621,7 +621,7 @@ int af_stream_close(af_stream_t s);
  * (one block of 1024 threads per SM, a few milliseconds, synchronous) and
  * returns, in thread-operations per second,
  *   add_per_s           32-bit 2-input additions (8 independent chains per thread)
- *   pattern_adds_per_s  sample additions of the dedispersion inner step: two
+ *   pattern_adds_per_s  sample additions of a dedispersion inner step: two
  *                       32-bit shared loads (4 uint8 samples each), widening
  *                       into 16-bit lanes (and-mask, byte permute) and the
  *                       paired adds, i.e. 8 sample additions per step.

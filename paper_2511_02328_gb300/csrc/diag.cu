@@ -4,10 +4,12 @@
 // Three probe kernels, one block of 1024 threads per SM (120 KB of dynamic
 // shared memory keeps it to one), a fixed number of iterations each:
 //   ADD:     8 independent chains of 2-input 32-bit additions per thread;
-//   PATTERN: the tile kernel's inner step -- two 32-bit shared loads (two
+//   PATTERN: a dedispersion inner step on bytes -- two 32-bit shared loads (two
 //            channels, 4 samples each), widening into 16-bit lanes
 //            (w & 0x00FF00FF, prmt(w, 0x4341)) and the paired adds -- counted
-//            as 8 sample additions per iteration;
+//            as 8 sample additions per iteration; the tile kernel itself sums
+//            the words unmasked (four integer instructions instead of six), so
+//            it can pass this rate;
 //   SHARED:  8 independent 32-bit shared loads per iteration at immediate
 //            offsets from one moving base (lane-consecutive words: no bank
 //            conflicts), each folded into an accumulator -- the shared-memory
