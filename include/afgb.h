@@ -642,7 +642,9 @@ int af_diag_smem_rate(double* bytes_per_s);
  * 128 threads on the legacy default stream: arrive = 0 waits on a barrier that
  * nothing arrives at, so every wait gives up after `polls` polls and the call
  * returns AF_ETIMEOUT; arrive != 0 lets one thread arrive first and returns
- * AF_OK.  *ms (nullable) receives the kernel's duration, i.e. how long `polls`
+ * AF_OK.  arrive = 2 lets it arrive too, but half of every warp's lanes give up at
+ * once: a warp has one answer, so every thread is told that the wait ran out and
+ * the call returns AF_ETIMEOUT (AF_ECUDA if the threads disagree).  *ms (nullable) receives the kernel's duration, i.e. how long `polls`
  * polls of a wait that never completes take on this device.  Synchronous;
  * allocates nothing; AF_EINVAL unless 1 <= polls <= 2^24.  Not a step of the
  * paper's method. */

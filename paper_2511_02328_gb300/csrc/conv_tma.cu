@@ -257,8 +257,7 @@ __global__ void __launch_bounds__(kThreads) k_tconv(const typename Op::Args args
         int g = 0;
         for (; g < mytiles; g++) {
             const int s = g % NS;
-            if (g >= NS && !__all_sync(0xffffffffu, afumma::wait_or_abort(empty0 + 8 * s, (uint32_t)(g / NS - 1) & 1u,
-                                                                           abort, kBackoffNs)))
+            if (g >= NS && !afumma::wait_warp_or_abort(empty0 + 8 * s, (uint32_t)(g / NS - 1) & 1u, abort, kBackoffNs))
                 break;
             if (lane == 0) afptx::mbar_arrive_expect_tx(full0 + 8 * s, op.tx(tile_of(g)));
             __syncwarp();
@@ -278,8 +277,7 @@ __global__ void __launch_bounds__(kThreads) k_tconv(const typename Op::Args args
         int g = 0;
         for (; g < mytiles; g++) {
             const int s = g % NS;
-            if (!__all_sync(0xffffffffu, afumma::wait_or_abort(full0 + 8 * s, (uint32_t)(g / NS) & 1u, abort, kBackoffNs)))
-                break;
+            if (!afumma::wait_warp_or_abort(full0 + 8 * s, (uint32_t)(g / NS) & 1u, abort, kBackoffNs)) break;
             op.fixup(sm + Op::RB + (size_t)s * Op::SSTAGE, tile_of(g), lane);
             __syncwarp();
             if (lane == 0) afptx::mbar_arrive(ready0 + 8 * s);
@@ -304,15 +302,15 @@ __global__ void __launch_bounds__(kThreads) k_tconv(const typename Op::Args args
             __syncwarp();
         }
         // every MMA reading the ring has completed before the block leaves
-        for (int h = g - NS < 0 ? 0 : g - NS; h < g && !*abort; h++)
-            afumma::wait_or_abort(empty0 + 8 * (h % NS), (uint32_t)(h / NS) & 1u, abort);
+        for (int h = g - NS < 0 ? 0 : g - NS; h < g; h++)
+            if (!afumma::wait_warp_or_abort(empty0 + 8 * (h % NS), (uint32_t)(h / NS) & 1u, abort)) break;
     } else {
         // ---------------- epilogue (warps 2-5)
         const int quarter = warp & 3;
         if (Op::PER_TILE) {
             for (int i = 0; i < mytiles; i++) {
                 const int b = i % NACC;
-                const bool ok = afumma::wait_or_abort(tfull0 + 8 * b, (uint32_t)(i / NACC) & 1u, abort);
+                const bool ok = afumma::wait_warp_or_abort(tfull0 + 8 * b, (uint32_t)(i / NACC) & 1u, abort);
                 if (epi_sync_any(!ok || *abort)) break;  // all four warps leave together
                 afumma::fence_after_sync();
                 op.epilogue(tile_of(i), tmem + (uint32_t)(b * Op::NCOL), quarter, lane, xv, xq);
@@ -332,7 +330,7 @@ __global__ void __launch_bounds__(kThreads) k_tconv(const typename Op::Args args
                 if (grp < mytiles) op.unpool_load(tile_of(grp), tg, pre);
                 for (int g = grp; g < mytiles; g += 2) {
                     const int s = g % NS;
-                    if (g >= NS && !afumma::wait_or_abort(empty0 + 8 * s, (uint32_t)(g / NS - 1) & 1u, abort)) {
+                    if (g >= NS && !afumma::wait_warp_or_abort(empty0 + 8 * s, (uint32_t)(g / NS - 1) & 1u, abort)) {
                         ok = false;
                         break;
                     }
@@ -344,7 +342,7 @@ __global__ void __launch_bounds__(kThreads) k_tconv(const typename Op::Args args
                 }
                 op.unpool_finish(t, lane, acc, xv);
             }
-            ok = afumma::wait_or_abort(tfull0, 0u, abort) && ok;
+            ok = afumma::wait_warp_or_abort(tfull0, 0u, abort) && ok;
             if (!epi_sync_any(!ok || *abort)) {
                 afumma::fence_after_sync();
                 if constexpr (Op::UNPOOL) op.unpool_add(tid - 64, xv);

@@ -159,14 +159,14 @@ __global__ void __launch_bounds__(kBlock) k_umma(const typename Op::Args args)
             __syncwarp();
         }
         // every stage's release has arrived before the block's shared memory goes away
-        for (int g = G - NS < 0 ? 0 : G - NS; g < G && !*abort; g++)
-            afumma::wait_or_abort(empty0 + 8 * (g % NS), (uint32_t)(g / NS) & 1u, abort);
+        for (int g = G - NS < 0 ? 0 : G - NS; g < G; g++)
+            if (!afumma::wait_warp_or_abort(empty0 + 8 * (g % NS), (uint32_t)(g / NS) & 1u, abort)) break;
     } else {
         // ---------------- epilogue
         const int quarter = warp & 3;
         for (int i = 0; i < mytiles; i++) {
             const int b = i % NACC;
-            if (!afumma::wait_or_abort(tfull0 + 8 * b, (uint32_t)(i / NACC) & 1u, abort)) break;
+            if (!afumma::wait_warp_or_abort(tfull0 + 8 * b, (uint32_t)(i / NACC) & 1u, abort)) break;
             afumma::fence_after_sync();
             op.epilogue((int)blockIdx.x + i * (int)gridDim.x, tmem + (uint32_t)(b * Op::NCOL), quarter, lane);
             afumma::fence_before_sync();

@@ -116,14 +116,17 @@ int time_probe(int nblk, float* ms)
     return af_cuda_check(e, "af_diag_int_rates probe");
 }
 
-// Error flag of the bounded-wait probe (a static device variable: no allocation).
+// Threads of the bounded-wait probe told that the wait ran out (a static device
+// variable: no allocation).
 __device__ int g_diag_wait_err;
 
-// One block of 128 threads waits on an mbarrier of one arrival.  arrive = 1:
-// thread 0 arrives, the phase completes and every wait succeeds.  arrive = 0:
-// nothing arrives, every thread's wait gives up after `polls` polls, lane 0 of
-// each warp raises the flag (as the ring kernels' warps do) and the block
-// returns.  No copy is in flight, so nothing else has to drain.
+// One block of 128 threads waits on an mbarrier of one arrival, warp by warp as
+// the ring kernels do.  arrive = 1: thread 0 arrives, the phase completes and
+// every wait succeeds.  arrive = 0: nothing arrives, every thread's wait gives up
+// after `polls` polls, each lane that is told so counts itself, and the block
+// returns.  arrive = 2: the phase completes, but every warp's odd lanes give up at
+// once: the answer is one for the warp, so every lane is told that the wait ran
+// out.  No copy is in flight, so nothing else has to drain.
 __global__ void __launch_bounds__(128) k_diag_wait(int arrive, uint32_t polls)
 {
     __shared__ __align__(8) uint64_t bar;
@@ -134,7 +137,8 @@ __global__ void __launch_bounds__(128) k_diag_wait(int arrive, uint32_t polls)
     }
     __syncthreads();
     if (arrive && threadIdx.x == 0) afptx::mbar_arrive(b);
-    if (!afptx::mbar_wait_bounded(b, 0u, polls) && (threadIdx.x & 31) == 0) atomicExch(&g_diag_wait_err, 1);
+    const uint32_t mine = arrive == 2 && (threadIdx.x & 1) ? 0u : polls;
+    if (!afptx::mbar_wait_warp(b, 0u, mine)) atomicAdd(&g_diag_wait_err, 1);
     __syncthreads();
     if (threadIdx.x == 0) afptx::mbar_inval(b);
 }
@@ -184,7 +188,7 @@ try {
     AF_CUDA(cudaEventCreate(&a));
     AF_CUDA(cudaEventCreate(&b));
     cudaEventRecord(a);
-    k_diag_wait<<<1, 128>>>(arrive ? 1 : 0, (uint32_t)polls);
+    k_diag_wait<<<1, 128>>>(arrive == 0 ? 0 : arrive == 2 ? 2 : 1, (uint32_t)polls);
     cudaEventRecord(b);
     cudaError_t e = cudaEventSynchronize(b);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -196,6 +200,8 @@ try {
     cudaEventDestroy(b);
     if (int rc = af_cuda_check(e, "af_diag_bounded_wait")) return rc;
     if (ms) *ms = t;
+    if (err != 0 && err != 128)
+        return af_set_error(AF_ECUDA, "af_diag_bounded_wait: %d of 128 threads were told that the wait ran out", err);
     if (err)
         return af_set_error(AF_ETIMEOUT, "af_diag_bounded_wait: the wait ran out after %lld polls (%.3f ms)",
                             (long long)polls, (double)t);

@@ -426,7 +426,7 @@ struct PairTile {
                     snxt = __ldg(a.soff + cdb.y + lane) + dt;
                 }
                 if (kk >= NS &&
-                    !afptx::mbar_wait_bounded(empty0 + 8 * st, (uint32_t)(kk / NS - 1) & 1u, kPWait)) {
+                    !afptx::mbar_wait_warp(empty0 + 8 * st, (uint32_t)(kk / NS - 1) & 1u, kPWait)) {
                     if (lane == 0) atomicExch(a.err, 1);
                     break;
                 }
@@ -439,7 +439,7 @@ struct PairTile {
             }
             // (a drain wait that runs out raises the error flag like any other)
             for (int k2 = max(0, kk - NS); k2 < kk; k2++)
-                if (!afptx::mbar_wait_bounded(full0 + 8 * (k2 % NS), (uint32_t)(k2 / NS) & 1u, kPWait) && lane == 0)
+                if (!afptx::mbar_wait_warp(full0 + 8 * (k2 % NS), (uint32_t)(k2 / NS) & 1u, kPWait) && lane == 0)
                     atomicExch(a.err, 1);
             return;
         }
@@ -455,7 +455,7 @@ struct PairTile {
         int npacc = 0;
         for (int kk = 0; kk < nchk; kk++) {
             const int st = kk % NS;
-            if (!afptx::mbar_wait_bounded(full0 + 8 * st, (uint32_t)(kk / NS) & 1u, kPWait)) {
+            if (!afptx::mbar_wait_warp(full0 + 8 * st, (uint32_t)(kk / NS) & 1u, kPWait)) {
                 if (lane == 0) atomicExch(a.err, 1);
                 return;
             }

@@ -78,6 +78,17 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     return false;
 }
 
+// The same by a whole warp, with one answer: true only if the phase completed
+// for every lane.  Lanes poll on their own, so one may run out while its
+// neighbour still sees the phase complete; a warp that went on without it would
+// wait for it in the next shuffle or __syncwarp, and warp-collective tensor-memory
+// instructions are undefined without all lanes.  The vote also reconverges the
+// warp after the poll loops.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t limit)
+{
+    return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, limit)) != 0;
+}
+
 // d = high 32 bits of (a * b) + c  (one IMAD.HI on the FMA pipe)
 __device__ __forceinline__ uint32_t mad_hi(uint32_t a, uint32_t b, uint32_t c)
 {

@@ -319,7 +319,7 @@ struct Tile {
                 const bool valid1 = c1 < cur.cend;
                 const int dmin1 = valid1 ? __ldg(pmin + c1) : 0;
                 if (kk >= NS &&
-                    !afptx::mbar_wait_bounded(empty0 + 8 * st, (uint32_t)(kk / NS - 1) & 1u, WAIT_LIMIT)) {
+                    !afptx::mbar_wait_warp(empty0 + 8 * st, (uint32_t)(kk / NS - 1) & 1u, WAIT_LIMIT)) {
                     if (lane == 0) atomicExch(a.err, 1);
                     break;
                 }
@@ -331,7 +331,7 @@ struct Tile {
             // leave no copy in flight behind (the consumers normally wait for all of them)
             // (a drain wait that runs out raises the error flag like any other)
             for (int k2 = max(0, kk - NS); k2 < kk; k2++)
-                if (!afptx::mbar_wait_bounded(full0 + 8 * (k2 % NS), (uint32_t)(k2 / NS) & 1u, WAIT_LIMIT) && lane == 0)
+                if (!afptx::mbar_wait_warp(full0 + 8 * (k2 % NS), (uint32_t)(k2 / NS) & 1u, WAIT_LIMIT) && lane == 0)
                     atomicExch(a.err, 1);
             return;
         }
@@ -366,7 +366,7 @@ struct Tile {
             dl = valid ? __ldg(prow + c) : 0;
             dmin = valid ? __ldg(pmin + c) : 0;
             __syncwarp();
-            if (!afptx::mbar_wait_bounded(full0 + 8 * st, (uint32_t)(kk / NS) & 1u, WAIT_LIMIT)) {
+            if (!afptx::mbar_wait_warp(full0 + 8 * st, (uint32_t)(kk / NS) & 1u, WAIT_LIMIT)) {
                 if (lane == 0) atomicExch(a.err, 1);
                 return;
             }

@@ -146,4 +146,13 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
     return false;
 }
 
+// The same by a whole warp, with one answer (false if any lane gave up) and the
+// lanes converged again: what the warp-collective tensor-memory instructions,
+// barriers and shuffles after a wait need.
+__device__ __forceinline__ bool wait_warp_or_abort(uint32_t bar, uint32_t parity, volatile int* abort,
+                                                   uint32_t backoff_ns = 0)
+{
+    return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort, backoff_ns)) != 0;
+}
+
 }  // namespace afumma
