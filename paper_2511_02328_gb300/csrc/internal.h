@@ -217,6 +217,7 @@ struct af_plan_s {
     int force_group = 0;                   // 2, 3 or 4: only that group size (AFGB_PAIR_GROUP)
     af_pair_tables pairs;                  // group-row path of brute-force plans (the one in use)
     af_pair_tables alt[5];                 // the other group sizes and block heights, until a reservation picks
+    int64_t rows_nout = 0, rows_search = 0;  // most outputs reserved on group rows: for any call, for af_search
 
     // two-stage subband dedispersion (sb_nsub > 0); `delays` then holds the
     // effective table D[j(m)][c] + R[m][s(c)]

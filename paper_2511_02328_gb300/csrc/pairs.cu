@@ -1208,7 +1208,7 @@ size_t af_pairs_lean_bytes(af_plan_t p, int64_t nout, bool allow_larger, size_t 
     return bytes;
 }
 
-static int reserve_once(af_plan_t p, int64_t nout, bool search, bool allow_larger, size_t max_bytes)
+static int reserve_once(af_plan_t p, int64_t nout, int64_t search, bool allow_larger, size_t max_bytes)
 {
     int64_t best_L = 0;
     if (int rc = af_pairs_pick(p, nout, allow_larger, max_bytes, &best_L)) return rc;
@@ -1216,10 +1216,10 @@ static int reserve_once(af_plan_t p, int64_t nout, bool search, bool allow_large
     af_pair_tables* T = &p->pairs;
     if (best_L > T->lay[0].L)
         if (int rc = pairs_layout(p, 0, best_L)) return rc;
-    if (search) {
+    if (search > 0) {
         // af_search's growing time blocks, so that the input copy overlaps the
         // work: the layout holds the longest of them
-        const std::vector<int64_t> blocks = af_search_block_tiles(p, nout, T->lay[0].L / kPTTE);
+        const std::vector<int64_t> blocks = af_search_block_tiles(p, search, T->lay[0].L / kPTTE);
         const int64_t Lmax = *std::max_element(blocks.begin(), blocks.end()) * kPTTE;
         if (int rc = pairs_layout(p, 1, Lmax)) return rc;
     }
@@ -1227,14 +1227,24 @@ static int reserve_once(af_plan_t p, int64_t nout, bool search, bool allow_large
 }
 
 // Reserves the picked group rows: the row buffer and the layouts of
-// af_dedisperse and (with `search`) af_search.  Nothing when none suits.  Where the
-// device cannot hold the fastest set's buffer, the fastest within the lean one.
+// af_dedisperse and (with `search`) af_search.  Nothing when none suits.  The set is
+// picked, and both layouts are made, for the most outputs any reservation of the plan
+// asked for: another length often prefers another set, and a shorter one must not
+// give up what a longer one reserved.  Where the device cannot hold the fastest
+// set's buffer, the fastest within the lean one.
 int af_pairs_reserve(af_plan_t p, int64_t nout, bool search, bool allow_larger, size_t max_bytes)
 {
-    const int rc = reserve_once(p, nout, search, allow_larger, max_bytes);
-    if (rc != AF_ENOMEM) return rc;
-    const size_t lean = af_pairs_lean_bytes(p, nout, allow_larger, max_bytes);
-    return lean ? reserve_once(p, nout, search, allow_larger, std::min(lean, max_bytes)) : rc;
+    nout = std::max(nout, p->rows_nout);
+    const int64_t srch = std::max(search ? nout : 0, p->rows_search);
+    int rc = reserve_once(p, nout, srch, allow_larger, max_bytes);
+    if (rc == AF_ENOMEM) {
+        const size_t lean = af_pairs_lean_bytes(p, nout, allow_larger, max_bytes);
+        if (lean) rc = reserve_once(p, nout, srch, allow_larger, std::min(lean, max_bytes));
+    }
+    if (rc) return rc;
+    p->rows_nout = nout;
+    p->rows_search = srch;
+    return AF_OK;
 }
 
 std::vector<int64_t> af_search_block_tiles(af_plan_t p, int64_t nout, int64_t cap_tiles)
@@ -1412,17 +1422,21 @@ int af_launch_pairs(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int64_t nou
             return rc;
     const int slot = T->tcalls > 0 ? T->tnext : -1;
     int b = 0;
+    int64_t rowbytes = 0;
     for (int64_t T0 = 0; T0 < nout; T0 += L, b++) {
         const bool rec = slot >= 0 && b < T->tblocks;
         cudaEvent_t* e = rec ? &T->tev[((size_t)slot * T->tblocks + b) * 3] : nullptr;
         if (rec) AF_CUDA(cudaEventRecord(e[0], s));
-        if (int rc = af_launch_pairs_block(p, d_in, nsamp, nout, d_plane, d_stats, s, 0, T0, rec ? e + 1 : nullptr))
+        // the last block, or a call shorter than the reservation, needs only its own tiles' rows
+        const int64_t Lb = std::min(L, (nout - T0 + kPTTE - 1) / kPTTE * kPTTE);
+        rowbytes += 2 * rows_elems(T, L) - 2 * (int64_t)T->nrows * ((L - Lb) & ~(int64_t)15);
+        if (int rc = af_launch_pairs_block(p, d_in, nsamp, nout, d_plane, d_stats, s, 0, T0, rec ? e + 1 : nullptr, Lb))
             return rc;
         if (rec) AF_CUDA(cudaEventRecord(e[2], s));
     }
     if (slot >= 0) {
         T->tnb[slot] = std::min(b, T->tblocks);
-        T->trowbytes[slot] = 2 * rows_elems(T, L) * (int64_t)b;
+        T->trowbytes[slot] = rowbytes;
         T->tcopybytes[slot] = (int64_t)((double)((nout + kPTTE - 1) / kPTTE) * T->copy_per_tile);
         T->tnext = (slot + 1) % T->tcalls;
     }
