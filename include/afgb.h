@@ -264,9 +264,12 @@ int af_dedisperse(af_plan_t plan, const uint8_t* d_in, int64_t nsamp,
  * its DMs long) fit the row budget (AFGB_PAIR_BUDGET_MB at plan creation,
  * default min(48 GiB, 1/5 of device memory)); later calls of any length run in
  * as many time blocks as they need.  Allocates and uploads synchronously (waits for the
- * device when it replaces a reservation); AF_OK without effect for plans that
- * cannot use group rows.  AF_EINVAL if max_nsamp <= Dmax, AF_ENOMEM / AF_ECUDA
- * on allocation failure.  Not a step of the paper's method: the same sum,
+ * device when it replaces a reservation); a shorter reservation after a longer
+ * one keeps the longer one's.  Where the device cannot hold the rows, shorter
+ * time blocks are reserved, and where it cannot hold even those the plan stays
+ * on the channel tile kernel.  AF_OK without effect for plans that cannot use
+ * group rows.  AF_EINVAL if max_nsamp <= Dmax, AF_ENOMEM / AF_ECUDA on
+ * allocation failure (AF_ENOMEM: the plan has no channel tile kernel either).  Not a step of the paper's method: the same sum,
  * grouped. */
 int af_dedisperse_reserve(af_plan_t plan, int64_t max_nsamp);
 /* Device bytes af_dedisperse_reserve(plan, max_nsamp) would allocate (the

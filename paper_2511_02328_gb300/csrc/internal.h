@@ -153,8 +153,9 @@ int64_t af_pairs_block(af_plan_t p, int64_t nout);
 int af_pairs_reserve(af_plan_t p, int64_t nout, bool search, bool allow_larger = true,
                      size_t max_bytes = SIZE_MAX);
 int af_pairs_pick(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L);
-// Row-buffer bytes of the set of 15-row blocks that moves the fewest bytes within
-// max_bytes (0: none): what callers short of memory limit the pick to.
+// Row-buffer bytes of the set of 15-row blocks (of 30-row blocks where there is no
+// other) that moves the fewest bytes within max_bytes (0: none): what callers short of
+// memory limit the pick to.
 size_t af_pairs_lean_bytes(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes);
 size_t af_pairs_workspace(af_plan_t p, int64_t nout);  // row-buffer bytes a reservation would allocate
 // Stage 1 alone (the rows of time block T0 of layout `layout`), the stage-2

@@ -1194,17 +1194,19 @@ size_t af_pairs_lean_bytes(af_plan_t p, int64_t nout, bool allow_larger, size_t 
 {
     size_t bytes = 0;
     double best = 0;
-    for (int k = 0; k < 6; k++) {
-        const af_pair_tables* T = k == 0 ? &p->pairs : &p->alt[k - 1];
-        if (!T->ok || T->dpw != 1 || (T->G != 2 && !allow_larger) || (p->force_group && T->G != p->force_group)) continue;
-        const int64_t L = block_len(T, nout, max_bytes);
-        if (L <= 0) continue;
-        const double r = rows_rate_cost(p, T, nout, L);
-        if (!bytes || r < best) {
-            best = r;
-            bytes = 2 * (size_t)rows_elems(T, L);
+    for (int dpw = 1; dpw <= 2 && !bytes; dpw++)  // sets of 30-row blocks only where there is no other
+        for (int k = 0; k < 6; k++) {
+            const af_pair_tables* T = k == 0 ? &p->pairs : &p->alt[k - 1];
+            if (!T->ok || T->dpw != dpw || (T->G != 2 && !allow_larger) || (p->force_group && T->G != p->force_group))
+                continue;
+            const int64_t L = block_len(T, nout, max_bytes);
+            if (L <= 0) continue;
+            const double r = rows_rate_cost(p, T, nout, L);
+            if (!bytes || r < best) {
+                best = r;
+                bytes = 2 * (size_t)rows_elems(T, L);
+            }
         }
-    }
     return bytes;
 }
 
@@ -1231,15 +1233,23 @@ static int reserve_once(af_plan_t p, int64_t nout, int64_t search, bool allow_la
 // picked, and both layouts are made, for the most outputs any reservation of the plan
 // asked for: another length often prefers another set, and a shorter one must not
 // give up what a longer one reserved.  Where the device cannot hold the fastest
-// set's buffer, the fastest within the lean one.
+// set's buffer, the fastest within the lean one where that fits what is free, then
+// within half of what is free, a quarter, and so on (shorter time blocks); where not
+// even a small block fits, the plan stays on the channel tile kernel.
 int af_pairs_reserve(af_plan_t p, int64_t nout, bool search, bool allow_larger, size_t max_bytes)
 {
     nout = std::max(nout, p->rows_nout);
     const int64_t srch = std::max(search ? nout : 0, p->rows_search);
     int rc = reserve_once(p, nout, srch, allow_larger, max_bytes);
     if (rc == AF_ENOMEM) {
+        size_t fr = 0, tot = 0;
+        AF_CUDA(cudaMemGetInfo(&fr, &tot));
         const size_t lean = af_pairs_lean_bytes(p, nout, allow_larger, max_bytes);
-        if (lean) rc = reserve_once(p, nout, srch, allow_larger, std::min(lean, max_bytes));
+        size_t room = std::min(max_bytes, lean && lean <= fr ? lean : fr / 2);
+        // ends: no set has a block that fits a small room, and nothing is allocated then
+        for (; rc == AF_ENOMEM; room /= 2) rc = reserve_once(p, nout, srch, allow_larger, room);
+        if (rc == AF_OK && !af_dedisp_uses_pairs(p, nout) && p->tile.ns1 == 0)
+            return af_set_error(AF_ENOMEM, "group rows: no room for a time block's rows");
     }
     if (rc) return rc;
     p->rows_nout = nout;
