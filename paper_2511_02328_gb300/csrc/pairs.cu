@@ -708,7 +708,7 @@ void af_pairs_free(af_pair_tables* T)
 // for the time block's first tile.
 typedef std::array<int32_t, 3> Key;
 
-static void build_groups(af_plan_t p, int G, int dpw, int optin, const std::vector<int>& order, af_pair_tables* T)
+static void build_groups(af_plan_t p, int G, int dpw, int NS, int optin, const std::vector<int>& order, af_pair_tables* T)
 {
     const int nchan = p->nchan, ndm = p->ndm, NW = kPNW * dpw, K = G - 1;  // NW: DM rows of a block
     const int nblk = (ndm + NW - 1) / NW;
@@ -783,8 +783,6 @@ static void build_groups(af_plan_t p, int G, int dpw, int optin, const std::vect
         }
     const int64_t rwe = r8((int64_t)spread + 1031);
     if (spread >= (1 << 20) || maxdr > kMaxDr) return;
-    int NS = 3;
-    if (const char* e = getenv("AFGB_PAIR_STAGES")) NS = std::min(4, std::max(2, atoi(e)));
     // one stage: up to kPSL windows back to back; the widest window must fit
     // (16 bytes stay free for the static shared memory of the persistent form)
     const int stage_bytes = (int)(((size_t)optin - tables_smem(NS, dpw) - 16) / NS) & ~15;
@@ -890,7 +888,6 @@ static void build_groups(af_plan_t p, int G, int dpw, int optin, const std::vect
     T->rwe = (int)rwe;
     T->maxdr = maxdr;
     T->rows_per_pair = rows_per_group;
-    T->budget = pair_budget();
     T->shape = NS;
     T->stage_bytes = stage_bytes;
     T->copy_per_tile = copy;
@@ -914,11 +911,22 @@ static void build_groups(af_plan_t p, int G, int dpw, int optin, const std::vect
     T->ok = true;
 }
 
+// Gives up the host copies of what a set's device tables hold.
+static void drop_uploaded(af_pair_tables* T)
+{
+    auto gone = [](auto& h) { std::remove_reference_t<decltype(h)>().swap(h); };
+    gone(T->h_rdelta), gone(T->h_gdr), gone(T->h_chunks), gone(T->h_chkoff), gone(T->h_srec), gone(T->h_perm);
+    gone(T->h_tabs);
+}
+
 // Device copies of a table set and its layouts' arrays (once, when a
 // reservation or a batch first uses the set; the host copies go).
 static int upload_groups(af_pair_tables* T)
 {
-    if (T->d_tabs) return AF_OK;
+    if (T->d_tabs) {
+        drop_uploaded(T);
+        return AF_OK;
+    }
     cudaError_t e = cudaSuccess;
     auto up = [&](auto** d, auto& h) {
         if (e == cudaSuccess) e = cudaMalloc(d, h.size() * sizeof(h[0]));
@@ -947,9 +955,40 @@ static int upload_groups(af_pair_tables* T)
         for (auto& l : T->lay) drop(l.d_pinfo), drop(l.d_rinfo), drop(l.d_rowoff), drop(l.d_soff);
         return af_cuda_check(e, "group tables");
     }
-    auto gone = [](auto& h) { std::remove_reference_t<decltype(h)>().swap(h); };
-    gone(T->h_rdelta), gone(T->h_gdr), gone(T->h_chunks), gone(T->h_chkoff), gone(T->h_srec), gone(T->h_perm);
-    gone(T->h_tabs);
+    drop_uploaded(T);
+    return AF_OK;
+}
+
+// Plane rows by ascending DM.
+static std::vector<int> dm_order(af_plan_t p)
+{
+    std::vector<int> order(p->ndm);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->dms[x] < p->dms[y]; });
+    return order;
+}
+
+// The tables of the sets that no reservation uses: the rows' sizes, which the
+// cost model reads, stay; the rest (about 20 MB a set on 4096 channels and 1001 DMs,
+// for the life of the plan and of every beam of a batch) goes, and is built again
+// if a later reservation picks the set.
+static void drop_unused(af_plan_t p)
+{
+    for (af_pair_tables& T : p->alt) {
+        drop_uploaded(&T);
+        std::vector<int32_t>().swap(T.h_srow);
+        std::vector<int32_t>().swap(T.h_scpart);
+    }
+}
+
+// The tables of set T again, where they were dropped (h_srow is empty then: a set
+// has at least one row window).
+static int restore_groups(af_plan_t p, af_pair_tables* T)
+{
+    if (!T->h_srow.empty()) return AF_OK;
+    int optin = 0;
+    AF_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
+    build_groups(p, T->G, T->dpw, T->shape, optin, dm_order(p), T);
     return AF_OK;
 }
 
@@ -960,9 +999,10 @@ int af_pairs_build(af_plan_t p)
 {
     int optin = 0;
     AF_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
-    std::vector<int> order(p->ndm);  // plane rows by ascending DM
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->dms[x] < p->dms[y]; });
+    const std::vector<int> order = dm_order(p);
+    int NS = 3;
+    if (const char* e = getenv("AFGB_PAIR_STAGES")) NS = std::min(4, std::max(2, atoi(e)));
+    const size_t budget = pair_budget();
     int only = 0;
     if (const char* e = getenv("AFGB_PAIR_DPW")) only = atoi(e);
     std::vector<std::future<void>> jobs;
@@ -974,7 +1014,8 @@ int af_pairs_build(af_plan_t p)
             af_pair_tables* T = k == 0 ? &p->pairs : &p->alt[k - 1];
             k++;
             jobs.push_back(std::async(threads ? std::launch::async : std::launch::deferred,
-                                      [=, &order] { build_groups(p, G, dpw, optin, order, T); }));
+                                      [=, &order] { build_groups(p, G, dpw, NS, optin, order, T); }));
+            T->budget = budget;
         }
     for (auto& j : jobs) j.get();
     return AF_OK;
@@ -1019,7 +1060,9 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
     af_pair_tables* T = &p->pairs;
     af_pair_tables::Layout& ly = T->lay[k];
     if (ly.L == L) return AF_OK;
+    if (int rc = restore_groups(p, T)) return rc;
     if (int rc = upload_groups(T)) return rc;
+    drop_unused(p);
     const int64_t need = rows_elems(T, L);
     if (ly.L || (size_t)need * 2 > T->ps_bytes)
         if (int rc = af_cuda_check(cudaDeviceSynchronize(), "pair layout")) return rc;
