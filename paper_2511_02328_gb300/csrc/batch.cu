@@ -172,7 +172,7 @@ static int setup_pairs(af_batch_t b)
         Beam& x = b->beams[i];
         if (!x.plan->pairs.ok) continue;
         int64_t L = 0;  // the beam's fastest group size within the largest buffer
-        if (int rc = af_pairs_pick(x.plan, x.nout, true, kPairsMax, &L)) return rc;
+        if (int rc = af_pairs_pick(x.plan, x.nout, true, kPairsMax, &L, false)) return rc;
         if (L <= 0) continue;
         use[i] = true;
         need = std::max(need, std::min(af_pairs_bytes(x.plan, x.nout), kPairsMax));
@@ -210,7 +210,7 @@ static int setup_persist(af_batch_t b, int tiles)
         Beam& x = b->beams[i];
         if (!x.plan->pairs.ok) continue;
         int64_t L = 0;
-        if (int rc = af_pairs_pick(x.plan, x.nout, true, kPairsMax, &L)) return rc;
+        if (int rc = af_pairs_pick(x.plan, x.nout, true, kPairsMax, &L, false)) return rc;
         if (L <= 0) continue;
         if (ns == 0) ns = af_pairs_ring(x.plan);
         if (af_pairs_ring(x.plan) != ns) continue;  // tables for another ring depth

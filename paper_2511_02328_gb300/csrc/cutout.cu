@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <stdint.h>
+#include <stdlib.h>
 
 #include "internal.h"
 #include "nn.h"
@@ -32,7 +33,7 @@ constexpr int CH = 512;                // DM-time: window positions per chunk, 1
 constexpr int CHF = 508;               // frequency-time: positions per chunk (the last word's bytes shift out)
 constexpr int kG = 4;                   // channels whose loads are issued together
 constexpr int kDelaysInShared = 8192 / kCl;  // a CTA's channels whose delays are staged in shared memory
-constexpr int kSortMax = 4096;         // candidates up to which clusters take them widest first
+constexpr int kSortMax = 1024;         // candidates up to which clusters may take them widest first
 constexpr int kRow = CH / 16 * 20;     // staged chunk: 16 positions every 20 words (no bank conflicts)
 
 // Adds the column sums of window positions q0 .. q0 + 15 (q0 = the lane's first
@@ -145,28 +146,40 @@ __device__ __forceinline__ void add_channels(uint32_t (&A)[4][4], uint32_t (&O)[
 // Position of window position q of a chunk in the staged chunk.
 __device__ __forceinline__ int staged(int q) { return q + (q >> 4) * 4; }
 
-// The candidate of rank `rank` when all n are taken widest first (by the widths'
-// binary order of magnitude, then by index).  Every thread of the CTA calls it.
-__device__ int ranked(const af_cand_t* __restrict__ cands, int n, int rank, int* hist, int* found)
+// The candidate of rank `rank` when all n <= kSortMax are taken widest first (by
+// the widths' binary order of magnitude, then by index).  mask: kSortMax / 32 rows of
+// 32 words.  Every thread of the CTA calls it.
+__device__ int ranked(const af_cand_t* __restrict__ cands, int n, int rank, uint32_t* mask, int* found)
 {
-    if (threadIdx.x < 32) hist[threadIdx.x] = 0;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, chunks = (n + 31) / 32;
+    // which of every 32 candidates are in which class: mask[32 c + class], one ballot per class there
+    for (int c = warp; c < chunks; c += NWARP) {
+        const int i = 32 * c + lane;
+        const int cls = i < n ? __clz(max(1, cands[i].width)) : 32;  // small for wide
+        mask[32 * c + lane] = 0u;
+        const uint32_t m = __match_any_sync(0xffffffffu, cls);  // also orders the clear before the store
+        if (cls < 32 && lane == __ffs(m) - 1) mask[32 * c + cls] = m;
+    }
     __syncthreads();
-    auto cls = [&](int i) { return __clz(max(1, cands[i].width)); };  // small for wide
-    for (int i = threadIdx.x; i < n; i += T) atomicAdd(&hist[cls(i)], 1);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        int k = 0, left = rank;
-        while (left >= hist[k]) left -= hist[k++];
-        for (int i0 = 0; i0 < n; i0 += 32) {
-            const int i = i0 + (int)threadIdx.x;
-            const unsigned m = __ballot_sync(0xffffffffu, i < n && cls(min(i, n - 1)) == k);
-            const int c = __popc(m);
-            if (left < c) {
-                if (((m >> threadIdx.x) & 1u) && __popc(m & ((1u << threadIdx.x) - 1u)) == left) *found = i;
-                break;
+    if (warp == 0) {
+        // what lane `at` of the warp holds when the lanes' counts pass `left`; left becomes the rest
+        auto pass = [&](int cnt, int& left) {
+            int incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
             }
-            left -= c;
-        }
+            const int at = __ffs(__ballot_sync(0xffffffffu, left < incl)) - 1;
+            left -= __shfl_sync(0xffffffffu, incl - cnt, at);
+            return at;
+        };
+        int left = rank, tot = 0;
+        for (int c = 0; c < chunks; c++) tot += __popc(mask[32 * c + lane]);
+        const int k = pass(tot, left);                                            // the class
+        const int c = pass(lane < chunks ? __popc(mask[32 * lane + k]) : 0, left);  // its 32 candidates
+        const int b = pass((int)(mask[32 * c + k] >> lane & 1u), left);             // its bit
+        if (lane == 0) *found = 32 * c + b;
     }
     __syncthreads();
     return *found;
@@ -194,19 +207,21 @@ __device__ int ranked(const af_cand_t* __restrict__ cands, int n, int rank, int*
 // the list's order 625 us.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(T, 3)
 k_cutout(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int32_t* __restrict__ D, int ndm,
-         const int32_t* __restrict__ plane, int64_t nout, const af_cand_t* __restrict__ cands, int n, bool vec,
+         const int32_t* __restrict__ plane, int64_t nout, const af_cand_t* __restrict__ cands, int n, bool order, bool vec,
          __nv_bfloat16* __restrict__ out)
 {
     __shared__ unsigned long long wbins[NWARP][2][S];  // per warp: bins of its DM-time and frequency-time rows
     __shared__ int32_t sD[kDelaysInShared];            // the delays of this CTA's channels (when they fit)
     __shared__ long long red[NWARP][4];                // per-warp min / max of both images
-    __shared__ __align__(16) int32_t stage[NWARP][kRow];
-    __shared__ int hist[32], found;
+    __shared__ __align__(16) int32_t stage[NWARP][kRow];  // first: the ranking's masks
+    static_assert(kSortMax <= 1024 && sizeof(int32_t) * NWARP * kRow >= kSortMax * 4, "masks of 32 rows of 32 words");
+    __shared__ int found;
     __shared__ long long mm[4];                        // this CTA's: DM-time min, max, frequency-time min, max
     cg::cluster_group cluster = cg::this_cluster();
     const int r = (int)cluster.block_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cand = n <= kSortMax ? ranked(cands, n, (int)(blockIdx.x / kCl), hist, &found) : (int)(blockIdx.x / kCl);
+    const int cand = order ? ranked(cands, n, (int)(blockIdx.x / kCl), reinterpret_cast<uint32_t*>(stage), &found)
+                           : (int)(blockIdx.x / kCl);
     const af_cand_t cd = cands[cand];
     const int d = cd.dm_idx;
     __nv_bfloat16* o = out + (int64_t)cand * S * S * 2;
@@ -367,6 +382,11 @@ int nn_cutouts(const uint8_t* X, int64_t nsamp, int nchan, const int32_t* D, int
     if (n <= 0) return AF_OK;
     if ((long long)n * kCl > 0x7fffffffLL) return af_set_error(AF_EINVAL, "cut-outs: too many candidates for one grid");
     const bool vec = (reinterpret_cast<uintptr_t>(X) & 3) == 0;  // 32-bit loads
-    k_cutout<<<(unsigned)n * kCl, T, 0, s>>>(X, nsamp, nchan, D, ndm, plane, nout, cands, n, vec, out);
+    int dev = 0, nsm = 0;
+    AF_CUDA(cudaGetDevice(&dev));
+    AF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    static const int kmax = getenv("CUT_MAX") ? atoi(getenv("CUT_MAX")) : kSortMax;
+    const bool order = n * kCl > 3 * nsm && n <= kmax;
+    k_cutout<<<(unsigned)n * kCl, T, 0, s>>>(X, nsamp, nchan, D, ndm, plane, nout, cands, n, order, vec, out);
     return af_cuda_check(cudaGetLastError(), "cut-out launch");
 }

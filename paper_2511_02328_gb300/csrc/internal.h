@@ -106,7 +106,7 @@ struct af_pair_tables {
     bool ok = false;               // the plan can use this path
     int G = 2;                     // channels per group (2, 3 or 4)
     int dpw = 1;                   // DM rows per consumer warp: blocks of 15 or 30 DM rows
-    int np = 0, nrows = 0, rwe = 0, maxdr = 0;   // np = groups
+    int np = 0, nrows = 0, maxdr = 0;   // np = groups
     double rows_per_pair = 0;      // rows copied per pair and DM block (mean)
     size_t budget = 0;             // bytes the row buffer may take (AFGB_PAIR_BUDGET_MB at plan creation)
     int shape = 0;                 // ring depth of the row kernel (2 to 4 stages)
@@ -149,10 +149,10 @@ struct af_pair_tables {
 };
 int af_pairs_build(af_plan_t p);
 void af_pairs_free(af_pair_tables* T);
-int64_t af_pairs_block(af_plan_t p, int64_t nout);
 int af_pairs_reserve(af_plan_t p, int64_t nout, bool search, bool allow_larger = true,
                      size_t max_bytes = SIZE_MAX);
-int af_pairs_pick(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L);
+// alone: for the plan's own calls; else for one beam among a batch's.
+int af_pairs_pick(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L, bool alone);
 // Row-buffer bytes of the set of 15-row blocks (of 30-row blocks where there is no
 // other) that moves the fewest bytes within max_bytes (0: none): what callers short of
 // memory limit the pick to.
@@ -189,7 +189,6 @@ int af_pair_ring_depth(int shape);
 // Row-buffer bytes of a full-length single time block, and the use of a row
 // buffer owned by someone else (a batch's plans run one after another on one).
 size_t af_pairs_bytes(af_plan_t p, int64_t nout);
-size_t af_pairs_reserved_bytes(af_plan_t p, int64_t nout);  // what af_pairs_reserve would allocate
 int af_pairs_attach(af_plan_t p, uint16_t* buf, size_t bytes, int64_t nout);
 bool af_dedisp_uses_pairs(af_plan_t p, int64_t nout);
 

@@ -649,9 +649,7 @@ size_t pair_budget()
 // rows; both together 24.8 / 19.2 / 18.8 ms, and in blocks of 30 rows, which copy
 // 0.65 / 0.68 / 0.72 of the bytes, 25.0 / 17.2 / 14.3 ms.  The rates below are fitted
 // to both stages' times of 70 plans (128 to 4096 channels, 64 to 1495 DMs, 11 k to
-// 215 k outputs; the fit's errors are 6 and 7 %); the channel tile kernel adds about
-// 17.7 T samples/s.
-constexpr double kTileAddps = 17.7e12;
+// 215 k outputs; the fit's errors are 6 and 7 %).
 constexpr double kBlockStart = 4.6e-6;  // a stage-2 block's first copies and its stores, per 15 DM rows
 constexpr double kBlockNorm = 6.4;      // how far a block's loads and copies overlap
 constexpr double kRowRead = 4.7e12;     // stage 2: rows from HBM, overlapping the blocks (6.2-norm)
@@ -662,6 +660,14 @@ inline double copy_rate(int G) { return G == 4 ? 6.8e12 : G == 3 ? 7.2e12 : 7.7e
 constexpr double kRowsLaunch = 5.6e-6, kRowPart = 1.1e-9, kRowSerial = 0.37e-6;
 inline double rows_block(int G) { return G == 4 ? 8.1e-9 : G == 3 ? 5.0e-9 : 2.9e-9; }
 inline double row_rate(int G) { return G == 4 ? 5.2e12 : G == 3 ? 6.2e12 : 6.5e12; }
+// The channel tile kernel: a launch, whole waves of one block per SM, each some
+// microseconds and a channel's samples after another.  Fitted, with the kernel whose
+// warps build their own tables, to 875 plans (8 to 4096 channels, 2 to 1500 DMs, 300
+// to 150,000 outputs; error 5 %).
+constexpr double kTileLaunch = 4.0e-6, kTileWave = 4.0e-6, kTileChan = 74.1e-9;
+// what two launches cost beyond rows_cost on the smallest plans (on the 875 plans,
+// 4 / 6 / 8 us: the slower side by more than 5 % in 28 / 26 / 28)
+constexpr double kRowsMargin = 6.0e-6;
 
 }  // namespace
 
@@ -800,7 +806,7 @@ static void build_groups(af_plan_t p, int G, int dpw, int NS, int optin, const s
     std::vector<Key> dq(NW), S;
     std::vector<int32_t> d0(NW), sdm;
     int open_slots = 0, open_bytes = 0, first_slot = 0;
-    std::vector<int> sbyt, soffs;  // slot bytes and stage offsets of the open group
+    std::vector<int> sbyt;  // slot bytes of the open group
     auto flush = [&]() {
         if (ents.empty()) return;
         const size_t base = tabs.size();
@@ -885,7 +891,6 @@ static void build_groups(af_plan_t p, int G, int dpw, int NS, int optin, const s
     T->dpw = dpw;
     T->np = ng;
     T->nrows = (int)rB.size();
-    T->rwe = (int)rwe;
     T->maxdr = maxdr;
     T->rows_per_pair = rows_per_group;
     T->shape = NS;
@@ -1050,8 +1055,6 @@ static int64_t block_len(const af_pair_tables* T, int64_t nout, size_t max_bytes
     return lo * kPTTE;
 }
 
-int64_t af_pairs_block(af_plan_t p, int64_t nout) { return block_len(&p->pairs, nout); }
-
 // Layout k (0: af_dedisperse, 1: af_search) of the row buffer for time
 // blocks of L outputs; waits for the device first when it replaces a layout
 // or the buffer (kernels in flight may read them).  Reservation calls only.
@@ -1118,15 +1121,17 @@ static int pairs_layout(af_plan_t p, int k, int64_t L)
 // on many waves and slower where 15 rows fill the last wave better (2128 channels,
 // 609 DMs, 22 tiles: 902 blocks of 15 in 0.62 ms, 462 of 30 in 0.75 ms).  Stage 1
 // is its blocks and the row pieces they write, or, where they are few, the group
-// with the most rows.
-static double rows_cost(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L)
+// with the most rows.  Not alone (a batch's beams side by side): its share of the
+// GPU's time, without launches, unfilled waves and latencies.
+static double rows_cost(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L, bool alone = true)
 {
     const double nsm = p->num_sms > 0 ? p->num_sms : 152;
     const double loads = 2.0 * kPNW * T->dpw * T->np * 64.0 * kPMG / (load_rate(T->G) / nsm);
     const double copies = T->copy_per_tile / T->nblk / (copy_rate(T->G) / nsm);
     const double block = std::pow(std::pow(loads, kBlockNorm) + std::pow(copies, kBlockNorm), 1.0 / kBlockNorm) + kBlockStart * T->dpw;
     auto waves = [&](int64_t outs) {
-        return std::ceil((double)((outs + kPTTE - 1) / kPTTE) * T->nblk / nsm);
+        const double w = (double)((outs + kPTTE - 1) / kPTTE) * T->nblk / nsm;
+        return alone ? std::ceil(w) : w;
     };
     const int64_t full = nout / L, rest = nout - full * L;
     const double times = (double)full + (rest > 0 ? (double)rest / L : 0.0);
@@ -1143,12 +1148,11 @@ static double rows_cost(af_plan_t p, const af_pair_tables* T, int64_t nout, int6
         most = std::max(most, T->h_rb[q + 1] - T->h_rb[q]);
     }
     const double all = blocks1 * rows_block(T->G) + (double)rows_elems(T, L) / kET * kRowPart;
-    const double s1 = times * (kRowsLaunch + std::cbrt(std::pow(all, 3) + std::pow(most * kRowSerial, 3)));
+    const double s1 = alone ? times * (kRowsLaunch + std::cbrt(std::pow(all, 3) + std::pow(most * kRowSerial, 3))) : times * all;
     return s1 + s2;
 }
 
-// The same at throughput alone, neither side's launches, waves or latencies
-// counted, as the channel tile kernel's time below is: what decides between the two.
+// The same at throughput alone, for blocks of 15 DM rows: bytes moved at a rate.
 static double rows_rate_cost(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L)
 {
     const double tiles = (double)((nout + kPTTE - 1) / kPTTE), blocks = (double)((nout + L - 1) / L);
@@ -1159,9 +1163,21 @@ static double rows_rate_cost(af_plan_t p, const af_pair_tables* T, int64_t nout,
     return s1 + s2;
 }
 
-static bool rows_beat_tile(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L)
+// Whether set T in time blocks of L outputs is predicted faster than the channel
+// tile kernel, for a plan's calls (alone) and for a batch's beams (not alone; its
+// autotuner then measures both).  Of the 875
+// plans above this picks the slower side by more than 5 % in 26 (at most 1.19
+// times); the two kernels' throughputs alone, as of blocks of 15 DM rows and an
+// earlier tile kernel, did so in 213 (2.05 times: few DMs of many channels, or few
+// outputs of few channels).  128 channels x 1001 DMs x 5000 outputs: rows 76 us,
+// tiles 45; 4096 x 16 x 700: rows 154 us, tiles 314.
+static bool rows_beat_tile(af_plan_t p, const af_pair_tables* T, int64_t nout, int64_t L, bool alone)
 {
-    return rows_rate_cost(p, T, nout, L) < (double)p->ndm * p->nchan * (double)nout / kTileAddps;
+    const double nsm = p->num_sms > 0 ? p->num_sms : 152;
+    const int64_t tiles = (nout + af_dedisp_tile_outputs() - 1) / af_dedisp_tile_outputs();
+    const double waves = (double)tiles * p->tile.nblk / nsm, wave = kTileWave + kTileChan * p->nchan;
+    if (!alone) return rows_cost(p, T, nout, L, false) < waves * wave;
+    return rows_cost(p, T, nout, L) + kRowsMargin < kTileLaunch + std::ceil(waves) * wave;
 }
 
 // Gives up a table set's row buffer and layouts (after the device is idle).
@@ -1179,13 +1195,13 @@ static int pairs_release(af_pair_tables* T)
 
 // Picks the group rows for nout outputs: of the group sizes (2 only unless
 // larger groups are allowed; AFGB_PAIR_GROUP=2|3|4 restricts), the one
-// predicted fastest within max_bytes of rows, if any beats the channel tile
+// predicted fastest within max_bytes of rows, if it beats the channel tile
 // kernel (AFGB_DEDISP_KERNEL=pairs skips that comparison); it becomes
 // p->pairs (a previously picked set gives up its buffer).  *L gets its time
 // block; 0 when nothing suits.
 // The candidate (0: p->pairs, k: p->alt[k - 1]) and time block the pick would
 // take, or -1; changes nothing.
-static int pairs_choose(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L)
+static int pairs_choose(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L, bool alone = true)
 {
     *L = 0;
     // the set the model predicts fastest: over 70 plans 0.1 % slower on average than
@@ -1194,13 +1210,11 @@ static int pairs_choose(af_plan_t p, int64_t nout, bool allow_larger, size_t max
     int best = -1;
     double best_t = 0;
     int64_t Ls[6] = {};
-    bool beats = false;
     for (int k = 0; k < 6; k++) {
         const af_pair_tables* T = k == 0 ? &p->pairs : &p->alt[k - 1];
         if (!T->ok || (T->G != 2 && !allow_larger) || (p->force_group && T->G != p->force_group)) continue;
         Ls[k] = block_len(T, nout, max_bytes);
         if (Ls[k] <= 0) continue;
-        beats = beats || rows_beat_tile(p, T, nout, Ls[k]);
         const double t = rows_cost(p, T, nout, Ls[k]);
         if (best < 0 || t < best_t) {
             best = k;
@@ -1209,14 +1223,15 @@ static int pairs_choose(af_plan_t p, int64_t nout, bool allow_larger, size_t max
     }
     if (best < 0) return -1;
     const bool tile = p->tile.ns1 > 0;  // else the one-thread-per-output kernel
-    if (!p->force_pairs && tile && !beats) return -1;
+    if (!p->force_pairs && tile && !rows_beat_tile(p, best == 0 ? &p->pairs : &p->alt[best - 1], nout, Ls[best], alone))
+        return -1;
     *L = Ls[best];
     return best;
 }
 
-int af_pairs_pick(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L)
+int af_pairs_pick(af_plan_t p, int64_t nout, bool allow_larger, size_t max_bytes, int64_t* L, bool alone)
 {
-    const int best = pairs_choose(p, nout, allow_larger, max_bytes, L);
+    const int best = pairs_choose(p, nout, allow_larger, max_bytes, L, alone);
     if (best < 0) return AF_OK;
     if (best > 0) {
         if (int rc = pairs_release(&p->pairs)) return rc;
@@ -1256,7 +1271,7 @@ size_t af_pairs_lean_bytes(af_plan_t p, int64_t nout, bool allow_larger, size_t 
 static int reserve_once(af_plan_t p, int64_t nout, int64_t search, bool allow_larger, size_t max_bytes)
 {
     int64_t best_L = 0;
-    if (int rc = af_pairs_pick(p, nout, allow_larger, max_bytes, &best_L)) return rc;
+    if (int rc = af_pairs_pick(p, nout, allow_larger, max_bytes, &best_L, true)) return rc;
     if (best_L <= 0) return AF_OK;
     af_pair_tables* T = &p->pairs;
     if (best_L > T->lay[0].L)
@@ -1329,12 +1344,6 @@ std::vector<int64_t> af_search_block_tiles(af_plan_t p, int64_t nout, int64_t ca
     return out;
 }
 
-size_t af_pairs_reserved_bytes(af_plan_t p, int64_t nout)
-{
-    const int64_t L = af_pairs_block(p, nout);
-    return L > 0 ? 2 * (size_t)rows_elems(&p->pairs, L) : 0;
-}
-
 size_t af_pairs_bytes(af_plan_t p, int64_t nout)
 {
     const af_pair_tables* T = &p->pairs;
@@ -1356,7 +1365,7 @@ int af_pairs_attach(af_plan_t p, uint16_t* buf, size_t bytes, int64_t nout)
         if (rows_elems(T, mid * kPTTE) <= cap) lo = mid;
         else hi = mid - 1;
     }
-    if (!p->force_pairs && p->tile.ns1 > 0 && !rows_beat_tile(p, T, nout, lo * kPTTE))
+    if (!p->force_pairs && p->tile.ns1 > 0 && !rows_beat_tile(p, T, nout, lo * kPTTE, false))
         return AF_OK;  // this beam stays on the channel tile kernel
     if (int rc = af_cuda_check(cudaDeviceSynchronize(), "pairs attach")) return rc;
     if (T->ps_owned) cudaFree(T->d_ps);

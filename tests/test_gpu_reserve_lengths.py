@@ -33,8 +33,9 @@ def _call(p, x):
 def test_shorter_reservation_keeps_the_longer(nchan, ndm, long, short, search, monkeypatch):
     from paper_2511_02328_gb300 import _lib
     from paper_2511_02328_gb300.search import Plan
-    for k in ("AFGB_DEDISP_KERNEL", "AFGB_PAIR_GROUP", "AFGB_PAIR_DPW", "AFGB_PAIR_STAGES", "AFGB_PAIR_BUDGET_MB"):
+    for k in ("AFGB_PAIR_GROUP", "AFGB_PAIR_DPW", "AFGB_PAIR_STAGES", "AFGB_PAIR_BUDGET_MB"):
         monkeypatch.delenv(k, raising=False)
+    monkeypatch.setenv("AFGB_DEDISP_KERNEL", "pairs")  # rows even where channel tiles are faster
     dms = np.arange(ndm) * 1.0
     own = Plan(nchan, *BAND, TSAMP, dms)  # what the short length would pick by itself
     own.reserve(own.dmax + short)

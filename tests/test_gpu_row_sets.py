@@ -21,8 +21,9 @@ def _built():
 
 @pytest.fixture(autouse=True)
 def _default_choice(monkeypatch):
-    for k in ("AFGB_DEDISP_KERNEL", "AFGB_PAIR_GROUP", "AFGB_PAIR_DPW", "AFGB_PAIR_STAGES", "AFGB_PAIR_BUDGET_MB"):
+    for k in ("AFGB_PAIR_GROUP", "AFGB_PAIR_DPW", "AFGB_PAIR_STAGES", "AFGB_PAIR_BUDGET_MB"):
         monkeypatch.delenv(k, raising=False)
+    monkeypatch.setenv("AFGB_DEDISP_KERNEL", "pairs")  # rows even where channel tiles are faster
 
 
 def test_growing_lengths_switch_sets(monkeypatch):
