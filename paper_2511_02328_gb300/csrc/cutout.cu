@@ -16,7 +16,6 @@
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <stdint.h>
-#include <stdlib.h>
 
 #include "internal.h"
 #include "nn.h"
@@ -153,12 +152,20 @@ __device__ int ranked(const af_cand_t* __restrict__ cands, int n, int rank, uint
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, chunks = (n + 31) / 32;
     // which of every 32 candidates are in which class: mask[32 c + class], one ballot per class there
-    for (int c = warp; c < chunks; c += NWARP) {
-        const int i = 32 * c + lane;
-        const int cls = i < n ? __clz(max(1, cands[i].width)) : 32;  // small for wide
+    constexpr int PER = kSortMax / 32 / NWARP;
+    int cls[PER];
+#pragma unroll
+    for (int k = 0; k < PER; k++) {
+        const int i = 32 * (warp + k * NWARP) + lane;
+        cls[k] = i < n ? __clz(max(1, __ldg(&cands[i].width))) : 32;  // small for wide
+    }
+#pragma unroll
+    for (int k = 0; k < PER; k++) {
+        const int c = warp + k * NWARP;
+        if (c >= chunks) break;  // the same in every lane
         mask[32 * c + lane] = 0u;
-        const uint32_t m = __match_any_sync(0xffffffffu, cls);  // also orders the clear before the store
-        if (cls < 32 && lane == __ffs(m) - 1) mask[32 * c + cls] = m;
+        const uint32_t m = __match_any_sync(0xffffffffu, cls[k]);  // also orders the clear before the store
+        if (cls[k] < 32 && lane == __ffs(m) - 1) mask[32 * c + cls[k]] = m;
     }
     __syncthreads();
     if (warp == 0) {
@@ -203,8 +210,8 @@ __device__ int ranked(const af_cand_t* __restrict__ cands, int n, int rank, uint
 // cut out and classified: 477 us (880 to 920 with 16-byte loads realigned by shuffles
 // and masked per channel, 64-bit bins and plane values loaded 64 bytes apart);
 // 3 CTAs per SM with 4 channels in flight a warp: 473, 2 with 8: 479, 4 with 2: 539.
-// Clusters take the widest candidates first, so that no long one starts last: in
-// the list's order 625 us.
+// Clusters take the widest candidates of a list of moderate length first, so that no
+// long one starts last: in the list's order 625 us.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(T, 3)
 k_cutout(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int32_t* __restrict__ D, int ndm,
          const int32_t* __restrict__ plane, int64_t nout, const af_cand_t* __restrict__ cands, int n, bool order, bool vec,
@@ -382,11 +389,11 @@ int nn_cutouts(const uint8_t* X, int64_t nsamp, int nchan, const int32_t* D, int
     if (n <= 0) return AF_OK;
     if ((long long)n * kCl > 0x7fffffffLL) return af_set_error(AF_EINVAL, "cut-outs: too many candidates for one grid");
     const bool vec = (reinterpret_cast<uintptr_t>(X) & 3) == 0;  // 32-bit loads
-    int dev = 0, nsm = 0;
-    AF_CUDA(cudaGetDevice(&dev));
-    AF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    static const int kmax = getenv("CUT_MAX") ? atoi(getenv("CUT_MAX")) : kSortMax;
-    const bool order = n * kCl > 3 * nsm && n <= kmax;
+    // Widest first pays where one wide candidate would start last, and costs every block a look at the whole list: worth
+    // it up to about 9 waves of clusters (57 of them run at a time), twice that where a candidate's own work is longer.
+    // 512 candidates, ordered / not: widths mixed 1 to 256, 4096 channels 805 / 945 us, 64 channels 238 / 242; width 1, 64
+    // channels 130 / 115; 1024 at 4096 channels 1605 / 1772; 4000, every block ranking all (before): 7264 / 6340.
+    const bool order = n > 8 && n <= (nchan >= 512 ? kSortMax : kSortMax / 2);
     k_cutout<<<(unsigned)n * kCl, T, 0, s>>>(X, nsamp, nchan, D, ndm, plane, nout, cands, n, order, vec, out);
     return af_cuda_check(cudaGetLastError(), "cut-out launch");
 }
