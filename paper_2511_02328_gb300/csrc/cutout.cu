@@ -105,8 +105,7 @@ __device__ __forceinline__ void add_words(uint32_t (&A)[4][4], uint32_t (&O)[4][
 
 // Adds nc channels' words: channel k's window starts at x + k * nsamp + dl[k],
 // x including the lane's 4 * lane bytes.  INNER: every word lies inside the input;
-// else words outside it (which hold no position that counts) are replaced by its
-// first or last.
+// else those outside its whole words first .. last read as 0.
 template <bool INNER>
 __device__ __forceinline__ void add_channels(uint32_t (&A)[4][4], uint32_t (&O)[4][4], const uint8_t* x, int64_t nsamp,
                                              const int32_t* dl, int nc, const uint8_t* first, const uint8_t* last)
@@ -118,8 +117,7 @@ __device__ __forceinline__ void add_channels(uint32_t (&A)[4][4], uint32_t (&O)[
 #pragma unroll
         for (int m = 0; m < 4; m++) {
             const uint8_t* am = a + 128 * m;
-            if (!INNER) am = am < first ? first : am > last ? last : am;
-            w[m] = __ldg(reinterpret_cast<const uint32_t*>(am));
+            w[m] = INNER || (am >= first && am <= last) ? __ldg(reinterpret_cast<const uint32_t*>(am)) : 0u;
         }
         x += nsamp;
         return sh;
@@ -144,6 +142,23 @@ __device__ __forceinline__ void add_channels(uint32_t (&A)[4][4], uint32_t (&O)[
 
 // Position of window position q of a chunk in the staged chunk.
 __device__ __forceinline__ int staged(int q) { return q + (q >> 4) * 4; }
+
+// An input that starts mis bytes after a 4-byte address: adds its bytes outside the
+// whole words (the first 4 - mis, of channel 0, and the last mis, of the last
+// channel) into the staged chunk of channels c .. c + nc - 1 (delays dl), n
+// positions from sample s0 on.
+__device__ __noinline__ void add_ends(int32_t* st, int lane, const uint8_t* X, int64_t nsamp, int nchan, int mis, int c,
+                                      int nc, const int32_t* dl, int64_t s0, int n, int64_t nout)
+{
+    const bool head = lane < 4 - mis && c == 0, tail = lane >= 4 - mis && lane < 4 && c + nc == nchan;
+    if (head || tail) {
+        const int64_t at = head ? lane : nsamp - 4 + lane;  // sample of its channel
+        const int64_t q = at - dl[head ? 0 : nc - 1] - s0;
+        if (q >= 0 && q < n && s0 + q >= 0 && s0 + q < nout)
+            st[staged((int)q)] += __ldg(X + (int64_t)(head ? 0 : nchan - 1) * nsamp + at);
+    }
+    __syncwarp();
+}
 
 // The candidate of rank `rank` when all n <= kSortMax are taken widest first (by
 // the widths' binary order of magnitude, then by index).  mask: kSortMax / 32 rows of
@@ -210,11 +225,13 @@ __device__ int ranked(const af_cand_t* __restrict__ cands, int n, int rank, uint
 // cut out and classified: 477 us (880 to 920 with 16-byte loads realigned by shuffles
 // and masked per channel, 64-bit bins and plane values loaded 64 bytes apart);
 // 3 CTAs per SM with 4 channels in flight a warp: 473, 2 with 8: 479, 4 with 2: 539.
+// Inputs at any byte address (1024 channels, rows off a 4-byte address, 64 candidates
+// of width 16: 93 us byte by byte, 33 so).
 // Clusters take the widest candidates of a list of moderate length first, so that no
 // long one starts last: in the list's order 625 us.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(T, 3)
 k_cutout(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int32_t* __restrict__ D, int ndm,
-         const int32_t* __restrict__ plane, int64_t nout, const af_cand_t* __restrict__ cands, int n, bool order, bool vec,
+         const int32_t* __restrict__ plane, int64_t nout, const af_cand_t* __restrict__ cands, int n, bool order,
          __nv_bfloat16* __restrict__ out)
 {
     __shared__ unsigned long long wbins[NWARP][2][S];  // per warp: bins of its DM-time and frequency-time rows
@@ -269,7 +286,10 @@ k_cutout(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int32_t*
         }
     }
     // frequency-time row: channels row * gsz .. (row + 1) * gsz
-    const int64_t last_word = (int64_t)nchan * nsamp - 4;  // nchan is a multiple of 64: whole words
+    // the input's first and last whole word; at a 4-byte address they hold all of it (nchan is a multiple of 64)
+    const int mis = (int)(reinterpret_cast<uintptr_t>(X) & 3);
+    const uint8_t* const first = X + (4 - mis) % 4;
+    const uint8_t* const last = X + (int64_t)nchan * nsamp - 4 - mis;
     const int32_t* dl = dsh ? sD + (row * gsz - cb) : D + (int64_t)d * nchan + row * gsz;  // the row's delays
     for (int p0 = 0; p0 < span; p0 += CHF) {
         const int64_t s0 = start + p0;  // sample of the chunk's first position
@@ -280,34 +300,18 @@ k_cutout(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int32_t*
             const int nc = min(256, gsz - c0);
             const uint8_t* x = X + (int64_t)(row * gsz + c0) * nsamp + s0;
             uint32_t u[4][4];  // column sums of positions 4 (lane + 32 m) + k, at most 255 * 256
-            if (vec) {
-                uint32_t A[4][4], O[4][4];
+            uint32_t A[4][4], O[4][4];
 #pragma unroll
-                for (int q = 0; q < 4; q++)
+            for (int q = 0; q < 4; q++)
 #pragma unroll
-                    for (int m = 0; m < 4; m++) A[q][m] = O[q][m] = 0u;
-                if (inner) add_channels<true>(A, O, x + 4 * lane, nsamp, dl + c0, nc, X, X + last_word);
-                else add_channels<false>(A, O, x + 4 * lane, nsamp, dl + c0, nc, X, X + last_word);
+                for (int m = 0; m < 4; m++) A[q][m] = O[q][m] = 0u;
+            if (inner) add_channels<true>(A, O, x + 4 * lane, nsamp, dl + c0, nc, first, last);
+            else add_channels<false>(A, O, x + 4 * lane, nsamp, dl + c0, nc, first, last);
 #pragma unroll
-                for (int m = 0; m < 4; m++)
+            for (int m = 0; m < 4; m++)
 #pragma unroll
-                    for (int k = 0; k < 4; k++) u[m][k] = 0u;
-                aftile::Tile<1, 4>::fold(A, O, u, lane);
-            } else {  // byte by byte
-#pragma unroll
-                for (int m = 0; m < 4; m++)
-#pragma unroll
-                    for (int k = 0; k < 4; k++) u[m][k] = 0u;
-#pragma unroll 1
-                for (int c = 0; c < nc; c++, x += nsamp)
-#pragma unroll
-                    for (int m = 0; m < 4; m++)
-#pragma unroll
-                        for (int k = 0; k < 4; k++) {
-                            const int p = 4 * (lane + 32 * m) + k;
-                            if (s0 + p >= 0 && s0 + p < nout) u[m][k] += __ldg(x + dl[c0 + c] + p);
-                        }
-            }
+                for (int k = 0; k < 4; k++) u[m][k] = 0u;
+            aftile::Tile<1, 4>::fold(A, O, u, lane);
 #pragma unroll
             for (int m = 0; m < 4; m++) {
                 const int p = 4 * (lane + 32 * m);
@@ -321,6 +325,7 @@ k_cutout(const uint8_t* __restrict__ X, int64_t nsamp, int nchan, const int32_t*
                 *reinterpret_cast<uint4*>(st + staged(p)) = make_uint4(u[m][0], u[m][1], u[m][2], u[m][3]);
             }
             __syncwarp();
+            if (mis && !inner) add_ends(st, lane, X, nsamp, nchan, mis, row * gsz + c0, nc, dl + c0, s0, min(CHF, span - p0), nout);
             add_bins(st, lane, p0 + 16 * lane, b, wbins[warp][1], fit);
             __syncwarp();
         }
@@ -388,12 +393,11 @@ int nn_cutouts(const uint8_t* X, int64_t nsamp, int nchan, const int32_t* D, int
 {
     if (n <= 0) return AF_OK;
     if ((long long)n * kCl > 0x7fffffffLL) return af_set_error(AF_EINVAL, "cut-outs: too many candidates for one grid");
-    const bool vec = (reinterpret_cast<uintptr_t>(X) & 3) == 0;  // 32-bit loads
     // Widest first pays where one wide candidate would start last, and costs every block a look at the whole list: worth
     // it up to about 9 waves of clusters (57 of them run at a time), twice that where a candidate's own work is longer.
     // 512 candidates, ordered / not: widths mixed 1 to 256, 4096 channels 805 / 945 us, 64 channels 238 / 242; width 1, 64
     // channels 130 / 115; 1024 at 4096 channels 1605 / 1772; 4000, every block ranking all (before): 7264 / 6340.
     const bool order = n > 8 && n <= (nchan >= 512 ? kSortMax : kSortMax / 2);
-    k_cutout<<<(unsigned)n * kCl, T, 0, s>>>(X, nsamp, nchan, D, ndm, plane, nout, cands, n, order, vec, out);
+    k_cutout<<<(unsigned)n * kCl, T, 0, s>>>(X, nsamp, nchan, D, ndm, plane, nout, cands, n, order, out);
     return af_cuda_check(cudaGetLastError(), "cut-out launch");
 }

@@ -1,5 +1,6 @@
-"""Cut-outs of candidate lists around the lengths up to which they are taken widest
-first, bit-exact against the oracle."""
+"""Cut-outs of inputs at every byte address (words across the input's ends) and of
+candidate lists around the lengths up to which they are taken widest first,
+bit-exact against the oracle."""
 import numpy as np
 import pytest
 
@@ -38,6 +39,17 @@ def _cutouts(X, dms, cands, offset=0):
     torch.cuda.synchronize()
     p.close()
     return out.float().cpu().numpy().transpose(0, 3, 1, 2), D, Y
+
+
+@pytest.mark.parametrize("nchan,nsamp", [(64, 2001), (320, 1503)])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3, 7])
+def test_input_addresses(nchan, nsamp, offset):
+    X = np.random.default_rng(nsamp + offset).integers(1, 256, (nchan, nsamp), dtype=np.uint8)
+    dms = np.arange(9.0)
+    nout = nsamp - int(oracle.delay_table(nchan, *BAND, TSAMP, dms).max())
+    cands = [(d, t, w) for d, w in ((0, 1), (8, 2), (4, 9), (8, 40), (0, 256)) for t in (0, 1, 2, 31, nout // 2, nout - 33, nout - 1)]
+    got, D, Y = _cutouts(X, dms, cands, offset)
+    assert np.array_equal(got, cutout.cutouts(X, D, Y, cands))
 
 
 @pytest.mark.parametrize("nchan,n", [(64, 8), (64, 9), (64, 31), (64, 33), (64, 511), (64, 512), (64, 513), (512, 1023),
