@@ -179,7 +179,8 @@ __device__ int ranked(const af_cand_t* __restrict__ cands, int n, int rank, uint
         const int c = warp + k * NWARP;
         if (c >= chunks) break;  // the same in every lane
         mask[32 * c + lane] = 0u;
-        const uint32_t m = __match_any_sync(0xffffffffu, cls[k]);  // also orders the clear before the store
+        __syncwarp();  // the clear comes before the store
+        const uint32_t m = __match_any_sync(0xffffffffu, cls[k]);
         if (cls[k] < 32 && lane == __ffs(m) - 1) mask[32 * c + cls[k]] = m;
     }
     __syncthreads();
