@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace cg = cooperative_groups;
@@ -216,9 +218,10 @@ try {
 // Zero-DM filter: q[t] = round_half_up(sum_c X[c][t] / nchan), out = clip(X - q + 128).
 // Up to 4096 channels, a cluster of 1, 2, 4 or 8 blocks owns a tile of 128
 // samples of every channel and holds it in shared memory, so that the input is
-// read once (k_zerodm_tile).  More channels: a block owns 512 samples of every
-// channel and reads them twice (k_zerodm16: rows of whole 16-byte pieces), or
-// one thread per 4 samples (k_zerodm, any shape).
+// read once (k_zerodm_tile).  More channels, and long rows of few (whose tiles would
+// leave most of a block idle): a block owns 512 samples of every channel and
+// reads them twice (k_zerodm16: rows of whole 16-byte pieces), or one thread per 4
+// samples (k_zerodm, any shape).
 // In place is safe: a tile's samples are read before any of them is written,
 // and only its own bytes are written.
 namespace {
@@ -429,7 +432,9 @@ k_zerodm16(const uint8_t* X, int nchan, int64_t nsamp, uint8_t* out)
     __shared__ int32_t q[kZTile];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t t0 = (int64_t)blockIdx.x * kZTile + 16 * lane;
-    const int c0 = (int)((int64_t)nchan * warp / kZW), c1 = (int)((int64_t)nchan * (warp + 1) / kZW);
+    const int c0 = (int)((int64_t)nchan * warp / kZW);
+    // the lane's 16 samples are in the row, or all past it: no channels then
+    const int c1 = t0 < nsamp ? (int)((int64_t)nchan * (warp + 1) / kZW) : c0;
     uint32_t sum[16];
 #pragma unroll
     for (int i = 0; i < 16; i++) sum[i] = 0u;
@@ -514,12 +519,18 @@ try {
     if (!d_in || !d_out) return af_set_error(AF_EINVAL, "af_zerodm: NULL buffer");
     if (nchan < 1 || nchan > 65536 || nsamp < 1) return af_set_error(AF_EINVAL, "af_zerodm: bad shape");
     cudaStream_t s = (cudaStream_t)stream;
-    if (nchan <= 8 * kZC) {
-        // blocks per tile: the fewest that hold every channel
-        int parts = 1;
-        while (parts * kZC < nchan) parts *= 2;
-        const int64_t tiles = (nsamp + kZS - 1) / kZS;
-        if (tiles * parts > 0x7fffffff) return af_set_error(AF_EINVAL, "af_zerodm: input too large");
+    const bool aligned = nsamp % 16 == 0 && ((uintptr_t)d_in % 16 == 0) && ((uintptr_t)d_out % 16 == 0);
+    // Blocks per tile: the fewest that hold every channel.  Long rows of few channels go to the kernels that read twice.  Tile /
+    // those, us: 1 x 2^24 aligned 385 / 31, off a boundary 1328 / 31; 16 x 2^24 523 / 373 and 1866 / 302; 64 x 2^23 354 / 298 and
+    // 1253 / 725; 96 x 2^22 174 / 189; 128 x 2^22 236 / 244 and 923 / 823; 256 x 2^21 178 / 237 and 742 / 857; 64 x 2^14 4.2 / 6.2 and 6.2 / 47.
+    int parts = 1;
+    while (parts * kZC < nchan) parts *= 2;
+    const int64_t tiles = (nsamp + kZS - 1) / kZS;
+    // (k_zerodm16 wants a channel for each of its warps.)
+    const bool few = nchan <= 2 ||
+                     (aligned ? nchan < 72 && nsamp >= (nchan < kZW ? std::max(65536, 16384 * nchan) : 65536)
+                              : nchan < 160 && nsamp >= 4096 * (int64_t)nchan);
+    if (nchan <= 8 * kZC && !few && tiles * parts <= 0x7fffffff) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(tiles * parts));
         cfg.blockDim = dim3(kZW * 32);
@@ -530,7 +541,6 @@ try {
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        const bool aligned = nsamp % 16 == 0 && ((uintptr_t)d_in % 16 == 0) && ((uintptr_t)d_out % 16 == 0);
         cfg.dynamicSmemBytes = aligned ? kZSmemA : kZSmemU;
         if (int rc = af_ensure_smem(aligned ? (const void*)k_zerodm_tile<true> : (const void*)k_zerodm_tile<false>,
                                     cfg.dynamicSmemBytes))
@@ -539,9 +549,8 @@ try {
                                      : cudaLaunchKernelEx(&cfg, k_zerodm_tile<false>, d_in, nchan, nsamp, d_out),
                              "af_zerodm launch");
     }
-    const bool fast = nsamp % kZTile == 0 && ((uintptr_t)d_in % 16 == 0) && ((uintptr_t)d_out % 16 == 0);
-    if (fast) {
-        const int64_t blocks = nsamp / kZTile;
+    if (aligned && nchan >= kZW) {
+        const int64_t blocks = (nsamp + kZTile - 1) / kZTile;
         if (blocks > 0x7fffffff) return af_set_error(AF_EINVAL, "af_zerodm: input too large");
         k_zerodm16<<<(unsigned)blocks, kZW * 32, 0, s>>>(d_in, nchan, nsamp, d_out);
     } else {
