@@ -422,6 +422,7 @@ k_zerodm_tile(const uint8_t* X, int nchan, int64_t nsamp, uint8_t* out)
             __syncwarp();
         }
     }
+    __syncwarp();  // lanes past the row or its channels ran fewer steps
     if (parts > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
