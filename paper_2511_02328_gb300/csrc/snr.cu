@@ -418,27 +418,27 @@ __device__ __forceinline__ uint32_t robust_key(int32_t v, int32_t base)
     return v >= base ? (uint32_t)v - (uint32_t)base : (uint32_t)base - (uint32_t)v;
 }
 
-// Calls f(v) for every value of the row y[0 .. n), spread over the block: a
-// scalar head up to the first 16-byte boundary, then kRU4 16-byte loads per
-// thread in flight per step, then the scalar tail.
+// Calls f(v) for every value of part `part` of `parts` of the row y[0 .. n), spread
+// over the block: kRU4 16-byte loads per thread in flight per step; the first
+// part also takes the values before the first 16-byte boundary and after the last.
 constexpr int kRU4 = 4;
 template <typename F>
-__device__ __forceinline__ void for_row(const int32_t* __restrict__ y, int64_t n, F&& f)
+__device__ __forceinline__ void for_row(const int32_t* __restrict__ y, int64_t n, int part, int parts, F&& f)
 {
     const int tid = threadIdx.x;
     int64_t head = (int64_t)(((16u - ((uint32_t)reinterpret_cast<uintptr_t>(y) & 15u)) & 15u) >> 2);
     if (head > n) head = n;
-    if (tid < head) f(__ldg(y + tid));
+    if (part == 0 && tid < head) f(__ldg(y + tid));
     const int4* y4 = reinterpret_cast<const int4*>(y + head);
-    const int64_t n4 = (n - head) >> 2;
-    for (int64_t i = tid; i < n4; i += (int64_t)kRT * kRU4) {
+    const int64_t n4 = (n - head) >> 2, q1 = n4 * (part + 1) / parts;
+    for (int64_t i = n4 * part / parts + tid; i < q1; i += (int64_t)kRT * kRU4) {
         int4 v[kRU4];
 #pragma unroll
         for (int u = 0; u < kRU4; u++)
-            if (i + u * kRT < n4) v[u] = __ldg(y4 + i + u * kRT);
+            if (i + u * kRT < q1) v[u] = __ldg(y4 + i + u * kRT);
 #pragma unroll
         for (int u = 0; u < kRU4; u++)
-            if (i + u * kRT < n4) {
+            if (i + u * kRT < q1) {
                 f(v[u].x);
                 f(v[u].y);
                 f(v[u].z);
@@ -446,7 +446,7 @@ __device__ __forceinline__ void for_row(const int32_t* __restrict__ y, int64_t n
             }
     }
     const int64_t t0 = head + 4 * n4;
-    if (t0 + tid < n) f(__ldg(y + t0 + tid));  // at most 3 values
+    if (part == 0 && t0 + tid < n) f(__ldg(y + t0 + tid));  // at most 3 values
 }
 
 // Block sum of one int64 per thread, returned to every thread (sred: kRT/32 slots).
@@ -463,64 +463,96 @@ __device__ __forceinline__ long long block_sum(long long x, long long* sred)
     return t;
 }
 
+// Scratch of the selection over a row, by one block or by the blocks of a cluster
+// (each one part of the row; every block adds up all blocks' counts through
+// distributed shared memory and so takes the same decisions).
+struct RobustScratch {
+    alignas(16) uint32_t hist[kRB];  // 4 bins a thread (16 bytes)
+    uint32_t wsum[kRT / 32];
+    int64_t found[2];                // a search's bin (-1: none) and the count before it
+    long long sred[kRT / 32];
+    int32_t smin[kRT / 32], smax[kRT / 32];
+    float ssq[kRT / 32];
+    // read by a cluster's other blocks
+    long long below, su;             // values below the window; sum of v - y[0]
+    int32_t lo, hi;
+    double m2;
+};
+static_assert(kRB == 4 * kRT, "four bins a thread");
+
 // The rank-th smallest key (0-based) among the row's keys in [0, width).  For
 // MODE 0, rank counts from the row's smallest value: the first pass counts
 // the values under `base` (none when base is the row minimum).  Returns false,
 // with every thread agreeing, when the first pass shows the rank outside the
 // window.
-template <int MODE>
-__device__ bool robust_select(const int32_t* __restrict__ y, int64_t n, int32_t base, uint64_t width, int64_t rank,
-                              uint32_t* hist, long long* sel, long long* sred, uint32_t* out)
+template <int MODE, bool CLUSTER>
+__device__ bool robust_select(const int32_t* __restrict__ y, int64_t n, int part, int parts, int32_t base,
+                              uint64_t width, int64_t rank, RobustScratch& sc, uint32_t* out)
 {
     uint32_t start = 0;
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     bool first = true;
     while (first || width > 1) {
         const int bits = width > 1 ? 64 - __clzll((long long)(width - 1)) : 0;
         const int s = bits > 11 ? bits - 11 : 0;
-        for (int i = tid; i < kRB; i += kRT) hist[i] = 0u;
+        reinterpret_cast<uint4*>(sc.hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
+        if (tid == 0) sc.found[0] = -1;
         __syncthreads();
         long long below = 0;
         const bool count_below = MODE == 0 && first;
-        for_row(y, n, [&](int32_t v) {
+        for_row(y, n, part, parts, [&](int32_t v) {
             const uint32_t k = robust_key<MODE>(v, base);
-            if (k >= start && (uint64_t)(k - start) < width) atomicAdd(&hist[(k - start) >> s], 1u);
+            if (k >= start && (uint64_t)(k - start) < width) atomicAdd(&sc.hist[(k - start) >> s], 1u);
             else if (count_below && v < base) below++;
         });
-        if (MODE == 0 && first) rank -= block_sum(below, sred);  // syncs the block
-        else __syncthreads();
-        if (tid < 32) {
-            // lane l owns bins [64 l, 64 l + 64): find the bin where the count passes rank
-            uint32_t own = 0;
-#pragma unroll 8
-            for (int i = 0; i < 64; i++) own += hist[lane * 64 + i];
-            uint32_t incl = own;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
+        if (count_below) below = block_sum(below, sc.sred);  // syncs the block
+        else if (!CLUSTER) __syncthreads();
+        uint4 h;
+        if (CLUSTER) {
+            cg::cluster_group cluster = cg::this_cluster();
+            if (tid == 0) sc.below = below;
+            cluster.sync();  // every block's counts are complete
+            h = make_uint4(0u, 0u, 0u, 0u);
+            below = 0;
+            for (int r = 0; r < parts; r++) {
+                const RobustScratch* o = cluster.map_shared_rank(&sc, r);
+                const uint4 c = reinterpret_cast<const uint4*>(o->hist)[tid];
+                h.x += c.x;
+                h.y += c.y;
+                h.z += c.z;
+                h.w += c.w;
+                if (count_below) below += o->below;
             }
-            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-            if (lane == 0) sel[2] = (rank >= 0 && rank < (int64_t)total) ? 1 : 0;
-            const uint32_t excl = incl - own;
-            if ((int64_t)excl <= rank && rank < (int64_t)incl) {
-                int64_t cum = excl;
-#pragma unroll 1
-                for (int i = 0; i < 64; i++) {
-                    const uint32_t h = hist[lane * 64 + i];
-                    if (rank < cum + (int64_t)h) {
-                        sel[0] = lane * 64 + i;
-                        sel[1] = cum;
-                        break;
-                    }
-                    cum += h;
-                }
-            }
+        } else {
+            h = reinterpret_cast<const uint4*>(sc.hist)[tid];
         }
+        if (count_below) rank -= below;
+        // the bin where the running count passes rank (bins in the threads' order)
+        const uint32_t own = h.x + h.y + h.z + h.w;
+        uint32_t incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) sc.wsum[warp] = incl;
         __syncthreads();
-        if (!sel[2]) return false;  // only on a first pass: later windows hold the rank by construction
-        const uint32_t b = (uint32_t)sel[0];
-        rank -= sel[1];
+        int64_t cum = (int64_t)(incl - own);
+        for (int k = 0; k < warp; k++) cum += sc.wsum[k];
+        if (cum <= rank && rank < cum + (int64_t)own) {
+            int b = 0;
+            if (rank >= cum + h.x) cum += h.x, b = 1;
+            if (b == 1 && rank >= cum + h.y) cum += h.y, b = 2;
+            if (b == 2 && rank >= cum + h.z) cum += h.z, b = 3;
+            sc.found[0] = 4 * tid + b;
+            sc.found[1] = cum;
+        }
+        // the answer, and no block clears counts that another still reads
+        if (CLUSTER) cg::this_cluster().sync();
+        else __syncthreads();
+        if (sc.found[0] < 0) return false;  // only on a first pass: later windows hold the rank by construction
+        const uint32_t b = (uint32_t)sc.found[0];
+        rank -= sc.found[1];
         start += b << s;
         const uint64_t left = width - ((uint64_t)b << s);
         width = left < ((uint64_t)1 << s) ? left : ((uint64_t)1 << s);
@@ -531,21 +563,13 @@ __device__ bool robust_select(const int32_t* __restrict__ y, int64_t n, int32_t 
     return true;
 }
 
-// Scratch of the selection over a whole row by one block.
-struct RobustScratch {
-    uint32_t hist[kRB];
-    long long sel[3];
-    long long sred[kRT / 32];
-    int32_t smin[kRT / 32], smax[kRT / 32];
-    float ssq[kRT / 32];
-};
-
 // Median and MAD of a row in up to three passes (the windows above).
-__device__ __noinline__ void row_robust_general(const int32_t* __restrict__ y, int64_t nout, RobustScratch& sc,
-                                   af_robust_t* __restrict__ out)
+template <bool CLUSTER>
+__device__ __noinline__ void row_robust_general(const int32_t* __restrict__ y, int64_t nout, int part_, int parts_,
+                                                RobustScratch& sc, af_robust_t* __restrict__ out)
 {
-    uint32_t* hist = sc.hist;
-    long long *sel = sc.sel, *sred = sc.sred;
+    const int part = CLUSTER ? part_ : 0, parts = CLUSTER ? parts_ : 1;
+    long long* sred = sc.sred;
     int32_t *smin = sc.smin, *smax = sc.smax;
     float* ssq = sc.ssq;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -554,7 +578,7 @@ __device__ __noinline__ void row_robust_general(const int32_t* __restrict__ y, i
     int32_t lo = INT32_MAX, hi = INT32_MIN;
     long long su = 0;
     float sq = 0.0f;
-    for_row(y, nout, [&](int32_t v) {
+    for_row(y, nout, part, parts, [&](int32_t v) {
         lo = min(lo, v);
         hi = max(hi, v);
         su += (long long)v - y0;
@@ -583,6 +607,25 @@ __device__ __noinline__ void row_robust_general(const int32_t* __restrict__ y, i
         hi = max(hi, smax[i]);
         m2 += (double)ssq[i];
     }
+    if (CLUSTER) {
+        cg::cluster_group cluster = cg::this_cluster();
+        if (tid == 0) {
+            sc.lo = lo;
+            sc.hi = hi;
+            sc.su = su;
+            sc.m2 = m2;
+        }
+        cluster.sync();
+        su = 0;
+        m2 = 0.0;
+        for (int r = 0; r < parts; r++) {
+            const RobustScratch* o = cluster.map_shared_rank(&sc, r);
+            lo = min(lo, o->lo);
+            hi = max(hi, o->hi);
+            su += o->su;
+            m2 += o->m2;
+        }
+    }
     const double nn = (double)nout, mean_u = (double)su / nn;
     m2 /= nn;
     // s >= sigma: the fp32 sums of u^2 (about nout / 512 terms per thread, then 32
@@ -596,18 +639,18 @@ __device__ __noinline__ void row_robust_general(const int32_t* __restrict__ y, i
     const int64_t wh = min((int64_t)hi, (int64_t)ceil(mu + sb) + 1);
     uint32_t key = 0;
     int32_t med;
-    if (wl <= wh && robust_select<0>(y, nout, (int32_t)wl, (uint64_t)(wh - wl) + 1, k, hist, sel, sred, &key))
+    if (wl <= wh && robust_select<0, CLUSTER>(y, nout, part, parts, (int32_t)wl, (uint64_t)(wh - wl) + 1, k, sc, &key))
         med = (int32_t)((uint32_t)(int32_t)wl + key);  // a row value: no overflow in the sum
     else {  // the same selection over the whole range [lo, hi]
-        robust_select<0>(y, nout, lo, (uint64_t)((int64_t)hi - lo) + 1, k, hist, sel, sred, &key);
+        robust_select<0, CLUSTER>(y, nout, part, parts, lo, (uint64_t)((int64_t)hi - lo) + 1, k, sc, &key);
         med = (int32_t)((uint32_t)lo + key);
     }
     const int64_t r2 = max((int64_t)hi - med, (int64_t)med - lo);
     const int64_t wm = min(r2, (int64_t)ceil(2.0 * sb) + 1);
     uint32_t mad = 0;
-    if (!robust_select<1>(y, nout, med, (uint64_t)wm + 1, k, hist, sel, sred, &mad))
-        robust_select<1>(y, nout, med, (uint64_t)r2 + 1, k, hist, sel, sred, &mad);
-    if (tid == 0) {
+    if (!robust_select<1, CLUSTER>(y, nout, part, parts, med, (uint64_t)wm + 1, k, sc, &mad))
+        robust_select<1, CLUSTER>(y, nout, part, parts, med, (uint64_t)r2 + 1, k, sc, &mad);
+    if (tid == 0 && part == 0) {
         out->median = med;
         out->mad = mad;
     }
@@ -617,12 +660,13 @@ __global__ void __launch_bounds__(kRT, 2) k_row_robust(const int32_t* __restrict
                                                     af_robust_t* __restrict__ out)
 {
     __shared__ RobustScratch sc;
-    row_robust_general(Y + (int64_t)blockIdx.x * nout, nout, sc, out + blockIdx.x);
+    row_robust_general<false>(Y + (int64_t)blockIdx.x * nout, nout, 0, 1, sc, out + blockIdx.x);
 }
 
-// ---- long rows: one pass.  A sample of 4096 values (1024 16-byte pieces at
-// even steps) gives estimates m of the median and M of the MAD, good to a few
-// hundredths of sigma on any smooth distribution.  One pass over the row then
+// ---- long rows: one pass.  A sample of 4096 values (1024 16-byte pieces, one at a
+// scattered place in each of as many equal stretches) gives estimates m of the
+// median and M of the MAD, good to a few hundredths of sigma on any smooth
+// distribution.  One pass over the row then
 // counts, at unit resolution, the values in three windows -- around m, m - M
 // and m + M, each a few estimate errors wide -- and the values below each
 // window.  Cumulative counts C(z) = #(v < z) are therefore exact for z inside a
@@ -630,9 +674,14 @@ __global__ void __launch_bounds__(kRT, 2) k_row_robust(const int32_t* __restrict
 // (the smallest x with C(med + x + 1) - C(med - x) > k) follow without another
 // pass: both are checked against the windows' edges, and a row whose answer
 // lies outside them (none seen on noise) takes the general selection.  Where
-// the windows meet (M of a few units) one dense window covers them all.
+// the windows meet (M of a few units) one dense window covers them all.  A row
+// whose windows would not fit the bins (M above some 5600), or whose sample has
+// too few values near its median to trust that estimate (two far-apart modes),
+// goes to the general selection without that pass.
 // A cluster of blocks shares a row, each counting one part; the first block
-// adds up the others' counts through distributed shared memory.  Bound by issue
+// adds up the others' counts through distributed shared memory.  The general
+// selection is shared as well where the sample asks for it (left to the first block,
+// 500 x 200001 rows that need it took 885 us, 590 so).  Bound by issue
 // (about 25 instructions per 32 values, the three window tests and counts) and
 // HBM: 1001 x 215261 plane 0.53 ms in three passes, 0.24 ms in one.
 // Rows below 16384 values keep the general selection: the sample would be a
@@ -645,9 +694,10 @@ struct RobustOnePass {
     union {
         RobustScratch gen;
         struct {
-            uint32_t hist[kRH];           // counts per bin, then exclusive prefix sums
+            alignas(16) uint32_t hist[kRH];  // counts per bin, then exclusive prefix sums (read 16 bytes at a time)
             uint32_t wsum[kRT / 32];
             uint32_t below[3];            // values below each window (of this block's part)
+            uint32_t near[kRT / 32];      // per warp: sample values near the median, two counts a word
             int32_t lo, hi;               // sample range
             uint32_t bin, cum;            // a search's answer
             int32_t med, mad;
@@ -714,7 +764,8 @@ __device__ __forceinline__ uint32_t sample_median(const uint32_t (&key)[kRS / kR
 __global__ void __launch_bounds__(kRT, 2)
 k_row_robust1(const int32_t* __restrict__ Y, int64_t nout, af_robust_t* __restrict__ out)
 {
-    __shared__ __align__(16) RobustOnePass sc;
+    extern __shared__ __align__(16) uint8_t robust_smem[];
+    RobustOnePass& sc = *reinterpret_cast<RobustOnePass*>(robust_smem);
     cg::cluster_group cluster = cg::this_cluster();
     const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
     const int64_t d = blockIdx.x / parts;
@@ -730,7 +781,8 @@ k_row_robust1(const int32_t* __restrict__ Y, int64_t nout, af_robust_t* __restri
         const int64_t step = n4 / (kRS / 4);
 #pragma unroll
         for (int j = 0; j < kRS / kRT / 4; j++) {
-            const int4 v = __ldg(y4 + (tid + j * kRT) * step);
+            const uint32_t piece = tid + j * kRT;  // even steps would see one phase of a periodic row
+            const int4 v = __ldg(y4 + piece * step + __umulhi(piece * 2654435761u, (uint32_t)step));
             sv[4 * j] = v.x;
             sv[4 * j + 1] = v.y;
             sv[4 * j + 2] = v.z;
@@ -775,7 +827,21 @@ k_row_robust1(const int32_t* __restrict__ Y, int64_t nout, af_robust_t* __restri
     const bool dense = in <= dc;
     const int64_t bins = dense ? 2 * (int64_t)outer + 1 : 2 * (int64_t)dc + 1 + 2 * (2 * (int64_t)dw + 1);
     // windows inside the int32 range, so that (v - start) mod 2^32 < width exactly for the values in them
-    const bool fits = sane && bins <= kRH && (int64_t)m - outer >= INT32_MIN && (int64_t)m + outer < INT32_MAX;
+    const bool inside = sane && bins <= kRH && (int64_t)m - outer >= INT32_MIN && (int64_t)m + outer < INT32_MAX;
+    // The median's rank must fall into its window: some values between the estimate and the window's edges, in a quarter
+    // of the sample from all over the row (a normal one has 39 +- 6 on either side, and the rank an error of 8 there).
+    bool fits = inside;
+    if (inside) {  // the same in every thread
+        const uint32_t wm = dense ? outer : dc;
+        auto near = [&](int j) -> uint32_t {  // at or below m | at or above
+            return key[j] > wm ? 0u : (sv[j] <= m ? 1u : 0u) + (sv[j] >= m ? 1u << 16 : 0u);
+        };
+        const uint32_t c = __reduce_add_sync(0xffffffffu, near(0) + near(kRS / kRT / 2));
+        if (lane == 0) sc.one.near[tid >> 5] = c;
+        __syncthreads();
+        const uint32_t n = __reduce_add_sync(0xffffffffu, sc.one.near[lane & 15]) >> 1;  // every warp's count twice
+        fits = min(n & 0xFFFFu, n >> 16) >= 16;
+    }
     // window starts (as v - m), widths and first bins: below m - M, around m, above m + M; dense: the first alone
     const int32_t w0 = -outer, w1 = -dc, w2 = in;
     const int nb0 = dense ? 2 * outer + 1 : 2 * dw + 1, nb1 = dense ? 0 : 2 * dc + 1, nb2 = dense ? 0 : 2 * dw + 1;
@@ -918,7 +984,8 @@ k_row_robust1(const int32_t* __restrict__ Y, int64_t nout, af_robust_t* __restri
         __syncthreads();
     }
     cluster.sync();  // the first block has read the others' shared memory
-    if (part == 0 && !done) row_robust_general(y, nout, sc.gen, out + d);
+    if (!fits && parts > 1) row_robust_general<true>(y, nout, part, parts, sc.gen, out + d);
+    else if (part == 0 && !done) row_robust_general<false>(y, nout, 0, 1, sc.gen, out + d);
 }
 
 // Robust S/N constants: snr = (B - w*med) * k, k = 1/(1.482602218505602 * mad * sqrt(w)).
@@ -945,13 +1012,18 @@ int af_launch_row_robust(const int32_t* d_plane, int ndm, int64_t nout, af_robus
         k_row_robust<<<ndm, kRT, 0, s>>>(d_plane, nout, d_robust);
         return af_cuda_check(cudaGetLastError(), "robust row statistics launch");
     }
-    // blocks per row: enough for two per SM, each with at least 32768 values
+    // blocks per row: enough for four waves of two per SM, each with at least 16384 values
+    int dev = 0, nsm = 0;
+    AF_CUDA(cudaGetDevice(&dev));
+    AF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     int parts = 1;
-    while (parts < 8 && (int64_t)ndm * parts < 1216 && nout / (2 * parts) >= 16384) parts *= 2;
+    while (parts < 8 && (int64_t)ndm * parts < 8 * nsm && nout / (2 * parts) >= 16384) parts *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(ndm * parts));
     cfg.blockDim = dim3(kRT);
+    cfg.dynamicSmemBytes = sizeof(RobustOnePass);
     cfg.stream = s;
+    if (int rc = af_ensure_smem((const void*)k_row_robust1, sizeof(RobustOnePass))) return rc;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)parts;
