@@ -77,17 +77,18 @@ __device__ __forceinline__ uint32_t gray(unsigned long long a, unsigned long lon
     return y;
 }
 
-// Area path.  Block = (slice, output row i, run of kGT output columns): the
-// plane rows that row i covers are added, weighted, column by column with
-// coalesced loads into V[c] = sum_r ovr(i, r) X[r][c] (shared memory, as many
-// columns at a time as fit), and thread j sums its pixel's columns from there, the
-// first and last weighted.  V is int32 while every value of the block's columns is
-// non-negative and (their bitwise or) x h is below 2^31 (planes of 8-bit sums);
-// otherwise the block starts again with int64.  PASS 0: min / max into work;
-// PASS 1: write Y.
+// Area path by columns, for wide pixels.  Block = (slice, output row i, run of kGT
+// output columns): the plane rows that row i covers are added, weighted, column by
+// column with coalesced loads into V[c] = sum_r ovr(i, r) X[r][c] (shared memory, as
+// many columns at a time as fit), and thread j sums its pixel's columns from there,
+// the first and last weighted.  V is int32: valid while every value of the block's
+// columns is non-negative and (their bitwise or) x h is below 2^31 (planes of 8-bit
+// sums); otherwise the block starts again with int64, in pass 1 at once where the
+// slice's sums show that int32 would not do.
+// PASS 0: min / max into work; PASS 1: write Y.
 // Bound by HBM (the plane twice).  22 slices of 1001 x 10173 to 512 x 512: a pass
 // took 0.42 ms with every pixel loading its own 20 columns of 2 to 3 rows (lanes
-// 80 bytes apart) and 64-bit divisions per pixel, 0.31 ms with V in int64, 0.23 ms so
+// 80 bytes apart) and 64-bit divisions per pixel, 0.23 ms so
 // (latency: a block's loads, sums and reduction follow one another; rows staged by
 // asynchronous copies in 128-thread blocks took the same).
 constexpr int kGU = 5;                    // columns per thread and step
@@ -172,6 +173,28 @@ __device__ __forceinline__ int div_m(long long a, int M, bool small)
     return small ? (int)((uint32_t)a / (uint32_t)M) : (int)(a / M);
 }
 
+// W of pixel (i, j) of the slice that starts at column c0: its rows and columns
+// with their weights, in 64 bits.
+__device__ __forceinline__ long long area_pixel(const int32_t* __restrict__ X, int64_t nout, int h, int64_t c0, int w,
+                                                int M, int i, int j, bool small)
+{
+    const long long ri0 = (long long)i * h, ri1 = ri0 + h, cj0 = (long long)j * w, cj1 = cj0 + w;
+    const int r_lo = div_m(ri0, M, small), r_hi = div_m(ri1 - 1, M, small);
+    const int c_lo = div_m(cj0, M, small), c_hi = div_m(cj1 - 1, M, small);
+    // weights of the first and last row and column, M of the others
+    const int rl = (int)(min(ri1, (long long)(r_lo + 1) * M) - ri0), rh = (int)(ri1 - (long long)r_hi * M);
+    const int cl = (int)(min(cj1, (long long)(c_lo + 1) * M) - cj0), ch = (int)(cj1 - (long long)c_hi * M);
+    const int32_t* x = X + (int64_t)r_lo * nout + c0;
+    long long W = 0;
+    for (int r = r_lo; r <= r_hi; r++, x += nout) {
+        long long row = (long long)cl * __ldg(x + c_lo);
+        for (int c = c_lo + 1; c < c_hi; c++) row += (long long)M * __ldg(x + c);
+        if (c_hi > c_lo) row += (long long)ch * __ldg(x + c_hi);
+        W += row * (r == r_lo ? rl : r == r_hi ? rh : M);
+    }
+    return W;
+}
+
 template <int PASS>
 __global__ void __launch_bounds__(kGT, 4)
 k_grid_area(const int32_t* __restrict__ X, int h, int64_t nout, int64_t ns, int s0, int M, unsigned runs, int cols,
@@ -210,7 +233,8 @@ k_grid_area(const int32_t* __restrict__ X, int h, int64_t nout, int64_t ns, int 
         if (e == c_hi && a <= e) sum -= (unsigned long long)((long long)V[c_hi - k0] * out_hi);
         W = (long long)((unsigned long long)W + sum);
     };
-    bool wide = false;
+    const long long lo = PASS == 1 ? work[2 * s] : 0, hi = PASS == 1 ? work[2 * s + 1] : 0;
+    bool wide = lo < 0 || hi > (long long)w << 31;  // hi / w: the slice's largest mean column sum
     for (int k0 = b_lo; k0 <= b_hi && !wide; k0 += cols) {
         const int n = min(cols, b_hi + 1 - k0);
         int32_t* V = reinterpret_cast<int32_t*>(smem);
@@ -232,9 +256,34 @@ k_grid_area(const int32_t* __restrict__ X, int h, int64_t nout, int64_t ns, int 
     if (PASS == 0) {
         slice_minmax(j < M ? W : LLONG_MAX, j < M ? W : LLONG_MIN, work + 2 * s);
     } else if (j < M) {
+        const unsigned long long rng = (unsigned long long)(hi - lo);
+        out[((int64_t)s * M + i) * M + j] = rng == 0 ? (uint8_t)0 : (uint8_t)gray((unsigned long long)(W - lo), rng);
+    }
+}
+
+// Area path pixel by pixel, for narrow pixels.  Block = (slice, run of kGT of its
+// M x M pixels), thread = pixel: no shared memory, no barriers but the reduction's,
+// and no lane idle however small M is.  Bound by the loads' latency and the sums.
+// 257 x 257 to 256 x 256, 605 slices: 334 us by columns (343 with 64-bit divisions), 190 so;
+// 3 x 7 to 2 x 2, 200,000 slices: 3016 us by columns (1491), 493 so.
+template <int PASS>
+__global__ void __launch_bounds__(kGT)
+k_grid_pixel(const int32_t* __restrict__ X, int h, int64_t nout, int64_t ns, int s0, int M, unsigned runs,
+             long long* __restrict__ work, uint8_t* __restrict__ out)
+{
+    const unsigned blk = PASS == 0 ? blockIdx.x : gridDim.x - 1 - blockIdx.x;
+    const int s = s0 + (int)(blk / runs), e = (int)(blk % runs) * kGT + (int)threadIdx.x;
+    const int64_t c0 = (int64_t)s * ns;
+    const int w = (int)min(ns, nout - c0);
+    const bool in = e < M * M, small = (long long)M * max(h, w) + w < (1LL << 32);
+    const int i = e / M;
+    const long long W = in ? area_pixel(X, nout, h, c0, w, M, i, e - i * M, small) : 0;
+    if (PASS == 0) {
+        slice_minmax(in ? W : LLONG_MAX, in ? W : LLONG_MIN, work + 2 * s);
+    } else if (in) {
         const long long lo = work[2 * s];
         const unsigned long long rng = (unsigned long long)(work[2 * s + 1] - lo);
-        out[((int64_t)s * M + i) * M + j] = rng == 0 ? (uint8_t)0 : (uint8_t)gray((unsigned long long)(W - lo), rng);
+        out[(int64_t)s * M * M + e] = rng == 0 ? (uint8_t)0 : (uint8_t)gray((unsigned long long)(W - lo), rng);
     }
 }
 
@@ -345,29 +394,46 @@ k_grid_lanczos(const int32_t* __restrict__ X, int h, int64_t nout, int64_t ns, i
     if (PASS == 0) slice_minmax(lo, hi, work + 2 * s);
 }
 
+// Area path: pixel by pixel, or by columns.  Pixel / column time on planes of 60,000 at most, by the pixel's height x width in
+// samples: M = 256: 1 x 1 0.52, 1 x 12 0.57, 1 x 20 0.76, 2 x 12 0.71, 2 x 20 0.98, 4 x 6 0.72, 4 x 20 1.2, 8 x 3 0.97; M = 64: 1 x 1
+// 0.14, 2 x 20 0.51, 8 x 6 0.41, 8 x 20 0.96, 1 x 40 0.84; M = 2: all below 0.7.  (By columns lanes read consecutive samples; by
+// pixels they read w / M apart, and rows of a few pixels leave no block half idle.)
+bool by_pixel(int h, int64_t w, int M)
+{
+    const double a = (double)h * (double)w / ((double)M * M);  // samples of a pixel
+    return M <= 32 ? a <= 300.0
+                   : w <= 24 * (int64_t)M && (M < 256 ? a <= (M < 128 ? 100.0 : 56.0) : a <= 28.0 && h <= 6 * (int64_t)M);
+}
+
 // One pass over slices s0 .. s0 + n - 1, all on one path.
 int launch_pass(int pass, bool area, int n, cudaStream_t st, const int32_t* X, int h, int64_t nout, int64_t ns, int s0,
                 int M, long long* work, uint8_t* out)
 {
-    if (area) {
-        const int64_t w = ns < nout - (int64_t)s0 * ns ? ns : nout - (int64_t)s0 * ns;
-        const unsigned runs = (unsigned)((M + kGT - 1) / kGT);
-        const int64_t span = (std::min(M, kGT) * w + M - 1) / M + 1;  // columns of a block's run
-        const int cols = (int)std::max<int64_t>(2, (std::min<int64_t>(span, kGCBytes / 4) + 1) & ~1);
-        const size_t smem = (size_t)cols * 4;
-        const unsigned blocks = (unsigned)n * (unsigned)M * runs;
-        if (pass == 0) k_grid_area<0><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s0, M, runs, cols, work, out);
-        else k_grid_area<1><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s0, M, runs, cols, work, out);
-        return af_cuda_check(cudaGetLastError(), "af_grid launch");
-    }
-    // rows per block: as many as their plane rows fit (one row needs 8)
+    const int64_t w = ns < nout - (int64_t)s0 * ns ? ns : nout - (int64_t)s0 * ns;
+    const bool pixel = area && by_pixel(h, w, M);
+    // area by columns: runs of kGT output columns of one row, with the columns they cover in shared memory
+    const int64_t span = (std::min(M, kGT) * w + M - 1) / M + 1;
+    const int cols = (int)std::max<int64_t>(2, (std::min<int64_t>(span, kGCBytes / 4) + 1) & ~1);
+    // Lanczos: rows per block, as many as their plane rows fit (one row needs 8)
     const int ti = (int)std::max<int64_t>(1, std::min<int64_t>(kLI, (int64_t)(kLR - 9) * M / h));
     const unsigned iruns = (unsigned)((M + ti - 1) / ti), jruns = (unsigned)((M + kLJ - 1) / kLJ);
-    const unsigned blocks = (unsigned)n * iruns * jruns;
-    const void* fn = pass == 0 ? (const void*)k_grid_lanczos<0> : (const void*)k_grid_lanczos<1>;
-    if (int rc = af_ensure_smem(fn, kLSmem)) return rc;
-    if (pass == 0) k_grid_lanczos<0><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s0, M, ti, iruns, jruns, work, out);
-    else k_grid_lanczos<1><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s0, M, ti, iruns, jruns, work, out);
+    const unsigned runs = (unsigned)(((pixel ? M * M : M) + kGT - 1) / kGT);
+    const unsigned each = pixel ? runs : area ? (unsigned)M * runs : iruns * jruns;  // blocks of a slice
+    if (!area)
+        if (int rc = af_ensure_smem(pass == 0 ? (const void*)k_grid_lanczos<0> : (const void*)k_grid_lanczos<1>, kLSmem))
+            return rc;
+    const unsigned blocks = (unsigned)n * each;
+    if (pixel) {
+        if (pass == 0) k_grid_pixel<0><<<blocks, kGT, 0, st>>>(X, h, nout, ns, s0, M, runs, work, out);
+        else k_grid_pixel<1><<<blocks, kGT, 0, st>>>(X, h, nout, ns, s0, M, runs, work, out);
+    } else if (area) {
+        const size_t smem = (size_t)cols * 4;
+        if (pass == 0) k_grid_area<0><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s0, M, runs, cols, work, out);
+        else k_grid_area<1><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s0, M, runs, cols, work, out);
+    } else {
+        if (pass == 0) k_grid_lanczos<0><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s0, M, ti, iruns, jruns, work, out);
+        else k_grid_lanczos<1><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s0, M, ti, iruns, jruns, work, out);
+    }
     return af_cuda_check(cudaGetLastError(), "af_grid launch");
 }
 
