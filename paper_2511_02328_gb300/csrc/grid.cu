@@ -405,7 +405,8 @@ bool by_pixel(int h, int64_t w, int M)
                    : w <= 24 * (int64_t)M && (M < 256 ? a <= (M < 128 ? 100.0 : 56.0) : a <= 28.0 && h <= 6 * (int64_t)M);
 }
 
-// One pass over slices s0 .. s0 + n - 1, all on one path.
+// One pass over slices s0 .. s0 + n - 1, all on one path, in launches of as many
+// slices as a grid holds.
 int launch_pass(int pass, bool area, int n, cudaStream_t st, const int32_t* X, int h, int64_t nout, int64_t ns, int s0,
                 int M, long long* work, uint8_t* out)
 {
@@ -422,19 +423,23 @@ int launch_pass(int pass, bool area, int n, cudaStream_t st, const int32_t* X, i
     if (!area)
         if (int rc = af_ensure_smem(pass == 0 ? (const void*)k_grid_lanczos<0> : (const void*)k_grid_lanczos<1>, kLSmem))
             return rc;
-    const unsigned blocks = (unsigned)n * each;
-    if (pixel) {
-        if (pass == 0) k_grid_pixel<0><<<blocks, kGT, 0, st>>>(X, h, nout, ns, s0, M, runs, work, out);
-        else k_grid_pixel<1><<<blocks, kGT, 0, st>>>(X, h, nout, ns, s0, M, runs, work, out);
-    } else if (area) {
-        const size_t smem = (size_t)cols * 4;
-        if (pass == 0) k_grid_area<0><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s0, M, runs, cols, work, out);
-        else k_grid_area<1><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s0, M, runs, cols, work, out);
-    } else {
-        if (pass == 0) k_grid_lanczos<0><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s0, M, ti, iruns, jruns, work, out);
-        else k_grid_lanczos<1><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s0, M, ti, iruns, jruns, work, out);
+    for (int at = 0, per = (int)(0x7fffffffu / each); at < n; at += per) {
+        const unsigned blocks = (unsigned)std::min(per, n - at) * each;
+        const int s = s0 + at;
+        if (pixel) {
+            if (pass == 0) k_grid_pixel<0><<<blocks, kGT, 0, st>>>(X, h, nout, ns, s, M, runs, work, out);
+            else k_grid_pixel<1><<<blocks, kGT, 0, st>>>(X, h, nout, ns, s, M, runs, work, out);
+        } else if (area) {
+            const size_t smem = (size_t)cols * 4;
+            if (pass == 0) k_grid_area<0><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s, M, runs, cols, work, out);
+            else k_grid_area<1><<<blocks, kGT, smem, st>>>(X, h, nout, ns, s, M, runs, cols, work, out);
+        } else {
+            if (pass == 0) k_grid_lanczos<0><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s, M, ti, iruns, jruns, work, out);
+            else k_grid_lanczos<1><<<blocks, kGT, kLSmem, st>>>(X, h, nout, ns, s, M, ti, iruns, jruns, work, out);
+        }
+        if (int rc = af_cuda_check(cudaGetLastError(), "af_grid launch")) return rc;
     }
-    return af_cuda_check(cudaGetLastError(), "af_grid launch");
+    return AF_OK;
 }
 
 }  // namespace
