@@ -381,8 +381,21 @@ int launch_boxcar_nch(const int32_t* d_plane, int ndm, int64_t nout, const af_wi
 int launch_boxcar_tiles(const int32_t* d_plane, int ndm, int64_t nout, const af_widths_t& w,
                         const af_rowconst_t* d_rowconst, float* d_best_snr, uint8_t* d_best_w, cudaStream_t s)
 {
-    // 6144 prefix words per tile for widths up to 1024 samples, 12288 up to 8192
-    const bool near = w.w[w.n - 1] <= 1024;
+    // 6144 prefix words per tile for widths up to 1024 samples, 12288 up to 8192; 2048 for widths up to 512 of planes whose
+    // larger tiles are no more than the four blocks that each SM holds (a block then works through six steps while
+    // others are idle).  32 widths up to 32, us by 6144 / 2048: 64 x 5000 28.8 / 20.7, 1 x 10^6 32.9 / 24.8, 200 x 12,000 (600 tiles)
+    // 51.3 / 41.1, 500 x 28,000 (2500) 172.8 / 168.0; 5 widths up to 256: 300 x 6000 21.2 / 16.7, 100 x 40,000 (700) 21.2 / 23.0,
+    // 500 x 28,000 49.2 / 57.4.
+    int dev = 0, nsm = 0;
+    AF_CUDA(cudaGetDevice(&dev));
+    AF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int wmax = w.w[w.n - 1];
+    const bool near = wmax <= 1024;
+    const int64_t outs = kBW * 6 * 128 - wmax;  // outputs of a 6144-word tile
+    const bool few = wmax <= 512 && (nout + outs - 1) / outs * ndm <= 4 * (int64_t)nsm;
+    if (few)
+        return w.small ? launch_boxcar_nch<true, 2>(d_plane, ndm, nout, w, d_rowconst, d_best_snr, d_best_w, s)
+                       : launch_boxcar_nch<false, 2>(d_plane, ndm, nout, w, d_rowconst, d_best_snr, d_best_w, s);
     if (w.small)
         return near ? launch_boxcar_nch<true, 6>(d_plane, ndm, nout, w, d_rowconst, d_best_snr, d_best_w, s)
                     : launch_boxcar_nch<true, 12>(d_plane, ndm, nout, w, d_rowconst, d_best_snr, d_best_w, s);
