@@ -334,7 +334,14 @@ extern "C" int af_model_forward(af_model_t m, const uint16_t* d_x, int32_t n, fl
 try {
     if (int rc = check_batch(m, d_x, n)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    return forward(m, (const __nv_bfloat16*)d_x, n, nullptr, d_logits, d_prob, s);
+    // The kernels write the caller's logits, unless those are not whole floats or lie over images that blocks still read: then
+    // they are copied from the model's at the end.
+    const uintptr_t lo = (uintptr_t)d_logits, x = (uintptr_t)d_x;
+    const size_t bytes = (size_t)n * 2 * sizeof(float);
+    const bool direct = lo % sizeof(float) == 0 && (lo + bytes <= x || x + (size_t)n * 64 * 64 * 2 * 2 <= lo);
+    if (int rc = forward(m, (const __nv_bfloat16*)d_x, n, nullptr, direct ? d_logits : nullptr, d_prob, s)) return rc;
+    if (d_logits && !direct) AF_CUDA(cudaMemcpyAsync(d_logits, m->d_logits, bytes, cudaMemcpyDeviceToDevice, s));
+    return AF_OK;
 } catch (...) {
     return af_host_exception("af_model_forward");
 }
