@@ -1011,14 +1011,15 @@ int af_pairs_build(af_plan_t p)
     int only = 0;
     if (const char* e = getenv("AFGB_PAIR_DPW")) only = atoi(e);
     std::vector<std::future<void>> jobs;
-    const bool threads = (int64_t)p->ndm * p->nchan > 20000;  // a thread takes longer to start than a smaller set
+    const bool threads = (int64_t)p->ndm * p->nchan > 2000;  // a thread takes longer to start than a smaller set
     int k = 0;
     for (int G = 2; G <= (p->nchan >= 8 ? 4 : 2); G++)
         for (int dpw = 1; dpw <= 2; dpw++) {
             if (only == 3 - dpw) continue;
             af_pair_tables* T = k == 0 ? &p->pairs : &p->alt[k - 1];
             k++;
-            jobs.push_back(std::async(threads ? std::launch::async : std::launch::deferred,
+            // (both bits: built here, later, if no thread can be had)
+            jobs.push_back(std::async(threads ? std::launch::async | std::launch::deferred : std::launch::deferred,
                                       [=, &order] { build_groups(p, G, dpw, NS, optin, order, T); }));
             T->budget = budget;
         }
