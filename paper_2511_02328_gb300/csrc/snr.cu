@@ -688,20 +688,22 @@ __global__ void __launch_bounds__(kRT, 2) k_row_robust(const int32_t* __restrict
 // pass: both are checked against the windows' edges, and a row whose answer
 // lies outside them (none seen on noise) takes the general selection.  Where
 // the windows meet (M of a few units) one dense window covers them all.  A row
-// whose windows would not fit the bins (M above some 5600), or whose sample has
-// too few values near its median to trust that estimate (two far-apart modes),
-// goes to the general selection without that pass.
+// whose windows would not fit the bins (M above some 11,000; noise that fills the
+// bytes of 40,000 channels stays below), or whose sample has too few values near its
+// median to trust that estimate (two far-apart modes), goes to the general selection
+// without that pass.
 // A cluster of blocks shares a row, each counting one part; the first block
 // adds up the others' counts through distributed shared memory.  The general
 // selection is shared as well where the sample asks for it (left to the first block,
-// 500 x 200001 rows that need it took 885 us, 590 so).  Bound by issue
+// 500 x 200001 rows that need it took 880 us, 540 so; called there and not after the
+// pass, whose rows it would slow down by 2 to 6 %).  Bound by issue
 // (about 25 instructions per 32 values, the three window tests and counts) and
 // HBM: 1001 x 215261 plane 0.53 ms in three passes, 0.24 ms in one.
 // Rows below 16384 values keep the general selection: the sample would be a
 // quarter of the row and more.
 constexpr int kRS = 4096;                 // sample values
 constexpr int64_t kRobustOnePass = 16384; // shortest row for the one-pass kernel
-constexpr int kRH = 6144;                 // histogram bins of all windows
+constexpr int kRH = 12288;                // histogram bins of all windows (48 KB: M up to 11,000)
 
 struct RobustOnePass {
     union {
@@ -772,6 +774,16 @@ __device__ __forceinline__ uint32_t sample_median(const uint32_t (&key)[kRS / kR
     }
     *res = s == 0 ? 0u : (1u << s);
     return start;
+}
+
+// The general selection of a cluster's row by all of its blocks.
+__device__ __noinline__ void row_robust_shared(const int32_t* __restrict__ Y, int64_t nout, af_robust_t* __restrict__ out)
+{
+    extern __shared__ __align__(16) uint8_t robust_smem[];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
+    const int64_t d = blockIdx.x / parts;
+    row_robust_general<true>(Y + d * nout, nout, part, parts, reinterpret_cast<RobustOnePass*>(robust_smem)->gen, out + d);
 }
 
 __global__ void __launch_bounds__(kRT, 2)
@@ -854,6 +866,11 @@ k_row_robust1(const int32_t* __restrict__ Y, int64_t nout, af_robust_t* __restri
         __syncthreads();
         const uint32_t n = __reduce_add_sync(0xffffffffu, sc.one.near[lane & 15]) >> 1;  // every warp's count twice
         fits = min(n & 0xFFFFu, n >> 16) >= 16;
+    }
+    if (!fits && parts > 1) {  // the same in every block of the cluster
+        __syncthreads();       // the scratch is the general selection's now
+        row_robust_shared(Y, nout, out);
+        return;
     }
     // window starts (as v - m), widths and first bins: below m - M, around m, above m + M; dense: the first alone
     const int32_t w0 = -outer, w1 = -dc, w2 = in;
@@ -997,8 +1014,7 @@ k_row_robust1(const int32_t* __restrict__ Y, int64_t nout, af_robust_t* __restri
         __syncthreads();
     }
     cluster.sync();  // the first block has read the others' shared memory
-    if (!fits && parts > 1) row_robust_general<true>(y, nout, part, parts, sc.gen, out + d);
-    else if (part == 0 && !done) row_robust_general<false>(y, nout, 0, 1, sc.gen, out + d);
+    if (part == 0 && !done) row_robust_general<false>(y, nout, 0, 1, sc.gen, out + d);
 }
 
 // Robust S/N constants: snr = (B - w*med) * k, k = 1/(1.482602218505602 * mad * sqrt(w)).
