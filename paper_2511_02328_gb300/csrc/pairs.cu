@@ -1485,21 +1485,21 @@ int af_launch_pairs(af_plan_t p, const uint8_t* d_in, int64_t nsamp, int64_t nou
             return rc;
     const int slot = T->tcalls > 0 ? T->tnext : -1;
     int b = 0;
-    int64_t rowbytes = 0;
+    int64_t cut = 0;  // samples by which the last block's rows are shorter
     for (int64_t T0 = 0; T0 < nout; T0 += L, b++) {
         const bool rec = slot >= 0 && b < T->tblocks;
         cudaEvent_t* e = rec ? &T->tev[((size_t)slot * T->tblocks + b) * 3] : nullptr;
         if (rec) AF_CUDA(cudaEventRecord(e[0], s));
         // the last block, or a call shorter than the reservation, needs only its own tiles' rows
         const int64_t Lb = std::min(L, (nout - T0 + kPTTE - 1) / kPTTE * kPTTE);
-        rowbytes += 2 * rows_elems(T, L) - 2 * (int64_t)T->nrows * ((L - Lb) & ~(int64_t)15);
+        cut = (L - Lb) & ~(int64_t)15;
         if (int rc = af_launch_pairs_block(p, d_in, nsamp, nout, d_plane, d_stats, s, 0, T0, rec ? e + 1 : nullptr, Lb))
             return rc;
         if (rec) AF_CUDA(cudaEventRecord(e[2], s));
     }
     if (slot >= 0) {
         T->tnb[slot] = std::min(b, T->tblocks);
-        T->trowbytes[slot] = rowbytes;
+        T->trowbytes[slot] = 2 * (rows_elems(T, L) * (int64_t)b - cut * T->nrows);
         T->tcopybytes[slot] = (int64_t)((double)((nout + kPTTE - 1) / kPTTE) * T->copy_per_tile);
         T->tnext = (slot + 1) % T->tcalls;
     }
